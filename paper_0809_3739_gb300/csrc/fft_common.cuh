@@ -18,15 +18,29 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace itp {
 
+#define ITP_HD __host__ __device__ __forceinline__
+
+// Pairs of reals in HBM.
 template <typename R> struct CplxOf;
 template <> struct CplxOf<float> { using type = float2; };
 template <> struct CplxOf<double> { using type = double2; };
 
-template <typename C> __device__ __forceinline__ C cadd(C a, C b) { C r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }
-template <typename C> __device__ __forceinline__ C csub(C a, C b) { C r; r.x = a.x - b.x; r.y = a.y - b.y; return r; }
-template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
+// Complex value of the FP64 passes: 64-bit fixed point (fft_fixed.cuh).
+struct __align__(16) cfx { long long x, y; };
+// Element type of half spectra, shared-memory tiles and FFT registers.
+template <typename R> struct SpecOf;
+template <> struct SpecOf<float> { using type = float2; };
+template <> struct SpecOf<double> { using type = cfx; };
+// a * exp(2 pi i DIR M / R) in fixed point
+template <int DIR, int M, int R> ITP_HD cfx fx_twc(cfx a);
+
+template <typename C> ITP_HD C cadd(C a, C b) { C r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }
+template <typename C> ITP_HD C csub(C a, C b) { C r; r.x = a.x - b.x; r.y = a.y - b.y; return r; }
+template <typename C> ITP_HD C cmul(C a, C b) {
   C r; r.x = a.x * b.x - a.y * b.y; r.y = a.x * b.y + a.y * b.x; return r;
 }
 // a * conj(b)
@@ -36,16 +50,28 @@ template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
 // FP32 complex values use the packed two-lane FP32 instructions of sm_100+
 // (one instruction updates re and im): add, multiply and fused multiply-add
 // on float2.  Each lane rounds as the scalar instruction does.
-template <> __device__ __forceinline__ float2 cadd<float2>(float2 a, float2 b) {
+template <> ITP_HD float2 cadd<float2>(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
   return __fadd2_rn(a, b);
+#else
+  return make_float2(a.x + b.x, a.y + b.y);
+#endif
 }
-template <> __device__ __forceinline__ float2 csub<float2>(float2 a, float2 b) {
+template <> ITP_HD float2 csub<float2>(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
   return __fadd2_rn(a, make_float2(-b.x, -b.y));
+#else
+  return make_float2(a.x - b.x, a.y - b.y);
+#endif
 }
-template <> __device__ __forceinline__ float2 cmul<float2>(float2 a, float2 b) {
+template <> ITP_HD float2 cmul<float2>(float2 a, float2 b) {
   // (a.x b.x, a.x b.y) + (a.y (-b.y), a.y b.x)
+#ifdef __CUDA_ARCH__
   return __ffma2_rn(make_float2(a.y, a.y), make_float2(-b.y, b.x),
                     __fmul2_rn(make_float2(a.x, a.x), b));
+#else
+  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+#endif
 }
 template <> __device__ __forceinline__ float2 cmulc<float2>(float2 a, float2 b) {
   // (a.x b.x, -a.x b.y) + (a.y b.y, a.y b.x)
@@ -53,7 +79,7 @@ template <> __device__ __forceinline__ float2 cmulc<float2>(float2 a, float2 b) 
                     __fmul2_rn(make_float2(a.x, a.x), make_float2(b.x, -b.y)));
 }
 // multiply by i*s, s = +-1
-template <int S, typename C> __device__ __forceinline__ C cmul_i(C a) {
+template <int S, typename C> ITP_HD C cmul_i(C a) {
   C r; if (S > 0) { r.x = -a.y; r.y = a.x; } else { r.x = a.y; r.y = -a.x; } return r;
 }
 
@@ -77,12 +103,14 @@ __host__ __device__ constexpr double sin48(int t) { return cos48(12 - t); }
 
 // a * exp(DIR * 2*pi*i * m / R) with compile-time m, R (48 % R == 0).
 template <int DIR, int M, int R, typename C>
-__device__ __forceinline__ C twc(C a) {
+ITP_HD C twc(C a) {
   constexpr int t = ((M % R) * (48 / R)) % 48;
   constexpr double c = cos48(t);
   constexpr double s = DIR * sin48(t);
   if constexpr (t == 0) {
     return a;
+  } else if constexpr (std::is_same<C, cfx>::value) {
+    return fx_twc<DIR, M, R>(a);
   } else if constexpr (t == 12 || t == 36) {
     return (s > 0) ? cmul_i<1>(a) : cmul_i<-1>(a);
   } else if constexpr (t == 24) {
@@ -100,15 +128,15 @@ __device__ __forceinline__ C twc(C a) {
 template <int R, int DIR, typename C> struct Dft;
 
 template <int DIR, typename C> struct Dft<1, DIR, C> {
-  static __device__ __forceinline__ void run(C*) {}
+  static ITP_HD void run(C*) {}
 };
 template <int DIR, typename C> struct Dft<2, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) {
+  static ITP_HD void run(C* a) {
     C t = a[0]; a[0] = cadd(t, a[1]); a[1] = csub(t, a[1]);
   }
 };
 template <int DIR, typename C> struct Dft<3, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) {
+  static ITP_HD void run(C* a) {
     using Rl = decltype(a[0].x);
     const Rl h = (Rl)0.86602540378443864676;  // sin(2pi/3)
     C s = cadd(a[1], a[2]);
@@ -122,7 +150,7 @@ template <int DIR, typename C> struct Dft<3, DIR, C> {
   }
 };
 template <int DIR, typename C> struct Dft<4, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) {
+  static ITP_HD void run(C* a) {
     C s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
     C s13 = cadd(a[1], a[3]), d13 = csub(a[1], a[3]);
     C r = cmul_i<DIR>(d13);   // DIR*i*(a1 - a3)
@@ -134,7 +162,7 @@ template <int DIR, typename C> struct Dft<4, DIR, C> {
 };
 
 template <int P, int Q, int DIR, int N1, int K2, typename C>
-__device__ __forceinline__ void tw_apply(C* b) {
+ITP_HD void tw_apply(C* b) {
   if constexpr (N1 < P) {
     if constexpr (K2 < Q) {
       b[N1 * Q + K2] = twc<DIR, N1 * K2, P * Q>(b[N1 * Q + K2]);
@@ -147,7 +175,7 @@ __device__ __forceinline__ void tw_apply(C* b) {
 
 // Composite R = P*Q in registers: n = n1 + P*n2, k = k2 + Q*k1.
 template <int P, int Q, int DIR, typename C>
-__device__ __forceinline__ void dft_pq(C* a) {
+ITP_HD void dft_pq(C* a) {
   C b[P * Q];
 #pragma unroll
   for (int n1 = 0; n1 < P; ++n1) {
@@ -171,16 +199,16 @@ __device__ __forceinline__ void dft_pq(C* a) {
   }
 }
 template <int DIR, typename C> struct Dft<6, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) { dft_pq<2, 3, DIR, C>(a); }
+  static ITP_HD void run(C* a) { dft_pq<2, 3, DIR, C>(a); }
 };
 template <int DIR, typename C> struct Dft<8, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) { dft_pq<2, 4, DIR, C>(a); }
+  static ITP_HD void run(C* a) { dft_pq<2, 4, DIR, C>(a); }
 };
 template <int DIR, typename C> struct Dft<12, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) { dft_pq<4, 3, DIR, C>(a); }
+  static ITP_HD void run(C* a) { dft_pq<4, 3, DIR, C>(a); }
 };
 template <int DIR, typename C> struct Dft<16, DIR, C> {
-  static __device__ __forceinline__ void run(C* a) { dft_pq<4, 4, DIR, C>(a); }
+  static ITP_HD void run(C* a) { dft_pq<4, 4, DIR, C>(a); }
 };
 
 // ---------------------------------------------------------------------------
@@ -188,103 +216,6 @@ template <int DIR, typename C> struct Dft<16, DIR, C> {
 struct Axis {
   int L, r1, r2;
 };
-
-// Shared-memory stages.  `addr(t, e)` gives the position of element e of
-// transform t.  Tasks are numbered with the transform index fastest so that
-// neighbouring lanes touch neighbouring transforms (conflict-free when the
-// transforms are adjacent columns or rows with an odd pitch).
-//
-// tw: the L roots exp(-2*pi*i*m/L), m = 0..L-1.
-template <int R2, int DIR, typename C, typename Addr>
-__device__ __forceinline__ void stage_a_r(C* sm, const Addr& addr, int ntr, const Axis ax,
-                                          const C* __restrict__ tw, int tid, int nthr) {
-  const int tasks = ntr * ax.r1;
-  for (int task = tid; task < tasks; task += nthr) {
-    const int t = task % ntr, n1 = task / ntr;
-    C a[R2];
-#pragma unroll
-    for (int j = 0; j < R2; ++j) a[j] = sm[addr(t, n1 + ax.r1 * j)];
-    Dft<R2, DIR, C>::run(a);
-    if (DIR < 0 && ax.r1 > 1) {
-#pragma unroll
-      for (int j = 1; j < R2; ++j) a[j] = cmul(a[j], __ldg(&tw[n1 * j]));
-    }
-#pragma unroll
-    for (int j = 0; j < R2; ++j) sm[addr(t, n1 + ax.r1 * j)] = a[j];
-  }
-}
-
-template <int R1, int DIR, typename C, typename Addr>
-__device__ __forceinline__ void stage_b_r(C* sm, const Addr& addr, int ntr, const Axis ax,
-                                          const C* __restrict__ tw, int tid, int nthr) {
-  const int tasks = ntr * ax.r2;
-  for (int task = tid; task < tasks; task += nthr) {
-    const int t = task % ntr, b = task / ntr;
-    C a[R1];
-#pragma unroll
-    for (int i = 0; i < R1; ++i) a[i] = sm[addr(t, i + R1 * b)];
-    Dft<R1, DIR, C>::run(a);
-    if (DIR > 0) {
-#pragma unroll
-      for (int i = 1; i < R1; ++i) a[i] = cmulc(a[i], __ldg(&tw[i * b]));
-    }
-#pragma unroll
-    for (int i = 0; i < R1; ++i) sm[addr(t, i + R1 * b)] = a[i];
-  }
-}
-
-#define ITP_RADIX_SWITCH(r, CALL)                  \
-  switch (r) {                                     \
-    case 2: CALL(2); break;                        \
-    case 3: CALL(3); break;                        \
-    case 4: CALL(4); break;                        \
-    case 6: CALL(6); break;                        \
-    case 8: CALL(8); break;                        \
-    case 12: CALL(12); break;                      \
-    case 16: CALL(16); break;                      \
-    default: break;                                \
-  }
-
-// Stage A (forward: DIR=-1, twiddle after; inverse A': DIR=+1, no twiddle).
-template <int DIR, typename C, typename Addr>
-__device__ __forceinline__ void stage_a(C* sm, const Addr& addr, int ntr, const Axis ax,
-                                        const C* __restrict__ tw, int tid, int nthr) {
-#define ITP_CALL_A(R) stage_a_r<R, DIR>(sm, addr, ntr, ax, tw, tid, nthr)
-  ITP_RADIX_SWITCH(ax.r2, ITP_CALL_A)
-#undef ITP_CALL_A
-}
-// Stage B (forward: DIR=-1, no twiddle; inverse B': DIR=+1, twiddle after).
-template <int DIR, typename C, typename Addr>
-__device__ __forceinline__ void stage_b(C* sm, const Addr& addr, int ntr, const Axis ax,
-                                        const C* __restrict__ tw, int tid, int nthr) {
-  if (ax.r1 == 1) return;
-#define ITP_CALL_B(R) stage_b_r<R, DIR>(sm, addr, ntr, ax, tw, tid, nthr)
-  ITP_RADIX_SWITCH(ax.r1, ITP_CALL_B)
-#undef ITP_CALL_B
-}
-
-// Forward transform (natural -> digit-swapped), barriers included.
-template <typename C, typename Addr>
-__device__ __forceinline__ void fft_forward(C* sm, const Addr& addr, int ntr, const Axis ax,
-                                            const C* __restrict__ tw) {
-  stage_a<-1>(sm, addr, ntr, ax, tw, threadIdx.x, blockDim.x);
-  __syncthreads();
-  if (ax.r1 > 1) {
-    stage_b<-1>(sm, addr, ntr, ax, tw, threadIdx.x, blockDim.x);
-    __syncthreads();
-  }
-}
-// Inverse transform (digit-swapped -> natural), barriers included.
-template <typename C, typename Addr>
-__device__ __forceinline__ void fft_inverse(C* sm, const Addr& addr, int ntr, const Axis ax,
-                                            const C* __restrict__ tw) {
-  if (ax.r1 > 1) {
-    stage_b<1>(sm, addr, ntr, ax, tw, threadIdx.x, blockDim.x);
-    __syncthreads();
-  }
-  stage_a<1>(sm, addr, ntr, ax, tw, threadIdx.x, blockDim.x);
-  __syncthreads();
-}
 
 // Position in shared memory of frequency k after a forward transform.
 __device__ __forceinline__ int spec_pos(const Axis& ax, int k) {

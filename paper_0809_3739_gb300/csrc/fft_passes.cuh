@@ -32,11 +32,17 @@
 #include <cooperative_groups.h>
 
 #include "fft_common.cuh"
+#include "fft_fixed.cuh"
 #include "itp_kernels.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace itp {
+
+template <int NX, int NY>
+cudaError_t plane64_dispatch(const GridDesc& g, int mode, const PlaneArgs<double>& a,
+                             const PlaneArgs<double>* args, const int2* rows, int nrows,
+                             size_t smem, cudaStream_t st);
 
 namespace {
 
@@ -101,6 +107,24 @@ __host__ __device__ constexpr long long pencil_smem_ct(int nz, int w, int rbytes
   return nz ? ((long long)nz * w + nz) * 2 * rbytes : 0;
 }
 
+// a.v[i] *= f(i), a real factor.
+template <int N, typename R, typename C, typename F>
+__device__ __forceinline__ void scale_by(SVec<C, N>& a, F&& f) {
+  if constexpr (SVec<C, N>::fixed) {
+    R fv[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) fv[i] = f(i);
+    a.mul_real(fv);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const R s = f(i);
+      a.v[i].x *= s;
+      a.v[i].y *= s;
+    }
+  }
+}
+
 // Padded position of element p of a packed row: one pad slot per 16 keeps
 // the strided reads of the split/merge free of bank conflicts.
 __device__ __forceinline__ int swz(int p) { return p + (p >> 4); }
@@ -118,26 +142,32 @@ __device__ __forceinline__ void for_tasks(int ntr, int nq, F&& f) {
 }
 
 // Radix dispatch: FN<r>(args...) for the run-time radix r (folds to one case
-// when r is a compile-time constant).
-#define ITP_WITH_RADIX(r, FN, ...)          \
-  switch (r) {                              \
-    case 1: FN<1>(__VA_ARGS__); break;      \
-    case 2: FN<2>(__VA_ARGS__); break;      \
-    case 3: FN<3>(__VA_ARGS__); break;      \
-    case 4: FN<4>(__VA_ARGS__); break;      \
-    case 6: FN<6>(__VA_ARGS__); break;      \
-    case 8: FN<8>(__VA_ARGS__); break;      \
-    case 12: FN<12>(__VA_ARGS__); break;    \
-    case 16: FN<16>(__VA_ARGS__); break;    \
-    default: break;                         \
+// when r is a compile-time constant).  outline: each case in a function of
+// its own.  The generic FP64 kernels hold all radices of every stage; inlined
+// they took minutes to compile, as functions they are shared by the modes.
+template <typename L>
+__device__ __noinline__ void call_out_of_line(L f) { f(); }
+#define ITP_RADIX_CASE(r, outline, FN, ...)                                   \
+  case r:                                                                     \
+    if constexpr (outline) call_out_of_line([=] { FN<r>(__VA_ARGS__); });      \
+    else FN<r>(__VA_ARGS__);                                                  \
+    break;
+#define ITP_WITH_RADIX(r, outline, FN, ...)     \
+  switch (r) {                                  \
+    ITP_RADIX_CASE(1, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(2, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(3, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(4, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(6, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(8, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(12, outline, FN, __VA_ARGS__) \
+    ITP_RADIX_CASE(16, outline, FN, __VA_ARGS__) \
+    default: break;                             \
   }
+// Whether the stages of an axis (N = 0: run-time length) are outlined.
+template <typename C, int N>
+constexpr bool outlined = std::is_same<C, cfx>::value && N == 0;
 
-template <typename C>
-__device__ __forceinline__ C cscale(C a, decltype(a.x) s) {
-  a.x *= s;
-  a.y *= s;
-  return a;
-}
 template <typename C>
 __device__ __forceinline__ C cmulri(C a, C f) {  // (a.x * f.x, a.y * f.y)
   a.x *= f.x;
@@ -149,14 +179,28 @@ __device__ __forceinline__ float2 cmulri<float2>(float2 a, float2 f) {
   return __fmul2_rn(a, f);
 }
 
-// a[j] *= w^(q j) (CONJ: w^(-q j)), j = 1..R-1, from the table tw of
-// roots.  For R = 8 and 16 the factor is w^(q j1) w^(4 q j2) with
+// a[j] *= w^(q j) (CONJ: w^(-q j)), j = 1..R-1, one table read each.
+template <bool CONJ = false, typename C, int R>
+__device__ __forceinline__ void twiddle_direct(SVec<C, R>& a, const C* tw, int q) {
+  if constexpr (SVec<C, R>::fixed) {
+    fx_twiddle<CONJ>(a, reinterpret_cast<const fx_tw*>(tw), q);
+  } else {
+#pragma unroll
+    for (int j = 1; j < R; ++j)
+      a.v[j] = CONJ ? cmulc(a.v[j], tw[q * j]) : cmul(a.v[j], tw[q * j]);
+  }
+}
+
+// The same from the table tw of roots, in FP32 with fewer table reads.  For R = 8 and 16 the factor is w^(q j1) w^(4 q j2) with
 // j = j1 + 4 j2: four or six table reads instead of seven or fifteen (the
 // reads are shared-memory wavefronts, the passes' bound), each product
 // within about an ulp of the table value.
 template <int R, bool CONJ = false, typename C>
-__device__ __forceinline__ void twiddle_stage(C (&a)[R], const C* tw, int q) {
-  if constexpr (R == 8 || R == 16) {
+__device__ __forceinline__ void twiddle_stage(SVec<C, R>& av, const C* tw, int q) {
+  if constexpr (SVec<C, R>::fixed) {
+    twiddle_direct<CONJ>(av, tw, q);
+  } else if constexpr (R == 8 || R == 16) {
+    C(&a)[R] = av.v;
     constexpr int NH = R / 4;   // hi factors w^(4 q j2), j2 = 1 .. NH-1
     C lo[4], hi[NH];
 #pragma unroll
@@ -170,8 +214,7 @@ __device__ __forceinline__ void twiddle_stage(C (&a)[R], const C* tw, int q) {
       a[j] = CONJ ? cmulc(a[j], w) : cmul(a[j], w);
     }
   } else {
-#pragma unroll
-    for (int j = 1; j < R; ++j) a[j] = CONJ ? cmulc(a[j], tw[q * j]) : cmul(a[j], tw[q * j]);
+    twiddle_direct<CONJ>(av, tw, q);
   }
 }
 
@@ -179,7 +222,7 @@ __device__ __forceinline__ void twiddle_stage(C (&a)[R], const C* tw, int q) {
 // Shared-memory geometry of one plane.
 template <typename R, int NX, int NY, int NTT>
 struct PlaneGeo {
-  using C = typename CplxOf<R>::type;
+  using C = typename SpecOf<R>::type;
   static constexpr int NT = NTT;
   AxisT<NX> ax;
   AxisT<NY> ay;
@@ -238,33 +281,44 @@ struct PlaneGeo {
 // Forward stage A with the global load fused in: element x of row pair t is
 // the pair (psi[y=2t][x], psi[y=2t+1][x]) = src[x * npair + t] (transposed
 // layout), times the factor pair f[x * npair + t].
-template <int R2, typename R, int NX, int NY, int NTT, typename C>
+template <int R2, typename R, int NX, int NY, int NTT, typename C, typename CR>
 __device__ __forceinline__ void xA_fwd_global_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm,
-                                                const C* __restrict__ src,
-                                                const C* __restrict__ f, const C* tw) {
+                                                const CR* __restrict__ src,
+                                                const CR* __restrict__ f, const C* tw) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.npair, G.ax.r1, [&](int t, int n1) {
-    C a[R2];
+    SVec<C, R2> a;
+    if constexpr (SVec<C, R2>::fixed) {
+      CR p[R2], q[R2];
 #pragma unroll
-    for (int j = 0; j < R2; ++j) {
-      const int x = n1 + G.ax.r1 * j;
-      a[j] = src[x * G.gpair + t];
-      if (f) a[j] = cmulri(a[j], __ldg(&f[x * G.gpair + t]));
+      for (int j = 0; j < R2; ++j) p[j] = src[(n1 + G.ax.r1 * j) * G.gpair + t];
+      if (f) {
+#pragma unroll
+        for (int j = 0; j < R2; ++j) q[j] = __ldg(&f[(n1 + G.ax.r1 * j) * G.gpair + t]);
+        a.template from_pairs<true>(p, q);
+      } else {
+        a.template from_pairs<false>(p, p);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < R2; ++j) {
+        const int x = n1 + G.ax.r1 * j;
+        a.v[j] = src[x * G.gpair + t];
+        if (f) a.v[j] = cmulri(a.v[j], __ldg(&f[x * G.gpair + t]));
+      }
     }
-    Dft<R2, -1, C>::run(a);
-    if (G.ax.r1 > 1) {   // (the two-table twiddles measured slower here)
+    a.template dft<-1>();
+    if (G.ax.r1 > 1) twiddle_direct(a, tw, n1);   // (the two-table twiddles measured slower here)
+    a.close();
 #pragma unroll
-      for (int j = 1; j < R2; ++j) a[j] = cmul(a[j], tw[n1 * j]);
-    }
-#pragma unroll
-    for (int j = 0; j < R2; ++j) sm[G.rowA(t, n1, j)] = a[j];
+    for (int j = 0; j < R2; ++j) sm[G.rowA(t, n1, j)] = a.v[j];
   });
 }
-template <typename R, int NX, int NY, int NTT, typename C>
+template <typename R, int NX, int NY, int NTT, typename C, typename CR>
 __device__ __forceinline__ void xA_fwd_global(const PlaneGeo<R, NX, NY, NTT>& G, C* sm,
-                                              const C* __restrict__ src,
-                                              const C* __restrict__ f, const C* tw) {
-  ITP_WITH_RADIX(G.ax.r2, xA_fwd_global_r, G, sm, src, f, tw)
+                                              const CR* __restrict__ src,
+                                              const CR* __restrict__ f, const C* tw) {
+  ITP_WITH_RADIX(G.ax.r2, (outlined<C, NX>), xA_fwd_global_r, G, sm, src, f, tw)
 }
 
 // Stage B (DIR = -1 forward, +1 inverse with the conjugate twiddle after).
@@ -272,16 +326,15 @@ template <int R1, int DIR, typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void xB_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.npair, G.ax.r2, [&](int t, int b) {
-    C a[R1];
+    SVec<C, R1> a;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) a[i] = sm[G.rowB(t, b, i)];
-    Dft<R1, DIR, C>::run(a);
-    if (DIR > 0) {
+    for (int i = 0; i < R1; ++i) a.v[i] = sm[G.rowB(t, b, i)];
+    a.open();
+    a.template dft<DIR>();
+    if (DIR > 0) twiddle_direct<true>(a, tw, b);
+    a.close();
 #pragma unroll
-      for (int i = 1; i < R1; ++i) a[i] = cmulc(a[i], tw[i * b]);
-    }
-#pragma unroll
-    for (int i = 0; i < R1; ++i) sm[G.rowB(t, b, i)] = a[i];
+    for (int i = 0; i < R1; ++i) sm[G.rowB(t, b, i)] = a.v[i];
   });
 }
 template <int R1, typename G_, typename C>
@@ -292,14 +345,14 @@ template <int DIR, typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void xB(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
   if (G.ax.r1 == 1) return;
   if (DIR < 0) {
-    ITP_WITH_RADIX(G.ax.r1, xB_fwd_r, G, sm, tw)
+    ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_fwd_r, G, sm, tw)
   } else {
-    ITP_WITH_RADIX(G.ax.r1, xB_inv_r, G, sm, tw)
+    ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_inv_r, G, sm, tw)
   }
 }
 
 // Inverse stage A' followed by an epilogue on the natural-order row data:
-// epi.apply<R2>(t, n1, a) receives a[j] = element x = n1 + r1*j of row pair
+// epi.apply<R2>(t, n1, a) receives a.v[j] = element x = n1 + r1*j of row pair
 // t and either stores it somewhere (returns false) or transforms it and asks
 // for the forward stage A to follow in registers (returns true).
 template <int R2, typename R, int NX, int NY, int NTT, typename C, typename Epi>
@@ -307,30 +360,50 @@ __device__ __forceinline__ void xA_inv_then_r(const PlaneGeo<R, NX, NY, NTT>& G,
                                               const Epi& epi) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.npair, G.ax.r1, [&](int t, int n1) {
-    C a[R2];
+    SVec<C, R2> a;
 #pragma unroll
-    for (int j = 0; j < R2; ++j) a[j] = sm[G.rowA(t, n1, j)];
-    Dft<R2, 1, C>::run(a);
+    for (int j = 0; j < R2; ++j) a.v[j] = sm[G.rowA(t, n1, j)];
+    a.open();
+    a.template dft<1>();
     if (epi.template apply<R2>(t, n1, a)) {
-      Dft<R2, -1, C>::run(a);
+      a.template dft<-1>();
       if (G.ax.r1 > 1) twiddle_stage<R2>(a, tw, n1);
+      a.close();
 #pragma unroll
-      for (int j = 0; j < R2; ++j) sm[G.rowA(t, n1, j)] = a[j];
+      for (int j = 0; j < R2; ++j) sm[G.rowA(t, n1, j)] = a.v[j];
     }
   });
 }
 template <typename R, int NX, int NY, int NTT, typename C, typename Epi>
 __device__ __forceinline__ void xA_inv_then(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw,
                                             const Epi& epi) {
-  ITP_WITH_RADIX(G.ax.r2, xA_inv_then_r, G, sm, tw, epi)
+  ITP_WITH_RADIX(G.ax.r2, (outlined<C, NX>), xA_inv_then_r, G, sm, tw, epi)
+}
+
+// A = FFT(a), B = FFT(b) at frequency k from Z[k] = zp and Z[nx - k] = zm
+// (fixed point: the halving goes into the exponent e).
+template <typename C>
+__device__ __forceinline__ void split_pair(C zp, C zm, C& A, C& B, int& e) {
+  if constexpr (std::is_same<C, cfx>::value) {
+    A.x = zp.x + zm.x;
+    A.y = zp.y - zm.y;
+    B.x = zp.y + zm.y;
+    B.y = zm.x - zp.x;
+    if (e < kFxPoison) e -= 1;
+  } else {
+    A.x = 0.5f * (zp.x + zm.x);
+    A.y = 0.5f * (zp.y - zm.y);
+    B.x = 0.5f * (zp.y + zm.y);
+    B.y = 0.5f * (zm.x - zp.x);
+  }
 }
 
 // Real transform along x, forward: split the spectrum Z of each packed row
 // (a + i b) into A = FFT(a), B = FFT(b), k = 0..nx/2.  One warp per row
 // pair; Z is read in digit-swapped order.
 template <typename R, int NX, int NY, int NTT>
-__device__ __forceinline__ void x_split(const PlaneGeo<R, NX, NY, NTT>& G, typename CplxOf<R>::type* sm) {
-  using C = typename CplxOf<R>::type;
+__device__ __forceinline__ void x_split(const PlaneGeo<R, NX, NY, NTT>& G, typename SpecOf<R>::type* sm) {
+  using C = typename SpecOf<R>::type;
   constexpr int MAXQ = NX ? (NX / 2 + 32) / 32 : 5;
   constexpr int NW = PlaneGeo<R, NX, NY, NTT>::NT / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -353,13 +426,21 @@ __device__ __forceinline__ void x_split(const PlaneGeo<R, NX, NY, NTT>& G, typen
     for (int q = 0; q < MAXQ; ++q) {
       const int k = lane + 32 * q;
       if (k <= half) {
-        C A, B;
-        A.x = (R)0.5 * (zp[q].x + zm[q].x);
-        A.y = (R)0.5 * (zp[q].y - zm[q].y);
-        B.x = (R)0.5 * (zp[q].y + zm[q].y);
-        B.y = (R)0.5 * (zm[q].x - zp[q].x);
-        row[k] = A;
-        row[G.nxh + k] = B;
+        SVec<C, 2> ab;
+        if constexpr (SVec<C, 2>::fixed) {
+          SVec<C, 2> z;
+          z.v[0] = zp[q];
+          z.v[1] = zm[q];
+          z.template open<1>();
+          ab.e = z.e;
+          split_pair(z.v[0], z.v[1], ab.v[0], ab.v[1], ab.e);
+        } else {
+          int e;
+          split_pair(zp[q], zm[q], ab.v[0], ab.v[1], e);
+        }
+        ab.close();
+        row[k] = ab.v[0];
+        row[G.nxh + k] = ab.v[1];
       }
     }
     __syncwarp();
@@ -370,8 +451,8 @@ __device__ __forceinline__ void x_split(const PlaneGeo<R, NX, NY, NTT>& G, typen
 // self-conjugate bins k = 0, nx/2 are dropped, as a complex-to-real
 // transform does), writing Z in digit-swapped order.
 template <typename R, int NX, int NY, int NTT>
-__device__ __forceinline__ void x_merge(const PlaneGeo<R, NX, NY, NTT>& G, typename CplxOf<R>::type* sm) {
-  using C = typename CplxOf<R>::type;
+__device__ __forceinline__ void x_merge(const PlaneGeo<R, NX, NY, NTT>& G, typename SpecOf<R>::type* sm) {
+  using C = typename SpecOf<R>::type;
   constexpr int MAXQ = NX ? (NX / 2 + 32) / 32 : 5;
   constexpr int NW = PlaneGeo<R, NX, NY, NTT>::NT / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -394,18 +475,19 @@ __device__ __forceinline__ void x_merge(const PlaneGeo<R, NX, NY, NTT>& G, typen
     for (int q = 0; q < MAXQ; ++q) {
       const int k = lane + 32 * q;
       if (k <= half) {
-        C A = av[q], B = bv[q];
+        SVec<C, 2> ab;
+        ab.v[0] = av[q];
+        ab.v[1] = bv[q];
+        ab.template open<1>();
+        C A = ab.v[0], B = ab.v[1];
         if (k == 0 || k == half) { A.y = 0; B.y = 0; }
-        C Z;
-        Z.x = A.x - B.y;
-        Z.y = A.y + B.x;
-        row[swz(spec_pos(ax, k))] = Z;
-        if (k > 0 && k < half) {
-          C Zm;
-          Zm.x = A.x + B.y;
-          Zm.y = B.x - A.y;
-          row[swz(spec_pos(ax, G.nx - k))] = Zm;
-        }
+        ab.v[0].x = A.x - B.y;   // Z[k]
+        ab.v[0].y = A.y + B.x;
+        ab.v[1].x = A.x + B.y;   // Z[nx - k]
+        ab.v[1].y = B.x - A.y;
+        ab.close();
+        row[swz(spec_pos(ax, k))] = ab.v[0];
+        if (k > 0 && k < half) row[swz(spec_pos(ax, G.nx - k))] = ab.v[1];
       }
     }
     __syncwarp();
@@ -431,32 +513,56 @@ __device__ __forceinline__ void xB_fwd_split_r(const PlaneGeo<R, NX, NY, NTT>& G
     const int t = rg * rpw + grp;
     const bool active = grp < rpw && t < G.npair;
     C* row = sm + (active ? t : 0) * G.pp;
-    C a[R1];
+    SVec<C, R1> a;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) a[i] = active ? sm[G.rowB(active ? t : 0, b, i)] : C{0, 0};
-    Dft<R1, -1, C>::run(a);   // a[k1] = Z[b + r2*k1]
-    C zm[R1];
+    for (int i = 0; i < R1; ++i) a.v[i] = active ? sm[G.rowB(active ? t : 0, b, i)] : C{0, 0};
+    a.open();
+    a.template dft<-1>();   // a.v[k1] = Z[b + r2*k1]
+    int down = 0, down_src = 0;   // fixed point: shifts to the common exponent of the two lanes
+    if constexpr (SVec<C, R1>::fixed) {
+      const int es = __shfl_sync(0xffffffffu, a.e, src), em = fx_max(a.e, es);
+      down = fx_min(em - a.e, 63);
+      down_src = fx_min(em - es, 63);
+      a.e = em;
+    }
+    // only k <= nx/2 is kept: k1 <= R1/2 (the senders know which they owe)
+    constexpr int KH = R1 / 2 + 1;
+    C zm[KH];
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) {
+    for (int k1 = 0; k1 < KH; ++k1) {
       // the receiver wants Z[nx - k]; its sender (lane src) holds it at index
       // (R1 - k1) % R1 when b == 0 and R1 - 1 - k1 otherwise
-      const C mine = (b == 0) ? a[(R1 - k1) % R1] : a[R1 - 1 - k1];
+      const C mine = (b == 0) ? a.v[(R1 - k1) % R1] : a.v[R1 - 1 - k1];
       zm[k1].x = __shfl_sync(0xffffffffu, mine.x, src);
       zm[k1].y = __shfl_sync(0xffffffffu, mine.y, src);
     }
+    SVec<C, 2 * KH> ab;   // A and B of each k1
+    if constexpr (SVec<C, R1>::fixed) {
+      ab.e = a.e;
+#pragma unroll
+      for (int k1 = 0; k1 < KH; ++k1) {
+        int e = 0;
+        const C zp{a.v[k1].x >> down, a.v[k1].y >> down};
+        const C zq{zm[k1].x >> down_src, zm[k1].y >> down_src};
+        split_pair(zp, zq, ab.v[2 * k1], ab.v[2 * k1 + 1], e);
+        if (b + r2 * k1 > half) ab.v[2 * k1] = ab.v[2 * k1 + 1] = C{0, 0};
+      }
+      if (ab.e < kFxPoison) ab.e -= 1;
+    } else {
+      int e;
+#pragma unroll
+      for (int k1 = 0; k1 < KH; ++k1)
+        split_pair(a.v[k1], zm[k1], ab.v[2 * k1], ab.v[2 * k1 + 1], e);
+    }
+    ab.close();
     __syncwarp();
     if (active) {
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) {
+      for (int k1 = 0; k1 < KH; ++k1) {
         const int k = b + r2 * k1;
         if (k <= half) {
-          C A, B;
-          A.x = (R)0.5 * (a[k1].x + zm[k1].x);
-          A.y = (R)0.5 * (a[k1].y - zm[k1].y);
-          B.x = (R)0.5 * (a[k1].y + zm[k1].y);
-          B.y = (R)0.5 * (zm[k1].x - a[k1].x);
-          row[k] = A;
-          row[G.nxh + k] = B;
+          row[k] = ab.v[2 * k1];
+          row[G.nxh + k] = ab.v[2 * k1 + 1];
         }
       }
     }
@@ -480,7 +586,7 @@ __device__ __forceinline__ void xB_inv_merge_r(const PlaneGeo<R, NX, NY, NTT>& G
   // loaded once into registers, not per row group (the row loop writes the
   // same shared array, so the compiler reloads them); at R1 = 16 the 30 more
   // registers would spill
-  constexpr bool kHold = R1 <= 8;
+  constexpr bool kHold = R1 <= 8 && !SVec<C, R1>::fixed;
   C twr[kHold ? R1 : 1];
   if constexpr (kHold) {
 #pragma unroll
@@ -490,37 +596,47 @@ __device__ __forceinline__ void xB_inv_merge_r(const PlaneGeo<R, NX, NY, NTT>& G
     const int t = rg * rpw + grp;
     const bool active = grp < rpw && t < G.npair;
     C* row = sm + (active ? t : 0) * G.pp;
-    C v[R1];
+    SVec<C, 2 * R1> ab;   // A and B, at k or (k > nx/2) at nx - k
+#pragma unroll
+    for (int i = 0; i < R1; ++i) {
+      const int k = b + r2 * i, kk = k <= half ? k : G.nx - k;
+      ab.v[2 * i] = ab.v[2 * i + 1] = C{0, 0};
+      if (active) {
+        ab.v[2 * i] = row[kk];
+        ab.v[2 * i + 1] = row[G.nxh + kk];
+      }
+    }
+    ab.template open<1>();
+    SVec<C, R1> v;
 #pragma unroll
     for (int i = 0; i < R1; ++i) {
       const int k = b + r2 * i;
-      C z = C{0, 0};
-      if (active) {
-        if (k <= half) {
-          C A = row[k], B = row[G.nxh + k];
-          if (k == 0 || k == half) { A.y = 0; B.y = 0; }
-          z.x = A.x - B.y;
-          z.y = A.y + B.x;
-        } else {
-          const C A = row[G.nx - k], B = row[G.nxh + G.nx - k];
-          z.x = A.x + B.y;
-          z.y = B.x - A.y;
-        }
+      C A = ab.v[2 * i], B = ab.v[2 * i + 1], z;
+      if (k <= half) {
+        if (k == 0 || k == half) { A.y = 0; B.y = 0; }
+        z.x = A.x - B.y;
+        z.y = A.y + B.x;
+      } else {
+        z.x = A.x + B.y;
+        z.y = B.x - A.y;
       }
-      v[i] = z;
+      v.v[i] = z;
     }
+    if constexpr (SVec<C, R1>::fixed) v.e = ab.e;
     __syncwarp();
-    Dft<R1, 1, C>::run(v);
+    v.template dft<1>();
     if (R1 > 1) {
+      if constexpr (kHold) {
 #pragma unroll
-      for (int i = 1; i < R1; ++i) {
-        if constexpr (kHold) v[i] = cmulc(v[i], twr[i]);
-        else v[i] = cmulc(v[i], tw[i * b]);
+        for (int i = 1; i < R1; ++i) v.v[i] = cmulc(v.v[i], twr[i]);
+      } else {
+        twiddle_direct<true>(v, tw, b);
       }
     }
+    v.close();
     if (active) {
 #pragma unroll
-      for (int i = 0; i < R1; ++i) sm[G.rowB(t, b, i)] = v[i];
+      for (int i = 0; i < R1; ++i) sm[G.rowB(t, b, i)] = v.v[i];
     }
     __syncwarp();
   }
@@ -532,7 +648,7 @@ __device__ __forceinline__ void xB_fwd_split(const PlaneGeo<R, NX, NY, NTT>& G, 
     x_split(G, sm);
     return;
   }
-  ITP_WITH_RADIX(G.ax.r1, xB_fwd_split_r, G, sm)
+  ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_fwd_split_r, G, sm)
 }
 template <typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void xB_inv_merge(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
@@ -542,7 +658,7 @@ __device__ __forceinline__ void xB_inv_merge(const PlaneGeo<R, NX, NY, NTT>& G, 
     xB<1>(G, sm, tw);
     return;
   }
-  ITP_WITH_RADIX(G.ax.r1, xB_inv_merge_r, G, sm, tw)
+  ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_inv_merge_r, G, sm, tw)
 }
 
 // ---- y stages (columns) -------------------------------------------------------
@@ -553,19 +669,21 @@ __device__ __forceinline__ void yB_inv_global_r(const PlaneGeo<R, NX, NY, NTT>& 
                                                 const C* __restrict__ spec, const C* tw) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.nxh, G.ay.r2, [&](int t, int b) {
-    C a[R1];
+    SVec<C, R1> a;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) a[i] = spec[(b + G.ay.r2 * i) * G.srs + t];
-    Dft<R1, 1, C>::run(a);
+    for (int i = 0; i < R1; ++i) a.v[i] = spec[(b + G.ay.r2 * i) * G.srs + t];
+    a.open();
+    a.template dft<1>();
     if (R1 > 1) twiddle_stage<R1, true>(a, tw, b);
+    a.close();
 #pragma unroll
-    for (int i = 0; i < R1; ++i) sm[G.colB(t, b, i)] = a[i];
+    for (int i = 0; i < R1; ++i) sm[G.colB(t, b, i)] = a.v[i];
   });
 }
 template <typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void yB_inv_global(const PlaneGeo<R, NX, NY, NTT>& G, C* sm,
                                               const C* __restrict__ spec, const C* tw) {
-  ITP_WITH_RADIX(G.ay.r1, yB_inv_global_r, G, sm, spec, tw)
+  ITP_WITH_RADIX(G.ay.r1, (outlined<C, NY>), yB_inv_global_r, G, sm, spec, tw)
 }
 
 // Stage A on columns (DIR = -1 forward with twiddle after; +1 inverse).
@@ -573,13 +691,15 @@ template <int R2, int DIR, typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void yA_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.nxh, G.ay.r1, [&](int t, int n1) {
-    C a[R2];
+    SVec<C, R2> a;
 #pragma unroll
-    for (int j = 0; j < R2; ++j) a[j] = sm[G.colA(t, n1, j)];
-    Dft<R2, DIR, C>::run(a);
+    for (int j = 0; j < R2; ++j) a.v[j] = sm[G.colA(t, n1, j)];
+    a.open();
+    a.template dft<DIR>();
     if (DIR < 0 && G.ay.r1 > 1) twiddle_stage<R2>(a, tw, n1);
+    a.close();
 #pragma unroll
-    for (int j = 0; j < R2; ++j) sm[G.colA(t, n1, j)] = a[j];
+    for (int j = 0; j < R2; ++j) sm[G.colA(t, n1, j)] = a.v[j];
   });
 }
 template <int R2, typename G_, typename C>
@@ -589,9 +709,9 @@ __device__ __forceinline__ void yA_inv_r(const G_& G, C* sm, const C* tw) { yA_r
 template <int DIR, typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void yA(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
   if (DIR < 0) {
-    ITP_WITH_RADIX(G.ay.r2, yA_fwd_r, G, sm, tw)
+    ITP_WITH_RADIX(G.ay.r2, (outlined<C, NY>), yA_fwd_r, G, sm, tw)
   } else {
-    ITP_WITH_RADIX(G.ay.r2, yA_inv_r, G, sm, tw)
+    ITP_WITH_RADIX(G.ay.r2, (outlined<C, NY>), yA_inv_r, G, sm, tw)
   }
 }
 
@@ -608,22 +728,22 @@ __device__ __forceinline__ void yB_fwd_global_r(const PlaneGeo<R, NX, NY, NTT>& 
                                                 C* __restrict__ spec, const KinFac<R>& kin) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.nxh, G.ay.r2, [&](int t, int b) {
-    C a[R1];
+    SVec<C, R1> a;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) a[i] = sm[G.colB(t, b, i)];
-    Dft<R1, -1, C>::run(a);
-    if (kin.fx) {
+    for (int i = 0; i < R1; ++i) a.v[i] = sm[G.colB(t, b, i)];
+    a.open();
+    a.template dft<-1>();
+    if (kin.fx)
+      scale_by<R1, R>(a, [&](int k1) { return kin_factor(kin, t, (b + G.ay.r2 * k1) * G.kym + G.kya); });
+    a.close();
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) a[k1] = cscale(a[k1], kin_factor(kin, t, (b + G.ay.r2 * k1) * G.kym + G.kya));
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) spec[(b + G.ay.r2 * k1) * G.srs + t] = a[k1];
+    for (int k1 = 0; k1 < R1; ++k1) spec[(b + G.ay.r2 * k1) * G.srs + t] = a.v[k1];
   });
 }
 template <typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void yB_fwd_global(const PlaneGeo<R, NX, NY, NTT>& G, C* sm,
                                               C* __restrict__ spec, const KinFac<R>& kin) {
-  ITP_WITH_RADIX(G.ay.r1, yB_fwd_global_r, G, sm, spec, kin)
+  ITP_WITH_RADIX(G.ay.r1, (outlined<C, NY>), yB_fwd_global_r, G, sm, spec, kin)
 }
 
 // ---- epilogues of the inverse x transform -------------------------------------
@@ -631,12 +751,21 @@ __device__ __forceinline__ void yB_fwd_global(const PlaneGeo<R, NX, NY, NTT>& G,
 // and continue with the forward stage A.
 template <typename R>
 struct EpiMerged {
-  using C = typename CplxOf<R>::type;
-  const C* f;
+  using C = typename SpecOf<R>::type;
+  using CR = typename CplxOf<R>::type;
+  const CR* f;
   int npair, r1;
-  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, C* a) const {
+  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, SVec<C, R2>& a) const {
+    if constexpr (SVec<C, R2>::fixed) {
+      CR q[R2];
 #pragma unroll
-    for (int j = 0; j < R2; ++j) a[j] = cmulri(a[j], __ldg(&f[(n1 + r1 * j) * npair + t]));
+      for (int j = 0; j < R2; ++j) q[j] = __ldg(&f[(n1 + r1 * j) * npair + t]);
+      a.mul_pairs(q);
+    } else {
+#pragma unroll
+      for (int j = 0; j < R2; ++j)
+        a.v[j] = cmulri(a.v[j], __ldg(&f[(n1 + r1 * j) * npair + t]));
+    }
     return true;
   }
 };
@@ -644,27 +773,34 @@ struct EpiMerged {
 // finished sum goes to phi in precision R instead of back to acc.
 template <typename R>
 struct EpiCombine {
-  using C = typename CplxOf<R>::type;
-  const C* f;
+  using C = typename SpecOf<R>::type;
+  using CR = typename CplxOf<R>::type;
+  const CR* f;
   double2* acc;
-  C* phi;
+  CR* phi;
   double c;
   int init, npair, r1;
-  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, C* a) const {
+  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, SVec<C, R2>& a) const {
 #pragma unroll
     for (int j = 0; j < R2; ++j) {
       const int idx = (n1 + r1 * j) * npair + t;
-      const C u = cmulri(a[j], __ldg(&f[idx]));
+      const CR fv = __ldg(&f[idx]);
       double2 v;
-      v.x = c * (double)u.x;
-      v.y = c * (double)u.y;
+      if constexpr (SVec<C, R2>::fixed) {
+        v.x = c * a.to_double_times(a.v[j].x, fv.x);
+        v.y = c * a.to_double_times(a.v[j].y, fv.y);
+      } else {
+        const CR u = cmulri(a.v[j], fv);
+        v.x = c * (double)u.x;
+        v.y = c * (double)u.y;
+      }
       if (!init) {
         const double2 o = acc[idx];
         v.x += o.x;
         v.y += o.y;
       }
       if (phi) {
-        C w;
+        CR w;
         w.x = (R)v.x;
         w.y = (R)v.y;
         phi[idx] = w;
@@ -685,48 +821,42 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
   e += (s - (t - bb)) + (x - bb);
   s = t;
 }
-template <typename R>
 struct EpiCombinePair {
-  using C = typename CplxOf<R>::type;
+  using C = float2;
   const C* f;
   float4* acc;   // per real pair: (s_re, e_re, s_im, e_im)
   C* phi;
   float c;
   int init, npair, r1;
-  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, C* a) const {
+  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, SVec<C, R2>& av) const {
+    const C(&a)[R2] = av.v;
 #pragma unroll
     for (int j = 0; j < R2; ++j) {
       const int idx = (n1 + r1 * j) * npair + t;
       const C fv = __ldg(&f[idx]);
-      const float vx = c * ((float)a[j].x * (float)fv.x);
-      const float vy = c * ((float)a[j].y * (float)fv.y);
+      const float vx = c * (a[j].x * fv.x);
+      const float vy = c * (a[j].y * fv.y);
       float4 q = init ? make_float4(0.f, 0.f, 0.f, 0.f) : acc[idx];
       two_sum_acc(q.x, q.y, vx);
       two_sum_acc(q.z, q.w, vy);
-      if (phi) {
-        C w;
-        w.x = (R)(q.x + q.y);
-        w.y = (R)(q.z + q.w);
-        phi[idx] = w;
-      } else {
-        acc[idx] = q;
-      }
+      if (phi) phi[idx] = make_float2(q.x + q.y, q.z + q.w);
+      else acc[idx] = q;
     }
     return false;
   }
 };
 
-// PLANE_TERM: the term's scaled contribution c * f_out * u, rounded to
-// precision R, written over the term's own spectrum plane (its real plane
-// fits in the half-spectrum plane; all of the plane was read before).
-template <typename R>
+// PLANE_TERM (FP32): the term's scaled contribution c * f_out * u, rounded to
+// FP32, written over the term's own spectrum plane (its real plane fits in
+// the half-spectrum plane; all of the plane was read before).
 struct EpiTerm {
-  using C = typename CplxOf<R>::type;
+  using C = float2;
   const C* f;
   C* out;
-  R c;   // c_i rounded to R: the term is an R value anyway
+  float c;   // c_i rounded to FP32: the term is an FP32 value anyway
   int npair, r1;
-  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, C* a) const {
+  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, SVec<C, R2>& av) const {
+    const C(&a)[R2] = av.v;
 #pragma unroll
     for (int j = 0; j < R2; ++j) {
       const int idx = (n1 + r1 * j) * npair + t;
@@ -747,29 +877,30 @@ struct EpiTerm {
 // instructions then still occupied GB300's narrow FP64 pipe.
 template <typename R>
 struct EpiHpsi {
-  using C = typename CplxOf<R>::type;
-  const C* psi;
+  using C = typename SpecOf<R>::type;
+  using CR = typename CplxOf<R>::type;
+  const CR* psi;
   const double2* V;
   double2* out;
-  const C* Vr;
-  C* outr;
+  const CR* Vr;
+  CR* outr;
   int npair, r1;
-  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, C* a) const {
+  template <int R2> __device__ __forceinline__ bool apply(int t, int n1, SVec<C, R2>& a) const {
 #pragma unroll
     for (int j = 0; j < R2; ++j) {
       const int idx = (n1 + r1 * j) * npair + t;
-      const C q = psi[idx];
+      const CR q = psi[idx];
       if constexpr (sizeof(R) == 4) {
-        const C v = __ldg(&Vr[idx]);
-        C h;
-        h.x = a[j].x + v.x * q.x;
-        h.y = a[j].y + v.y * q.y;
+        const CR v = __ldg(&Vr[idx]);
+        CR h;
+        h.x = a.v[j].x + v.x * q.x;
+        h.y = a.v[j].y + v.y * q.y;
         outr[idx] = h;
       } else {
         const double2 v = __ldg(&V[idx]);
         double2 h;
-        h.x = (double)a[j].x + v.x * (double)q.x;
-        h.y = (double)a[j].y + v.y * (double)q.y;
+        h.x = a.to_double(a.v[j].x) + v.x * q.x;
+        h.y = a.to_double(a.v[j].y) + v.y * q.y;
         out[idx] = h;
       }
     }
@@ -782,7 +913,8 @@ struct EpiHpsi {
 template <typename R, int NX, int NY, int MODE>
 __device__ __forceinline__ void plane_body(const GridDesc& g, const PlaneArgs<R>& a, int z,
                                            int s) {
-  using C = typename CplxOf<R>::type;
+  using C = typename SpecOf<R>::type;
+  using CR = typename CplxOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int NTT = kThreads;
   const PlaneGeo<R, NX, NY, NTT> G(g);
@@ -799,8 +931,8 @@ __device__ __forceinline__ void plane_body(const GridDesc& g, const PlaneArgs<R>
   __syncthreads();
 
   if constexpr (MODE == PLANE_FWD_REAL) {
-    const C* src = reinterpret_cast<const C*>(a.in_real + real_off);
-    const C* f = a.f_in ? reinterpret_cast<const C*>(a.f_in + fac_off) : nullptr;
+    const CR* src = reinterpret_cast<const CR*>(a.in_real + real_off);
+    const CR* f = a.f_in ? reinterpret_cast<const CR*>(a.f_in + fac_off) : nullptr;
     xA_fwd_global(G, sm, src, f, twx);
     __syncthreads();
   } else {
@@ -812,27 +944,28 @@ __device__ __forceinline__ void plane_body(const GridDesc& g, const PlaneArgs<R>
     xB_inv_merge(G, sm, twx);
     __syncthreads();
     if constexpr (MODE == PLANE_MERGED) {
-      EpiMerged<R> epi{reinterpret_cast<const C*>(a.f_mid + fac_off), G.npair, G.ax.r1};
+      EpiMerged<R> epi{reinterpret_cast<const CR*>(a.f_mid + fac_off), G.npair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       __syncthreads();
     } else if constexpr (MODE == PLANE_TERM) {
-      EpiTerm<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off),
-                     static_cast<C*>(a.spec) + spec_off, (R)a.coef, G.npair, G.ax.r1};
+      static_assert(sizeof(R) == 4, "the FP64 path accumulates its terms");
+      EpiTerm epi{reinterpret_cast<const CR*>(a.f_out + fac_off),
+                  static_cast<C*>(a.spec) + spec_off, (R)a.coef, G.npair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       return;
     } else if constexpr (MODE == PLANE_COMBINE) {
-      EpiCombine<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off),
+      EpiCombine<R> epi{reinterpret_cast<const CR*>(a.f_out + fac_off),
                         reinterpret_cast<double2*>(a.acc + real_off),
-                        a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) : nullptr,
+                        a.phi_out ? reinterpret_cast<CR*>(a.phi_out + real_off) : nullptr,
                         a.coef, a.acc_init, G.npair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       return;
     } else {
-      EpiHpsi<R> epi{reinterpret_cast<const C*>(a.in_real + real_off),
+      EpiHpsi<R> epi{reinterpret_cast<const CR*>(a.in_real + real_off),
                      reinterpret_cast<const double2*>(a.V + fac_off),
                      reinterpret_cast<double2*>(a.acc + real_off),
-                     a.V_r ? reinterpret_cast<const C*>(a.V_r + fac_off) : nullptr,
-                     a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) : nullptr,
+                     a.V_r ? reinterpret_cast<const CR*>(a.V_r + fac_off) : nullptr,
+                     a.phi_out ? reinterpret_cast<CR*>(a.phi_out + real_off) : nullptr,
                      G.npair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       return;
@@ -857,6 +990,18 @@ __global__ void __launch_bounds__(launch_threads(kThreads),
 // Grouped plane pass: one launch over the states of several problems with
 // the same grid (a batch of independent problems).  CTA row y of the grid
 // is state rows[y].y of problem rows[y].x, whose arguments are args[rows[y].x].
+// (FP64: one kernel for both forms, to halve the compile time; rows null: the
+// arguments are `a`.)
+template <int NX, int NY, int MODE>
+__global__ void __launch_bounds__(launch_threads(kThreads),
+                                  min_blocks(plane_smem_ct(NX, NY, 8), 2))
+    plane64_kernel(const GridDesc g, const PlaneArgs<double> a,
+                   const PlaneArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
+  const int2 r = rows ? rows[blockIdx.y] : make_int2(0, (int)blockIdx.y);
+  const PlaneArgs<double> la = rows ? args[r.x] : a;
+  plane_body<double, NX, NY, MODE>(g, la, blockIdx.x, r.y);
+}
+
 template <typename R, int NX, int NY, int MODE>
 __global__ void __launch_bounds__(launch_threads(kThreads),
                                   min_blocks(plane_smem_ct(NX, NY, sizeof(R)),
@@ -880,16 +1025,15 @@ __device__ __forceinline__ void pencil_fwdA_r(nt_tag<NT>, C* sm, const C* __rest
                                               int r1) {
   for_tasks<NT>(pw, r1, [&](int t, int n1) {
     if (t >= w) return;
-    C v[R2];
+    SVec<C, R2> v;
 #pragma unroll
-    for (int j = 0; j < R2; ++j) v[j] = base[(n1 + r1 * j) * zstride + t];
-    Dft<R2, -1, C>::run(v);
-    if (r1 > 1) {
+    for (int j = 0; j < R2; ++j) v.v[j] = base[(n1 + r1 * j) * zstride + t];
+    v.open();
+    v.template dft<-1>();
+    if (r1 > 1) twiddle_direct(v, tw, n1);
+    v.close();
 #pragma unroll
-      for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], tw[n1 * j]);
-    }
-#pragma unroll
-    for (int j = 0; j < R2; ++j) sm[(n1 + r1 * j) * pw + t] = v[j];
+    for (int j = 0; j < R2; ++j) sm[(n1 + r1 * j) * pw + t] = v.v[j];
   });
 }
 
@@ -898,29 +1042,32 @@ template <int R1, typename C, typename R, int MODE, int NT>
 __device__ __forceinline__ void pencil_mid_r(nt_tag<NT>, C* sm, const C* tw,
                                              const R* __restrict__ kx_tab,
                                              const R* __restrict__ kz_tab, R fy, R scale, int w,
-                                             int pw, int r2, int kx0, mode_tag<MODE>) {
+                                             int pw, int r2, int kx0, mode_tag<MODE>, int mode) {
   for_tasks<NT>(pw, r2, [&](int t, int b) {
     if (t >= w) return;
-    C v[R1];
+    SVec<C, R1> v;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) v[i] = sm[(i + R1 * b) * pw + t];
-    Dft<R1, -1, C>::run(v);
+    for (int i = 0; i < R1; ++i) v.v[i] = sm[(i + R1 * b) * pw + t];
+    v.open();
+    v.template dft<-1>();
     const R fx = __ldg(&kx_tab[kx0 + t]);
-#pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) {
-      const R fz = __ldg(&kz_tab[b + r2 * k1]);
-      R f;
-      if constexpr (MODE == PENCIL_PROPAGATE) f = fx * fy * fz;
-      else f = (fx + fy + fz) * scale;
-      v[k1] = cscale(v[k1], f);
+    if constexpr (MODE < 0) {   // FP64: p fz + q, one FP64 instruction per value in either mode
+      R p = scale, q = 0;
+      if (mode == PENCIL_PROPAGATE) p = fx * fy;
+      else q = (fx + fy) * scale;
+      scale_by<R1, R>(v, [&](int k1) -> R { return fma(__ldg(&kz_tab[b + r2 * k1]), p, q); });
+    } else {
+      scale_by<R1, R>(v, [&](int k1) -> R {
+        const R fz = __ldg(&kz_tab[b + r2 * k1]);
+        if constexpr (MODE == PENCIL_PROPAGATE) return fx * fy * fz;
+        else return (fx + fy + fz) * scale;
+      });
     }
-    Dft<R1, 1, C>::run(v);
-    if (R1 > 1) {
+    v.template dft<1>();
+    if (R1 > 1) twiddle_direct<true>(v, tw, b);
+    v.close();
 #pragma unroll
-      for (int i = 1; i < R1; ++i) v[i] = cmulc(v[i], tw[i * b]);
-    }
-#pragma unroll
-    for (int i = 0; i < R1; ++i) sm[(i + R1 * b) * pw + t] = v[i];
+    for (int i = 0; i < R1; ++i) sm[(i + R1 * b) * pw + t] = v.v[i];
   });
 }
 
@@ -930,12 +1077,14 @@ __device__ __forceinline__ void pencil_invA_r(nt_tag<NT>, const C* sm, C* __rest
                                               long long zstride, int w, int pw, int r1) {
   for_tasks<NT>(pw, r1, [&](int t, int n1) {
     if (t >= w) return;
-    C v[R2];
+    SVec<C, R2> v;
 #pragma unroll
-    for (int j = 0; j < R2; ++j) v[j] = sm[(n1 + r1 * j) * pw + t];
-    Dft<R2, 1, C>::run(v);
+    for (int j = 0; j < R2; ++j) v.v[j] = sm[(n1 + r1 * j) * pw + t];
+    v.open();
+    v.template dft<1>();
+    v.close();
 #pragma unroll
-    for (int j = 0; j < R2; ++j) base[(n1 + r1 * j) * zstride + t] = v[j];
+    for (int j = 0; j < R2; ++j) base[(n1 + r1 * j) * zstride + t] = v.v[j];
   });
 }
 
@@ -1046,12 +1195,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1)
       xA_inv_then(G, sm, twx, epi);
       __syncthreads();
     } else if constexpr (MODE == PLANE_TERM) {
-      EpiTerm<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
+      EpiTerm epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
                      static_cast<C*>(a.spec) + spec_off + t0, (R)a.coef, G.gpair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       return;
     } else if constexpr (MODE == PLANE_COMBINE) {
-      EpiCombinePair<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
+      EpiCombinePair epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
                             reinterpret_cast<float4*>(a.acc + real_off) + t0,
                             a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) + t0 : nullptr,
                             (float)a.coef, a.acc_init, G.gpair, G.ax.r1};
@@ -1188,12 +1337,12 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kC4Threads, 3)
       xA_inv_then(G, sm, twx, epi);
       __syncthreads();
     } else if constexpr (MODE == PLANE_TERM) {
-      EpiTerm<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
+      EpiTerm epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
                      static_cast<C*>(a.spec) + spec_off + t0, (R)a.coef, G.gpair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       return;
     } else if constexpr (MODE == PLANE_COMBINE) {
-      EpiCombinePair<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
+      EpiCombinePair epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
                             reinterpret_cast<float4*>(a.acc + real_off) + t0,
                             a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) + t0 : nullptr,
                             (float)a.coef, a.acc_init, G.gpair, G.ax.r1};
@@ -1238,7 +1387,8 @@ struct RowGeo : PlaneGeo<R, NX, 2 * TB, kThreads> {
 template <typename R, int NX, int TB, int MODE>
 __global__ void __launch_bounds__(kThreads)
     rowpass_kernel(const GridDesc g, const PlaneArgs<R> a) {
-  using C = typename CplxOf<R>::type;
+  using C = typename SpecOf<R>::type;
+  using CR = typename CplxOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
   const RowGeo<R, NX, TB> G(g);
   C* sm = reinterpret_cast<C*>(smraw);
@@ -1255,8 +1405,8 @@ __global__ void __launch_bounds__(kThreads)
   __syncthreads();
 
   if constexpr (MODE == PLANE_FWD_REAL) {
-    const C* src = reinterpret_cast<const C*>(a.in_real + real_off) + t0;
-    const C* f = a.f_in ? reinterpret_cast<const C*>(a.f_in + fac_off) + t0 : nullptr;
+    const CR* src = reinterpret_cast<const CR*>(a.in_real + real_off) + t0;
+    const CR* f = a.f_in ? reinterpret_cast<const CR*>(a.f_in + fac_off) + t0 : nullptr;
     xA_fwd_global(G, sm, src, f, twx);
     __syncthreads();
   } else {
@@ -1269,30 +1419,30 @@ __global__ void __launch_bounds__(kThreads)
     xB_inv_merge(G, sm, twx);
     __syncthreads();
     if constexpr (MODE == PLANE_MERGED) {
-      EpiMerged<R> epi{reinterpret_cast<const C*>(a.f_mid + fac_off) + t0, G.gpair, G.ax.r1};
+      EpiMerged<R> epi{reinterpret_cast<const CR*>(a.f_mid + fac_off) + t0, G.gpair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       __syncthreads();
     } else if constexpr (MODE == PLANE_COMBINE) {
       if constexpr (sizeof(R) == 4) {
-        EpiCombinePair<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
+        EpiCombinePair epi{reinterpret_cast<const CR*>(a.f_out + fac_off) + t0,
                               reinterpret_cast<float4*>(a.acc + real_off) + t0,
-                              a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) + t0 : nullptr,
+                              a.phi_out ? reinterpret_cast<CR*>(a.phi_out + real_off) + t0 : nullptr,
                               (float)a.coef, a.acc_init, G.gpair, G.ax.r1};
         xA_inv_then(G, sm, twx, epi);
       } else {
-        EpiCombine<R> epi{reinterpret_cast<const C*>(a.f_out + fac_off) + t0,
+        EpiCombine<R> epi{reinterpret_cast<const CR*>(a.f_out + fac_off) + t0,
                           reinterpret_cast<double2*>(a.acc + real_off) + t0,
-                          a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) + t0 : nullptr,
+                          a.phi_out ? reinterpret_cast<CR*>(a.phi_out + real_off) + t0 : nullptr,
                           a.coef, a.acc_init, G.gpair, G.ax.r1};
         xA_inv_then(G, sm, twx, epi);
       }
       return;
     } else if constexpr (MODE == PLANE_HPSI) {
-      EpiHpsi<R> epi{reinterpret_cast<const C*>(a.in_real + real_off) + t0,
+      EpiHpsi<R> epi{reinterpret_cast<const CR*>(a.in_real + real_off) + t0,
                      reinterpret_cast<const double2*>(a.V + fac_off) + t0,
                      reinterpret_cast<double2*>(a.acc + real_off) + t0,
-                     a.V_r ? reinterpret_cast<const C*>(a.V_r + fac_off) + t0 : nullptr,
-                     a.phi_out ? reinterpret_cast<C*>(a.phi_out + real_off) + t0 : nullptr,
+                     a.V_r ? reinterpret_cast<const CR*>(a.V_r + fac_off) + t0 : nullptr,
+                     a.phi_out ? reinterpret_cast<CR*>(a.phi_out + real_off) + t0 : nullptr,
                      G.gpair, G.ax.r1};
       xA_inv_then(G, sm, twx, epi);
       return;
@@ -1310,22 +1460,22 @@ __global__ void __launch_bounds__(kThreads)
 
 // Column pass: the y transform of a block of kx columns of one plane (same
 // slab structure as the pencil pass, along y).
-template <int R1, typename C, int NT>
+template <int R1, typename C, typename R, int NT>
 __device__ __forceinline__ void col_fwdB_store_r(nt_tag<NT>, const C* sm, C* __restrict__ base,
                                                  long long rstride, int w, int pw, int r2,
-                                                 const KinFac<decltype(C{}.x)>& kin, int kx0) {
+                                                 const KinFac<R>& kin, int kx0) {
   for_tasks<NT>(pw, r2, [&](int t, int b) {
     if (t >= w) return;
-    C v[R1];
+    SVec<C, R1> v;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) v[i] = sm[(i + R1 * b) * pw + t];
-    Dft<R1, -1, C>::run(v);
-    if (kin.fx) {
+    for (int i = 0; i < R1; ++i) v.v[i] = sm[(i + R1 * b) * pw + t];
+    v.open();
+    v.template dft<-1>();
+    if (kin.fx)
+      scale_by<R1, R>(v, [&](int k1) { return kin_factor(kin, kx0 + t, b + r2 * k1); });
+    v.close();
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) v[k1] = cscale(v[k1], kin_factor(kin, kx0 + t, b + r2 * k1));
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) base[(b + r2 * k1) * rstride + t] = v[k1];
+    for (int k1 = 0; k1 < R1; ++k1) base[(b + r2 * k1) * rstride + t] = v.v[k1];
   });
 }
 template <int R1, typename C, int NT>
@@ -1334,16 +1484,15 @@ __device__ __forceinline__ void col_invB_load_r(nt_tag<NT>, C* sm, const C* __re
                                                 int r2) {
   for_tasks<NT>(pw, r2, [&](int t, int b) {
     if (t >= w) return;
-    C v[R1];
+    SVec<C, R1> v;
 #pragma unroll
-    for (int i = 0; i < R1; ++i) v[i] = base[(b + r2 * i) * rstride + t];
-    Dft<R1, 1, C>::run(v);
-    if (R1 > 1) {
+    for (int i = 0; i < R1; ++i) v.v[i] = base[(b + r2 * i) * rstride + t];
+    v.open();
+    v.template dft<1>();
+    if (R1 > 1) twiddle_direct<true>(v, tw, b);
+    v.close();
 #pragma unroll
-      for (int i = 1; i < R1; ++i) v[i] = cmulc(v[i], tw[i * b]);
-    }
-#pragma unroll
-    for (int i = 0; i < R1; ++i) sm[(i + R1 * b) * pw + t] = v[i];
+    for (int i = 0; i < R1; ++i) sm[(i + R1 * b) * pw + t] = v.v[i];
   });
 }
 
@@ -1352,7 +1501,7 @@ __global__ void __launch_bounds__(launch_threads(task_threads(W)))
     colpass_kernel(const GridDesc g, void* spec, const void* twy_g, int pw_rt,
                    const KinFac<R> kin) {
   constexpr int NT = task_threads(W);
-  using C = typename CplxOf<R>::type;
+  using C = typename SpecOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const AxisT<NY> ay(g.ny, g.ry1, g.ry2);
@@ -1366,16 +1515,16 @@ __global__ void __launch_bounds__(launch_threads(task_threads(W)))
   C* base = static_cast<C*>(spec) + plane * (long long)ny * g.nxh + kx0;
   __syncthreads();
   if constexpr (DIR < 0) {
-    ITP_WITH_RADIX(ay.r2, pencil_fwdA_r, nt_tag<NT>(), sm, base, twy, (long long)g.nxh, w, pw,
+    ITP_WITH_RADIX(ay.r2, (outlined<C, NY>), pencil_fwdA_r, nt_tag<NT>(), sm, base, twy, (long long)g.nxh, w, pw,
                    ay.r1)
     __syncthreads();
-    ITP_WITH_RADIX(ay.r1, col_fwdB_store_r, nt_tag<NT>(), sm, base, (long long)g.nxh, w, pw,
+    ITP_WITH_RADIX(ay.r1, (outlined<C, NY>), col_fwdB_store_r, nt_tag<NT>(), sm, base, (long long)g.nxh, w, pw,
                    ay.r2, kin, kx0)
   } else {
-    ITP_WITH_RADIX(ay.r1, col_invB_load_r, nt_tag<NT>(), sm, base, twy, (long long)g.nxh, w, pw,
+    ITP_WITH_RADIX(ay.r1, (outlined<C, NY>), col_invB_load_r, nt_tag<NT>(), sm, base, twy, (long long)g.nxh, w, pw,
                    ay.r2)
     __syncthreads();
-    ITP_WITH_RADIX(ay.r2, pencil_invA_r, nt_tag<NT>(), sm, base, (long long)g.nxh, w, pw, ay.r1)
+    ITP_WITH_RADIX(ay.r2, (outlined<C, NY>), pencil_invA_r, nt_tag<NT>(), sm, base, (long long)g.nxh, w, pw, ay.r1)
   }
 }
 
@@ -1385,7 +1534,7 @@ template <typename R, int NZ, int W, int MODE>
 __device__ __forceinline__ void pencil_body(const GridDesc& g, const PencilArgs<R>& a, int bx,
                                             int s) {
   constexpr int NT = task_threads(W);
-  using C = typename CplxOf<R>::type;
+  using C = typename SpecOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const AxisT<NZ> az(g.nz, g.rz1, g.rz2);
@@ -1401,12 +1550,12 @@ __device__ __forceinline__ void pencil_body(const GridDesc& g, const PencilArgs<
   const R fy = a.ky_tab[ky];
   __syncthreads();
 
-  ITP_WITH_RADIX(az.r2, pencil_fwdA_r, nt_tag<NT>(), sm, base, twz, zstride, w, pw, az.r1)
+  ITP_WITH_RADIX(az.r2, (outlined<C, NZ>), pencil_fwdA_r, nt_tag<NT>(), sm, base, twz, zstride, w, pw, az.r1)
   __syncthreads();
-  ITP_WITH_RADIX(az.r1, pencil_mid_r, nt_tag<NT>(), sm, twz, a.kx_tab, a.kz_tab, fy, a.scale, w,
-                 pw, az.r2, kx0, mode_tag<MODE>())
+  ITP_WITH_RADIX(az.r1, (outlined<C, NZ>), pencil_mid_r, nt_tag<NT>(), sm, twz, a.kx_tab, a.kz_tab, fy, a.scale, w,
+                 pw, az.r2, kx0, mode_tag<MODE>(), a.mode)
   __syncthreads();
-  ITP_WITH_RADIX(az.r2, pencil_invA_r, nt_tag<NT>(), sm, base, zstride, w, pw, az.r1)
+  ITP_WITH_RADIX(az.r2, (outlined<C, NZ>), pencil_invA_r, nt_tag<NT>(), sm, base, zstride, w, pw, az.r1)
 }
 
 template <typename R, int NZ, int W, int MODE>
@@ -1415,6 +1564,17 @@ __global__ void __launch_bounds__(launch_threads(task_threads(W)),
                                              pencil_min_ctas(NZ, sizeof(R))))
     pencil_kernel(const GridDesc g, const PencilArgs<R> a) {
   pencil_body<R, NZ, W, MODE>(g, a, blockIdx.x, blockIdx.y);
+}
+
+// FP64 pencil pass, single or grouped (rows set) launches, either mode.
+template <int NZ, int W>
+__global__ void __launch_bounds__(launch_threads(task_threads(W)),
+                                  min_blocks(pencil_smem_ct(NZ, W, 8), pencil_min_ctas(NZ, 8)))
+    pencil64_kernel(const GridDesc g, const PencilArgs<double> a,
+                    const PencilArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
+  const int2 r = rows ? rows[blockIdx.y] : make_int2(0, (int)blockIdx.y);
+  const PencilArgs<double> la = rows ? args[r.x] : a;
+  pencil_body<double, NZ, W, -1>(g, la, blockIdx.x, r.y);
 }
 
 // Grouped pencil pass (see plane_group_kernel).
@@ -1532,26 +1692,30 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 template <typename R, int NX, int NY>
 cudaError_t plane_dispatch(const GridDesc& g, const PlaneArgs<R>& a, size_t smem, cudaStream_t st) {
-  dim3 grid(g.nz, a.m);
-  const int nthr = kThreads;
-  cudaError_t e;
-  switch (a.mode) {
+  if constexpr (sizeof(R) == 8) {
+    return plane64_dispatch<NX, NY>(g, a.mode, a, nullptr, nullptr, a.m, smem, st);
+  } else {
+    dim3 grid(g.nz, a.m);
+    const int nthr = kThreads;
+    cudaError_t e;
+    switch (a.mode) {
 #define ITP_PLANE_CASE(M)                                                   \
-  case M:                                                                   \
-    e = set_smem(plane_kernel<R, NX, NY, M>, smem);                         \
-    if (e != cudaSuccess) return e;                                         \
-    plane_kernel<R, NX, NY, M><<<grid, nthr, smem, st>>>(g, a);             \
-    break;
-    ITP_PLANE_CASE(PLANE_FWD_REAL)
-    ITP_PLANE_CASE(PLANE_MERGED)
-    ITP_PLANE_CASE(PLANE_COMBINE)
-    ITP_PLANE_CASE(PLANE_HPSI)
-    ITP_PLANE_CASE(PLANE_TERM)
+    case M:                                                                 \
+      e = set_smem(plane_kernel<R, NX, NY, M>, smem);                       \
+      if (e != cudaSuccess) return e;                                       \
+      plane_kernel<R, NX, NY, M><<<grid, nthr, smem, st>>>(g, a);           \
+      break;
+      ITP_PLANE_CASE(PLANE_FWD_REAL)
+      ITP_PLANE_CASE(PLANE_MERGED)
+      ITP_PLANE_CASE(PLANE_COMBINE)
+      ITP_PLANE_CASE(PLANE_HPSI)
+      ITP_PLANE_CASE(PLANE_TERM)
 #undef ITP_PLANE_CASE
-    default:
-      return cudaErrorInvalidValue;
+      default:
+        return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 template <typename R, int NZ, int W>
@@ -1561,7 +1725,11 @@ cudaError_t pencil_dispatch(const GridDesc& g, const PencilArgs<R>& a, size_t sm
   dim3 grid(g.ny * chunks, a.m);
   const int nthr = launch_threads(task_threads(W));
   cudaError_t e;
-  if (a.mode == PENCIL_PROPAGATE) {
+  if constexpr (sizeof(R) == 8) {
+    e = set_smem(pencil64_kernel<NZ, W>, smem);
+    if (e != cudaSuccess) return e;
+    pencil64_kernel<NZ, W><<<grid, nthr, smem, st>>>(g, a, nullptr, nullptr);
+  } else if (a.mode == PENCIL_PROPAGATE) {
     e = set_smem(pencil_kernel<R, NZ, W, PENCIL_PROPAGATE>, smem);
     if (e != cudaSuccess) return e;
     pencil_kernel<R, NZ, W, PENCIL_PROPAGATE><<<grid, nthr, smem, st>>>(g, a);
@@ -1574,6 +1742,41 @@ cudaError_t pencil_dispatch(const GridDesc& g, const PencilArgs<R>& a, size_t sm
 }
 
 }  // namespace
+
+// The FP64 plane passes of one plane size, instantiated by translation units
+// of their own: over the a.m states of `a`, or nrows rows of a table (no
+// PLANE_TERM: FP64 terms are accumulated).
+template <int NX, int NY>
+cudaError_t plane64_dispatch(const GridDesc& g, int mode, const PlaneArgs<double>& a,
+                             const PlaneArgs<double>* args, const int2* rows, int nrows,
+                             size_t smem, cudaStream_t st) {
+  dim3 grid(g.nz, nrows);
+  cudaError_t e;
+  switch (mode) {
+#define ITP_PLANE64_CASE(M)                                                     \
+  case M:                                                                       \
+    e = set_smem(plane64_kernel<NX, NY, M>, smem);                              \
+    if (e != cudaSuccess) return e;                                             \
+    plane64_kernel<NX, NY, M><<<grid, kThreads, smem, st>>>(g, a, args, rows);  \
+    break;
+    ITP_PLANE64_CASE(PLANE_FWD_REAL)
+    ITP_PLANE64_CASE(PLANE_MERGED)
+    ITP_PLANE64_CASE(PLANE_COMBINE)
+    ITP_PLANE64_CASE(PLANE_HPSI)
+#undef ITP_PLANE64_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+#ifndef ITP_PLANE64_UNIT   // units that instantiate a size define this
+extern template cudaError_t plane64_dispatch<0, 0>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<32, 32>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<48, 48>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<64, 64>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<96, 96>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<128, 128>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+#endif
 
 template <typename R, int NX, int TB>
 cudaError_t rowpass_dispatch(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_t st) {
@@ -1605,7 +1808,8 @@ cudaError_t rowpass_launch(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_
     if constexpr (sizeof(R) == 4) return rowpass_dispatch<R, 256, 32>(g, a, st);
     else return rowpass_dispatch<R, 256, 16>(g, a, st);
   }
-  if (tb == 32) return rowpass_dispatch<R, 0, 32>(g, a, st);
+  if constexpr (sizeof(R) == 4)
+    if (tb == 32) return rowpass_dispatch<R, 0, 32>(g, a, st);
   if (tb == 16) return rowpass_dispatch<R, 0, 16>(g, a, st);
   if (tb == 8) return rowpass_dispatch<R, 0, 8>(g, a, st);
   return cudaErrorInvalidValue;
@@ -1788,25 +1992,29 @@ cudaError_t launch_transpose_planes(const TS* src, TD* dst, long long nplanes, i
 template <typename R, int NX, int NY>
 cudaError_t plane_group_dispatch(const GridDesc& g, int mode, const PlaneArgs<R>* args,
                                  const int2* rows, int nrows, size_t smem, cudaStream_t st) {
-  dim3 grid(g.nz, nrows);
-  cudaError_t e;
-  switch (mode) {
+  if constexpr (sizeof(R) == 8) {
+    return plane64_dispatch<NX, NY>(g, mode, PlaneArgs<double>{}, args, rows, nrows, smem, st);
+  } else {
+    dim3 grid(g.nz, nrows);
+    cudaError_t e;
+    switch (mode) {
 #define ITP_PLANE_GROUP_CASE(M)                                             \
-  case M:                                                                   \
-    e = set_smem(plane_group_kernel<R, NX, NY, M>, smem);                   \
-    if (e != cudaSuccess) return e;                                         \
-    plane_group_kernel<R, NX, NY, M><<<grid, kThreads, smem, st>>>(g, args, rows); \
-    break;
-    ITP_PLANE_GROUP_CASE(PLANE_FWD_REAL)
-    ITP_PLANE_GROUP_CASE(PLANE_MERGED)
-    ITP_PLANE_GROUP_CASE(PLANE_COMBINE)
-    ITP_PLANE_GROUP_CASE(PLANE_HPSI)
-    ITP_PLANE_GROUP_CASE(PLANE_TERM)
+    case M:                                                                 \
+      e = set_smem(plane_group_kernel<R, NX, NY, M>, smem);                 \
+      if (e != cudaSuccess) return e;                                       \
+      plane_group_kernel<R, NX, NY, M><<<grid, kThreads, smem, st>>>(g, args, rows); \
+      break;
+      ITP_PLANE_GROUP_CASE(PLANE_FWD_REAL)
+      ITP_PLANE_GROUP_CASE(PLANE_MERGED)
+      ITP_PLANE_GROUP_CASE(PLANE_COMBINE)
+      ITP_PLANE_GROUP_CASE(PLANE_HPSI)
+      ITP_PLANE_GROUP_CASE(PLANE_TERM)
 #undef ITP_PLANE_GROUP_CASE
-    default:
-      return cudaErrorInvalidValue;
+      default:
+        return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 template <typename R>
@@ -1834,7 +2042,11 @@ cudaError_t pencil_group_dispatch(const GridDesc& g, int mode, const PencilArgs<
   dim3 grid(g.ny * chunks, nrows);
   const int nthr = launch_threads(task_threads(W));
   cudaError_t e;
-  if (mode == PENCIL_PROPAGATE) {
+  if constexpr (sizeof(R) == 8) {   // (the mode is in the arguments)
+    e = set_smem(pencil64_kernel<NZ, W>, smem);
+    if (e != cudaSuccess) return e;
+    pencil64_kernel<NZ, W><<<grid, nthr, smem, st>>>(g, PencilArgs<double>{}, args, rows);
+  } else if (mode == PENCIL_PROPAGATE) {
     e = set_smem(pencil_group_kernel<R, NZ, W, PENCIL_PROPAGATE>, smem);
     if (e != cudaSuccess) return e;
     pencil_group_kernel<R, NZ, W, PENCIL_PROPAGATE><<<grid, nthr, smem, st>>>(g, args, rows);

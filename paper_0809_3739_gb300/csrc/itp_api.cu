@@ -257,8 +257,9 @@ double mp_coefficient(int i, int k) {
   return (double)num / (double)den;
 }
 
-template <typename R>
-void roots_table(int L, std::vector<R>& out) {
+// exp(-2 pi i j / L), j < L: FP32 values, or the 16-byte fixed-point entries
+// of the FP64 passes (fx_tw: a component c as c 2^29 = h + l 2^-32).
+void roots_table(int L, std::vector<float>& out) {
   out.resize(2 * (size_t)L);
   for (int j = 0; j < L; ++j) {
     double c, s;
@@ -271,8 +272,53 @@ void roots_table(int L, std::vector<R>& out) {
       c = std::cos(ang);
       s = -std::sin(ang);
     }
-    out[2 * j] = (R)c;
-    out[2 * j + 1] = (R)s;
+    out[2 * j] = (float)c;
+    out[2 * j + 1] = (float)s;
+  }
+}
+
+// cos(2 pi j / L) * 2^61 (sine: j - L/4), rounded; by reduction to at most an
+// eighth of a turn and the Taylor series in integers with 2^-120 units, so
+// that every machine gets the same table.
+__int128 fx_cos61(int j, int L) {
+  j = ((j % L) + L) % L;
+  if (2 * j > L) j = L - j;                       // cos(-x) = cos(x)
+  bool neg = false;
+  if (4 * j > L) { neg = true; j = L / 2 - j; }   // cos(pi - x) = -cos(x)
+  const bool sine = 8 * j > L;                    // cos(x) = sin(pi/2 - x)
+  // angle = 2 pi num / den with num/den <= 1/8
+  const int num = sine ? L - 4 * j : j, den = sine ? 4 * L : L;
+  const __int128 one = (__int128)1 << 120;
+  auto mul = [](__int128 a, __int128 b) {   // a b 2^-120, 0 <= a, b <= 2^120
+    const __int128 ah = a >> 60, al = a & (((__int128)1 << 60) - 1);
+    const __int128 bh = b >> 60, bl = b & (((__int128)1 << 60) - 1);
+    return ah * bh + ((ah * bl) >> 60) + ((al * bh) >> 60);
+  };
+  // pi/4 in 2^-120 units: hex digits of pi/4 = 0.C90FDAA2 2168C234 C4C6628B 80DC1C..
+  const __int128 pi4 = ((__int128)0xC90FDAA22168C2LL << 64) | (__int128)0x34C4C6628B80DC1CULL;
+  const __int128 x = pi4 * 8 / den * num;         // 2 pi num / den <= pi/4
+  const __int128 x2 = mul(x, x);
+  __int128 term = sine ? x : one, sum = term;
+  for (int k = sine ? 2 : 1; k < 40; k += 2) {
+    term = -mul(term < 0 ? -term : term, x2) / (k * (k + 1)) * (term < 0 ? -1 : 1);
+    sum += term;
+  }
+  const __int128 r = (sum + ((__int128)1 << 58)) >> 59;
+  return neg ? -r : r;
+}
+
+void roots_table(int L, std::vector<double>& out) {
+  out.resize(2 * (size_t)L);
+  for (int j = 0; j < L; ++j) {
+    int w[4];
+    for (int part = 0; part < 2; ++part) {
+      const __int128 v = part == 0 ? fx_cos61(4 * j, 4 * L) : -fx_cos61(4 * j - L, 4 * L);
+      const __int128 h = (v + ((__int128)1 << 31)) >> 32;
+      const __int128 l = v - (h << 32);
+      w[2 * part] = (int)h;
+      w[2 * part + 1] = (int)std::max<long long>((long long)l, -2147483647LL);
+    }
+    memcpy(&out[2 * j], w, sizeof(w));
   }
 }
 
@@ -295,9 +341,9 @@ int alloc_lane(itp_handle h, Lane<R>& L) {
   if (h->have_V)
     ITP_LAUNCH(h, ITP_KERNEL_OTHER, (launch_convert<double, R>(h->V, L.Vr, (long long)N, h->st)));
   std::vector<R> tx, ty, tz;
-  roots_table<R>(g.nx, tx);
-  roots_table<R>(g.ny, ty);
-  roots_table<R>(g.nz, tz);
+  roots_table(g.nx, tx);
+  roots_table(g.ny, ty);
+  roots_table(g.nz, tz);
   ITP_CUDA(h, cudaMalloc(&L.twx, tx.size() * sizeof(R)));
   ITP_CUDA(h, cudaMalloc(&L.twy, ty.size() * sizeof(R)));
   ITP_CUDA(h, cudaMalloc(&L.twz, tz.size() * sizeof(R)));
