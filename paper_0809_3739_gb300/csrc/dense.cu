@@ -1,8 +1,7 @@
 // Dense n x n side of one iteration (Eq. 4 and the subspace step of
-// Sec. III): Gram sums over the grid, Cholesky + triangular inverse, the
-// symmetric eigen-decomposition, and the application of an n x n matrix to
-// the block of states.  These are the CUDA-core versions; all small-matrix
-// work is FP64.
+// Sec. III): the reduction of the Gram sums, Cholesky + triangular inverse and
+// the symmetric eigen-decomposition, all FP64 (the contractions over the grid
+// are in tc_gemm.cu and fx_gemm.cu).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -15,117 +14,37 @@ namespace itp {
 namespace {
 
 constexpr int kMaxM = 256;   // states of the n x n work at most
-constexpr int kBlk = 128;    // rows of one state block of the Gram and apply kernels
 
 // ---------------------------------------------------------------------------
-// Gram partial sums over chunks of points.  The m x m result is cut into
-// 128 x 128 blocks; CTA (chunk c, block b) sums rows [128 bi, +128) of A
-// against rows [128 bj, +128) of B, (bi, bj) = block b of the list that
-// launch_gram_partial builds (with A == B only bj <= bi, each off-diagonal
-// block also written transposed).  512 threads as 16 (tx) x 32 (ty); thread
-// owns block rows i = ty + 32*q (q < 4) and cols j = tx + 16*r (r < 8).
-// points per shared tile: 32 (FP32) or 16 (FP64), 33 KB of shared tiles;
-// FP32 products are summed over runs of 256 points, then in FP64.
-template <typename TC> struct GramTile { static constexpr int KT = sizeof(TC) == 4 ? 32 : 16; };
-constexpr int kGramRun = 256;
-
-// Block b of the Gram kernels' block list: (bi, bj) packed as bi * 256 + bj.
-struct GramBlocks {
-  int n;
-  int ij[(kMaxM / kBlk) * (kMaxM / kBlk)];
-};
-
-template <typename TA, typename TB, typename TC>
-__global__ void __launch_bounds__(512) gram_partial_kernel(const TA* __restrict__ A,
-                                                           const TB* __restrict__ B, int m,
-                                                           long long N, long long chunk,
-                                                           double* __restrict__ partial,
-                                                           const GramBlocks blocks, int mirror) {
-  constexpr int KT = GramTile<TC>::KT;
-  constexpr int kFlushTiles = kGramRun / KT;
-  __shared__ TC sA[KT][kBlk + 1];
-  __shared__ TC sB[KT][kBlk + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int bi = blocks.ij[blockIdx.y] >> 8, bj = blocks.ij[blockIdx.y] & 255;
-  const int ia = kBlk * bi, jb = kBlk * bj;   // first row of A and of B
-  const long long p_begin = (long long)blockIdx.x * chunk;
-  const long long p_end = min(N, p_begin + chunk);
-  double accd[4][8];
-  TC accf[4][8];
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) { accd[q][r] = 0.0; accf[q][r] = (TC)0; }
-  int tiles_in_run = 0;
-  for (long long p0 = p_begin; p0 < p_end; p0 += KT) {
-    // load tiles: element (row i, point p0 + k)
-    for (int e = threadIdx.x; e < KT * kBlk; e += blockDim.x) {
-      const int i = e / KT, k = e - i * KT;
-      const long long p = p0 + k;
-      TC va = (TC)0, vb = (TC)0;
-      if (p < p_end) {
-        if (ia + i < m) va = (TC)A[(long long)(ia + i) * N + p];
-        if (jb + i < m) vb = (TC)B[(long long)(jb + i) * N + p];
-      }
-      sA[k][i] = va;
-      sB[k][i] = vb;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < KT; ++k) {
-      TC a[4], b[8];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) a[q] = sA[k][ty + 32 * q];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) b[r] = sB[k][tx + 16 * r];
-      if constexpr (sizeof(TC) == 8) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int r = 0; r < 8; ++r) accd[q][r] = fma((double)a[q], (double)b[r], accd[q][r]);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int r = 0; r < 8; ++r) accf[q][r] = fma(a[q], b[r], accf[q][r]);
-      }
-    }
-    __syncthreads();
-    if (sizeof(TC) == 4 && ++tiles_in_run == kFlushTiles) {
-      tiles_in_run = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int r = 0; r < 8; ++r) { accd[q][r] += (double)accf[q][r]; accf[q][r] = (TC)0; }
-    }
-  }
-  double* out = partial + (long long)blockIdx.x * m * m;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = ia + ty + 32 * q;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int j = jb + tx + 16 * r;
-      if (i < m && j < m) {
-        const double v = accd[q][r] + (double)accf[q][r];
-        out[i * m + j] = v;
-        if (mirror && bi != bj) out[j * m + i] = v;
-      }
-    }
-  }
-}
-
-__global__ void gram_reduce_kernel(const double* __restrict__ partial, int n_chunks, int m,
-                                   double scale, int sym, double* __restrict__ G) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= m * m) return;
-  const int i = e / m, j = e - i * m;
+// G = scale * the sum of the chunks' partial sums: 32 entries per CTA, eight
+// warps over the chunks (one thread per entry walked all of them, a chain of
+// up to 608 dependent FP64 additions, 78 cycles each).
+__global__ void __launch_bounds__(256) gram_reduce_kernel(const double* __restrict__ partial,
+                                                          int n_chunks, int m, double scale,
+                                                          int sym, double* __restrict__ G) {
+  __shared__ double ss[8][32], st[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
   double s = 0.0, t = 0.0;
-  for (int c = 0; c < n_chunks; ++c) {
-    s += partial[(long long)c * m * m + i * m + j];
-    if (sym) t += partial[(long long)c * m * m + j * m + i];
+  if (e < m * m) {
+    const int i = e / m, j = e - i * m;
+    const double* p = partial + e;
+    const double* q = partial + j * m + i;
+    for (int c = warp; c < n_chunks; c += 8) {
+      s += p[(long long)c * m * m];
+      if (sym) t += q[(long long)c * m * m];
+    }
   }
-  G[e] = sym ? 0.5 * scale * (s + t) : scale * s;
+  ss[warp][lane] = s;
+  st[warp][lane] = t;
+  __syncthreads();
+  if (warp == 0 && e < m * m) {
+    for (int w = 1; w < 8; ++w) {
+      s += ss[w][lane];
+      t += st[w][lane];
+    }
+    G[e] = sym ? 0.5 * scale * (s + t) : scale * s;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -618,67 +537,6 @@ __global__ void residual_final_kernel(const double* __restrict__ partial, int ch
   out[j] = t * dV;
 }
 
-// ---------------------------------------------------------------------------
-// Y[r0 + i] (=|+=) sum_k M[r0 + i][k0 + k] X[k0 + k] for i < nr, k < nk: one
-// block of Y = M X (the host walks the blocks of 128 rows).  Persistent CTAs
-// over tiles of 32 points; the M block (as TC) stays in shared memory.  512
-// threads: tx = point in tile, ty = row group (16 rows).  lower: M[i][k] = 0
-// for k > i (global indices).  add: the block's product is added to Y.
-constexpr int kApplyPT = 32;
-
-template <typename TX, typename TY, typename TC>
-__global__ void __launch_bounds__(512) apply_matrix_kernel(const double* __restrict__ M, int m,
-                                                           int lower, const TX* __restrict__ X,
-                                                           TY* __restrict__ Y, long long N,
-                                                           int r0, int nr, int k0, int nk,
-                                                           int add) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  TC* sM = reinterpret_cast<TC*>(smraw);            // nr x nk
-  TC* sX = sM + nr * nk;                            // nk x kApplyPT
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // ty in 0..15
-  for (int e = threadIdx.x; e < nr * nk; e += blockDim.x) {
-    const int i = e / nk, k = e - i * nk;
-    sM[e] = (TC)M[(long long)(r0 + i) * m + k0 + k];
-  }
-  const long long ntiles = (N + kApplyPT - 1) / kApplyPT;
-  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const long long p0 = tile * kApplyPT;
-    __syncthreads();
-    for (int e = threadIdx.x; e < nk * kApplyPT; e += blockDim.x) {
-      const int k = e / kApplyPT, j = e - k * kApplyPT;
-      const long long p = p0 + j;
-      sX[e] = (p < N) ? (TC)X[(long long)(k0 + k) * N + p] : (TC)0;
-    }
-    __syncthreads();
-    const long long p = p0 + tx;
-    for (int i0 = ty; i0 < nr; i0 += 16 * 8) {
-      TC acc[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = (TC)0;
-      // lower triangular: row r0 + i needs k0 + k <= r0 + i
-      const int kmax = lower ? max(0, min(nk, r0 + i0 + 16 * 7 + 1 - k0)) : nk;
-      for (int k = 0; k < kmax; ++k) {
-        const TC x = sX[k * kApplyPT + tx];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = i0 + 16 * q;
-          if (i < nr) acc[q] = fma(sM[i * nk + k], x, acc[q]);
-        }
-      }
-      if (p < N) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = i0 + 16 * q;
-          if (i < nr) {
-            TY* y = Y + (long long)(r0 + i) * N + p;
-            *y = add ? (TY)((TC)*y + acc[q]) : (TY)acc[q];
-          }
-        }
-      }
-    }
-  }
-}
-
 template <typename TS, typename TD>
 __global__ void convert_kernel(const TS* __restrict__ src, TD* __restrict__ dst, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -686,33 +544,11 @@ __global__ void convert_kernel(const TS* __restrict__ src, TD* __restrict__ dst,
     dst[i] = (TD)src[i];
 }
 
-template <typename T> struct ComputeOf;
-template <> struct ComputeOf<float> { using type = float; };
-template <> struct ComputeOf<double> { using type = double; };
-
 }  // namespace
-
-template <typename TA, typename TB, typename TC>
-cudaError_t launch_gram_partial(const TA* A, const TB* B, int m, long long n_points, int n_chunks,
-                                double* partial, cudaStream_t st) {
-  if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
-  long long chunk = (n_points + n_chunks - 1) / n_chunks;
-  chunk = (chunk + kGramRun - 1) / kGramRun * kGramRun;
-  // 128 x 128 blocks of the result; A A^T: the lower blocks, mirrored
-  const bool same = (const void*)A == (const void*)B;
-  const int nb = (m + kBlk - 1) / kBlk;
-  GramBlocks blocks{};
-  for (int bi = 0; bi < nb; ++bi)
-    for (int bj = 0; bj < nb; ++bj)
-      if (!same || bj <= bi) blocks.ij[blocks.n++] = bi * 256 + bj;
-  gram_partial_kernel<TA, TB, TC><<<dim3(n_chunks, blocks.n), 512, 0, st>>>(
-      A, B, m, n_points, chunk, partial, blocks, same ? 1 : 0);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_gram_reduce(const double* partial, int n_chunks, int m, double scale, int sym,
                                double* G, cudaStream_t st) {
-  gram_reduce_kernel<<<(m * m + 255) / 256, 256, 0, st>>>(partial, n_chunks, m, scale, sym, G);
+  gram_reduce_kernel<<<(m * m + 31) / 32, 256, 0, st>>>(partial, n_chunks, m, scale, sym, G);
   return cudaGetLastError();
 }
 
@@ -802,52 +638,12 @@ cudaError_t launch_diag(const double* H, int m, double* E, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <typename TX, typename TY>
-cudaError_t launch_apply_matrix(const double* M, int m, int lower, const TX* X, TY* Y,
-                                long long n_points, cudaStream_t st) {
-  using TC = typename ComputeOf<TY>::type;
-  if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
-  const int bm = m < kBlk ? m : kBlk;   // rows of an M block
-  const size_t smem = ((size_t)bm * bm + (size_t)bm * kApplyPT) * sizeof(TC);
-  cudaError_t e = cudaFuncSetAttribute(apply_matrix_kernel<TX, TY, TC>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const long long ntiles = (n_points + kApplyPT - 1) / kApplyPT;
-  const long long cap = (long long)sms * (smem > 110000 ? 1 : 2);
-  const int blocks = (int)(ntiles < cap ? ntiles : cap);
-  // Y block bi = sum over bk of M[bi][bk] X[bk] (bk <= bi when lower), in
-  // stream order: the first block product sets Y[bi], the others add to it
-  for (int r0 = 0; r0 < m; r0 += kBlk) {
-    const int nr = m - r0 < kBlk ? m - r0 : kBlk;
-    for (int k0 = 0; k0 < m && (!lower || k0 <= r0 + nr - 1); k0 += kBlk) {
-      const int nk = m - k0 < kBlk ? m - k0 : kBlk;
-      apply_matrix_kernel<TX, TY, TC><<<blocks, 512, smem, st>>>(M, m, lower, X, Y, n_points,
-                                                                 r0, nr, k0, nk, k0 > 0);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return cudaSuccess;
-}
-
 template <typename TS, typename TD>
 cudaError_t launch_convert(const TS* src, TD* dst, long long count, cudaStream_t st) {
   convert_kernel<TS, TD><<<4 * 152, 256, 0, st>>>(src, dst, count);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_gram_partial<double, double, double>(const double*, const double*, int,
-                                                                 long long, int, double*,
-                                                                 cudaStream_t);
-template cudaError_t launch_apply_matrix<double, double>(const double*, int, int, const double*,
-                                                         double*, long long, cudaStream_t);
-template cudaError_t launch_apply_matrix<double, float>(const double*, int, int, const double*,
-                                                        float*, long long, cudaStream_t);
-template cudaError_t launch_apply_matrix<float, float>(const double*, int, int, const float*,
-                                                       float*, long long, cudaStream_t);
 template cudaError_t launch_convert<float, double>(const float*, double*, long long, cudaStream_t);
 template cudaError_t launch_convert<double, float>(const double*, float*, long long, cudaStream_t);
 template cudaError_t launch_convert<double, double>(const double*, double*, long long, cudaStream_t);

@@ -1,0 +1,439 @@
+// FP64 contractions over the grid in integer arithmetic: the overlap and the
+// subspace matrix (Gram), and the update by an m x m matrix.
+//
+// The FP64 form of these kernels was bound by the FP64 pipe, one instruction
+// per 78 cycles and sub-partition (128 states at 128^3: 65 ms per Gram matrix,
+// 58 ms per update, and the Gram computed 128 x 128 products however few the
+// states).  A 32 x 32 + 64-bit integer multiply-add (IMAD.WIDE) issues every
+// 2 cycles.  So the operands are scaled to integers of 55 or 56 bits, split
+// into two signed halves v = h 2^28 + l, and a product takes
+//   Gram:   h h', and h l' + l h' (l l' is below the precision, see there);
+//   update: h h', h l' + l h', and l l',
+// accumulated exactly in 64-bit integers over up to 512 terms.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "fft_fixed.cuh"
+#include "itp_kernels.cuh"
+
+namespace itp {
+
+namespace {
+
+constexpr int kMaxM = 256;   // states of the n x n work at most
+constexpr int kBlk = 128;    // rows of one state block of the update
+constexpr int kHalf = 28;    // bits of the lower half
+
+// The double d as an integer of scale 2^(BITS - 1) at the biased exponent e
+// (|d| < 2^(e - 1022)): |result| <= 2^BITS, rounded to nearest, 0 for
+// subnormal d; as halves (h, l) with l in [-2^27, 2^27).
+template <int BITS>
+__device__ __forceinline__ int2 to_halves(double d, int e) {
+  const long long b = __double_as_longlong(d);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  constexpr int kUp = 9;   // 53-bit mantissa to 62 bits: room to round
+  long long m = ((b & 0xfffffffffffffLL) | 0x10000000000000LL) << kUp;
+  const int s = fx_max(1, fx_min(e - ex + (53 + kUp - BITS), 63));   // >= 7 for finite d != 0
+  m = (m + ((1LL << s) >> 1)) >> s;
+  m = ex == 0 ? 0 : m;
+  const long long sg = b >> 63;
+  m = (m ^ sg) - sg;
+  int2 r;
+  r.x = (int)((m + (1LL << (kHalf - 1))) >> kHalf);
+  r.y = (int)((unsigned)m << (32 - kHalf)) >> (32 - kHalf);
+  return r;
+}
+// Biased exponent of |d| (0: zero or subnormal, 2047: not finite).
+__device__ __forceinline__ int exponent(double d) {
+  return (__double2hiint(d) >> 20) & 0x7ff;
+}
+// The same of d 2^x: kNone for zero or subnormal d, kNotFinite for infinity
+// and NaN.
+constexpr int kNone = -(1 << 16), kNotFinite = 1 << 16;
+__device__ __forceinline__ int scaled_exponent(double d, int x) {
+  const int e = exponent(d);
+  return e == 0 ? kNone : (e == 2047 ? kNotFinite : e + x);
+}
+// 2^k as a double, k clamped to the normal range
+__device__ __forceinline__ double pow2(int k) {
+  k = fx_max(-1022, fx_min(1023, k));
+  return __longlong_as_double((long long)(k + 1023) << 52);
+}
+// s * 2^k by the exponent field; in two multiplications where that leaves the
+// normal range
+__device__ __forceinline__ double scale2(double s, int k) {
+  const int e = exponent(s) + k;
+  if (e > 0 && e < 2047 && exponent(s) != 0)
+    return __hiloint2double(__double2hiint(s) + (k << 20), __double2loint(s));
+  return s * pow2(k / 2) * pow2(k - k / 2);
+}
+// N pairs from shared memory, 16 bytes at a time where N is even (p is then
+// 16-byte aligned)
+template <int N>
+__device__ __forceinline__ void load_pairs(const int2* p, int2 (&v)[N]) {
+  if constexpr (N % 2 == 0) {
+#pragma unroll
+    for (int q = 0; q < N; q += 2) {
+      const int4 w = *reinterpret_cast<const int4*>(p + q);
+      v[q] = make_int2(w.x, w.y);
+      v[q + 1] = make_int2(w.z, w.w);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = p[q];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Gram partial sums P[c][i][j] = sum over the points p of chunk c of
+// A[i][p] B[j][p].  The result is cut into blocks of 16 TT rows and columns;
+// a CTA of 16 x 16 threads sums one block over one chunk, TT x TT entries per
+// thread (TT up to 4: 64 x 64 blocks, so that few states do not pay for
+// 128).  A chunk is walked in runs of kRun points: the run's largest
+// exponent of every row first (the reads bring the run into L2), then tiles
+// of kTile points converted into shared memory as halves, [point][row].
+//
+// Precision: with the row's largest value in the run scaled to 2^54, an
+// element is off by at most 2^-55 of it and the missing l l' by about 2^-56
+// of the two largest values, with random signs, so a sum is off by less than
+// one FP64 rounding of |A_i| |B_j| whatever the states' shape.
+constexpr int kRun = 512;
+constexpr int kTile = 16;   // (32 points needed more registers for the tile in flight)
+constexpr int kGramBits = 54;
+
+// (bi, bj) of the blocks, packed as bi * 256 + bj.
+struct GramBlocks {
+  int n;
+  short ij[16];
+};
+
+template <int TT>
+__global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
+    fx_gram_kernel(const double* __restrict__ A, const double* __restrict__ B, int m, long long N,
+                   long long chunk, double* __restrict__ partial, const GramBlocks blocks,
+                   int same) {
+  constexpr int ROWS = 16 * TT;            // rows of a block
+  constexpr int PITCH = ROWS + 2;          // 16-byte rows of pairs, few bank conflicts
+  constexpr int PER = ROWS * kTile / 256;  // elements per thread and operand tile (TT)
+  __shared__ __align__(16) int2 sA[kTile][PITCH];
+  __shared__ __align__(16) int2 sB[kTile][PITCH];
+  __shared__ int eA[ROWS], eB[ROWS];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
+  const int bi = blocks.ij[blockIdx.y] >> 8, bj = blocks.ij[blockIdx.y] & 255;
+  const bool one = same && bi == bj;       // a diagonal block: one operand
+  const int ia = ROWS * bi, jb = ROWS * bj;
+  const long long p_begin = (long long)blockIdx.x * chunk;
+  const long long p_end = p_begin + chunk < N ? p_begin + chunk : N;
+  double* out = partial + (long long)blockIdx.x * m * m;
+  // this CTA's sums stay in its slice of `partial` (L2) between runs
+  auto add_sum = [&](int i, int j, double v, bool first) {
+    if (i >= m || j >= m) return;
+    if (!first) v += out[i * m + j];
+    out[i * m + j] = v;
+    if (same && bi != bj) out[j * m + i] = v;
+  };
+  if (p_begin >= p_end) {
+#pragma unroll
+    for (int q = 0; q < TT; ++q)
+#pragma unroll
+      for (int r = 0; r < TT; ++r) add_sum(ia + ty * TT + q, jb + tx * TT + r, 0.0, true);
+  }
+
+  // element q of this thread's share of a tile: point tx, row ty + 16 q
+  auto load = [&](const double* X, int r0, long long p0, long long pe, double (&v)[PER]) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int i = ty + 16 * q;
+      const long long p = p0 + tx;
+      v[q] = (r0 + i < m && p < pe) ? X[(long long)(r0 + i) * N + p] : 0.0;
+    }
+  };
+  for (long long run = p_begin; run < p_end; run += kRun) {
+    const long long re = run + kRun < p_end ? run + kRun : p_end;
+    // largest exponents, one warp per row
+    for (int op = 0; op < (one ? 1 : 2); ++op) {
+      const double* X = op == 0 ? A : B;
+      const int r0 = op == 0 ? ia : jb;
+      for (int i = warp; i < ROWS; i += 8) {
+        int e = 0;
+        if (r0 + i < m) {
+          const double* row = X + (long long)(r0 + i) * N + run;
+#pragma unroll 8
+          for (int k = lane; k < (int)(re - run); k += 32) e = fx_max(e, exponent(row[k]));
+        }
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) (op == 0 ? eA : eB)[i] = e;
+      }
+    }
+    __syncthreads();
+    long long hh[TT][TT], hl[TT][TT];
+#pragma unroll
+    for (int q = 0; q < TT; ++q)
+#pragma unroll
+      for (int r = 0; r < TT; ++r) hh[q][r] = hl[q][r] = 0;
+    double va[PER], vb[PER];
+    load(A, ia, run, re, va);
+    if (!one) load(B, jb, run, re, vb);
+    const int2(*tB)[PITCH] = one ? sA : sB;
+    int done = 0;
+    for (long long p0 = run; p0 < re; p0 += kTile) {
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        const int i = ty + 16 * q;
+        sA[tx][i] = to_halves<kGramBits>(va[q], eA[i]);
+        if (!one) sB[tx][i] = to_halves<kGramBits>(vb[q], eB[i]);
+      }
+      __syncthreads();
+      if (p0 + kTile < re) {   // the next tile's loads are in flight meanwhile
+        load(A, ia, p0 + kTile, re, va);
+        if (!one) load(B, jb, p0 + kTile, re, vb);
+      }
+#pragma unroll 2
+      for (int k = 0; k < kTile; ++k) {
+        int2 a[TT], b[TT];
+        load_pairs(&sA[k][ty * TT], a);
+        load_pairs(&tB[k][tx * TT], b);
+#pragma unroll
+        for (int q = 0; q < TT; ++q)
+#pragma unroll
+          for (int r = 0; r < TT; ++r) {
+            hh[q][r] = fx_wide(a[q].x, b[r].x, hh[q][r]);   // <= 512 * 2^52
+            hl[q][r] = fx_wide(a[q].x, b[r].y, hl[q][r]);   // <= 256 * 2^54, see below
+            hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
+          }
+      }
+      __syncthreads();
+      done += kTile;
+      if (done == kRun / 2) {   // keep the middle sums within 64 bits
+#pragma unroll
+        for (int q = 0; q < TT; ++q)
+#pragma unroll
+          for (int r = 0; r < TT; ++r) {
+            hh[q][r] += hl[q][r] >> kHalf;
+            hl[q][r] &= (1LL << kHalf) - 1;
+          }
+      }
+    }
+    // the run's sums to FP64: (hh 2^56 + hl 2^28) 2^(ea + eb - 2 * (1022 + 54))
+#pragma unroll
+    for (int q = 0; q < TT; ++q) {
+      const int ea = eA[ty * TT + q];
+#pragma unroll
+      for (int r = 0; r < TT; ++r) {
+        const int eb = (one ? eA : eB)[tx * TT + r];
+        const double s = fma((double)hh[q][r], (double)(1LL << kHalf), (double)hl[q][r]);
+        double v = scale2(s, ea + eb - 2 * (1022 + kGramBits) + kHalf);
+        if (ea == 2047 || eb == 2047) v = __longlong_as_double(0x7ff8000000000000LL);
+        add_sum(ia + ty * TT + q, jb + tx * TT + r, v, run == p_begin);
+      }
+    }
+    __syncthreads();   // the exponents are rewritten by the next run
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Y[r0 + i] (=|+=) sum_k M[r0 + i][k0 + k] X[k0 + k] for i < nr, k < nk (both
+// <= 4 RG): one block of Y = M X.  Persistent CTAs of 256 threads over tiles
+// of PT = 1024 / RG points.  State k is scaled by the power of two nearest
+// to its norm, from the diagonal of its overlap matrix S (null: all states of
+// norm one), and column k of M by the inverse; the rows of that M, scaled by
+// their largest entry to 55 bits, stay in shared memory as halves [k][i], a
+// tile of X, each point scaled by its largest value over the states, comes
+// as halves [k][point].
+// A thread holds 4 rows x 4 points.  lower: M[i][k] = 0 for k > i (global
+// indices), so a row group stops there; warps w and w + 4, which share a
+// sub-partition, take row groups that add up to the same work.
+//
+// Precision: products are exact in 110 bits, so a sum is off by the rounding
+// of its operands, 2^-56 of the largest |M_ik| times the point's largest
+// |X_k| (both scaled) per term with random signs, and the rounding to a double;
+// an FP64 sum rounds by up to 2^-53 of the same size.
+constexpr int kApplyBits = 55;
+
+template <int RG>
+__global__ void __launch_bounds__(256)
+    fx_apply_kernel(const double* __restrict__ M, int m, int lower, const double* __restrict__ S,
+                    const double* __restrict__ X, double* __restrict__ Y, long long N, int r0, int nr, int k0, int nk, int add) {
+  constexpr int ROWS = 4 * RG, TX = 256 / RG, PT = 4 * TX;
+  constexpr int MP = ROWS + 2;                    // pitch of sM (16-byte rows)
+  constexpr int STEP = PT >= 256 ? 1 : 256 / PT;  // threads per point of a tile load
+  constexpr int PER = ROWS / STEP;
+  static_assert(PT <= 256, "at least four row groups");
+  extern __shared__ __align__(16) unsigned char smraw[];
+  int2* sM = reinterpret_cast<int2*>(smraw);      // [ROWS k][MP]
+  int2* sX = sM + ROWS * MP;                      // [ROWS k][PT]
+  int* eM = reinterpret_cast<int*>(sX + ROWS * PT);   // [ROWS]
+  int* xs = eM + ROWS;                            // [ROWS] scales of the states
+  int* eX = xs + ROWS;                            // [STEP][PT]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // thread -> (row group, point): the warps of the upper half in reverse
+  int ty = tid / TX;
+  const int tx = tid - ty * TX;
+  if (tid >= 128) ty = RG / 2 + (RG - 1 - ty);
+  for (int k = tid; k < ROWS; k += 256) {
+    const int e = S && k < nk ? exponent(S[(long long)(k0 + k) * (m + 1)]) : 0;
+    xs[k] = e > 0 && e < 2047 ? (e - 1023) >> 1 : 0;
+  }
+  __syncthreads();
+  for (int i = warp; i < ROWS; i += 8) {
+    int e = kNone;
+    if (i < nr)
+      for (int k = lane; k < nk; k += 32)
+        e = fx_max(e, scaled_exponent(M[(long long)(r0 + i) * m + k0 + k], xs[k]));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) eM[i] = e;
+    for (int k = lane; k < ROWS; k += 32)
+      sM[k * MP + i] = i < nr && k < nk
+                           ? to_halves<kApplyBits>(M[(long long)(r0 + i) * m + k0 + k], e - xs[k])
+                           : make_int2(0, 0);
+  }
+  const long long ntiles = (N + PT - 1) / PT;
+  const int lp = tid & (PT - 1), lk = tid / PT;   // tile load: point, first state
+  auto load = [&](long long tile, double (&v)[PER]) {
+    const long long p = tile * PT + lp;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int k = lk + STEP * q;
+      v[q] = (k < nk && p < N) ? X[(long long)(k0 + k) * N + p] : 0.0;
+    }
+  };
+  double v[PER];
+  if ((long long)blockIdx.x < ntiles) load(blockIdx.x, v);
+  const int kmax = lower ? fx_max(0, fx_min(nk, r0 + 4 * ty + 4 - k0)) : nk;
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    int e = kNone;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) e = fx_max(e, scaled_exponent(v[q], -xs[lk + STEP * q]));
+    __syncthreads();   // the previous tile is consumed (and M is stored)
+    eX[lk * PT + lp] = e;
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < STEP; ++s) e = fx_max(e, eX[s * PT + lp]);
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      sX[(lk + STEP * q) * PT + lp] = to_halves<kApplyBits>(v[q], e + xs[lk + STEP * q]);
+    __syncthreads();
+    if (tile + gridDim.x < ntiles) load(tile + gridDim.x, v);   // in flight meanwhile
+    long long hh[4][4], hl[4][4], ll[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) hh[q][r] = hl[q][r] = ll[q][r] = 0;
+#pragma unroll 2
+    for (int k = 0; k < kmax; ++k) {
+      int2 a[4], b[4];
+      load_pairs(&sM[k * MP + 4 * ty], a);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) b[r] = sX[k * PT + tx + TX * r];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {   // 128 terms: <= 2^61, 2^62, 2^61
+          hh[q][r] = fx_wide(a[q].x, b[r].x, hh[q][r]);
+          hl[q][r] = fx_wide(a[q].x, b[r].y, hl[q][r]);
+          hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
+          ll[q][r] = fx_wide(a[q].y, b[r].y, ll[q][r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const long long p = tile * PT + tx + TX * r;
+      if (p >= N) continue;
+      int ex = kNone;
+#pragma unroll
+      for (int s = 0; s < STEP; ++s) ex = fx_max(ex, eX[s * PT + tx + TX * r]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = 4 * ty + q;
+        if (i >= nr) continue;
+        // hh 2^56 + hl 2^28 + ll, normalised to 62 bits
+        const long long mid = hl[q][r] + (ll[q][r] >> kHalf);
+        const long long top = hh[q][r] + (mid >> kHalf);
+        const long long low = (long long)((unsigned long long)mid << (64 - kHalf));
+        const int th = fx_hi(top);
+        const int n = fx_max(0, fx_clz((unsigned)(th ^ (th >> 31))) - 2);
+        const long long w = n == 0 ? top
+                                   : (long long)(((unsigned long long)top << n) |
+                                                 ((unsigned long long)low >> (64 - n)));
+        const int em = eM[i];
+        const int ev = em == kNotFinite || ex == kNotFinite
+                           ? kFxPoison
+                           : em + ex - 2 * (1022 + kApplyBits) + 2 * kHalf - n + kFxBias;
+        double* y = Y + (long long)(r0 + i) * N + p;
+        const double d = fx_to_double(w, ev);
+        *y = add ? *y + d : d;
+      }
+    }
+  }
+}
+
+template <int TT>
+cudaError_t gram_launch(const double* A, const double* B, int m, long long N, long long chunk,
+                        int n_chunks, double* partial, const GramBlocks& blocks, int same,
+                        cudaStream_t st) {
+  fx_gram_kernel<TT><<<dim3(n_chunks, blocks.n), 256, 0, st>>>(A, B, m, N, chunk, partial, blocks,
+                                                              same);
+  return cudaGetLastError();
+}
+
+template <int RG>
+cudaError_t apply_launch(const double* M, int m, int lower, const double* S, const double* X,
+                         double* Y, long long N, int sms, cudaStream_t st) {
+  constexpr int ROWS = 4 * RG, PT = 1024 / RG, STEP = PT >= 256 ? 1 : 256 / PT;
+  const size_t smem = ((size_t)ROWS * (ROWS + 2) + (size_t)ROWS * PT) * sizeof(int2) +
+                      ((size_t)2 * ROWS + (size_t)STEP * PT) * sizeof(int);
+  cudaError_t e = cudaFuncSetAttribute(fx_apply_kernel<RG>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const long long ntiles = (N + PT - 1) / PT, cap = (long long)sms * (RG == 32 ? 1 : 2);
+  const int grid = (int)(ntiles < cap ? ntiles : cap);
+  // Y block bi = sum over bk of M[bi][bk] X[bk] (bk <= bi when lower), in
+  // stream order: the first block product sets Y[bi], the others add to it
+  for (int r0 = 0; r0 < m; r0 += kBlk) {
+    const int nr = m - r0 < kBlk ? m - r0 : kBlk;
+    for (int k0 = 0; k0 < m && (!lower || k0 <= r0 + nr - 1); k0 += kBlk) {
+      const int nk = m - k0 < kBlk ? m - k0 : kBlk;
+      fx_apply_kernel<RG><<<grid, 256, smem, st>>>(M, m, lower, S, X, Y, N, r0, nr, k0, nk, k0 > 0);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t launch_gram_partial(const double* A, const double* B, int m, long long n_points,
+                                int n_chunks, double* partial, cudaStream_t st) {
+  if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
+  long long chunk = (n_points + n_chunks - 1) / n_chunks;
+  chunk = (chunk + kTile - 1) / kTile * kTile;
+  // blocks of at most 64 rows, as few as that takes and then as small; A A^T:
+  // the lower blocks, mirrored
+  const bool same = A == B;
+  const int nb = (m + 63) / 64, tt = (m + 16 * nb - 1) / (16 * nb);
+  GramBlocks blocks{};
+  for (int bi = 0; bi < nb; ++bi)
+    for (int bj = 0; bj < nb; ++bj)
+      if (!same || bj <= bi) blocks.ij[blocks.n++] = (short)(bi * 256 + bj);
+  switch (tt) {
+    case 1: return gram_launch<1>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
+    case 2: return gram_launch<2>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
+    case 3: return gram_launch<3>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
+    default: return gram_launch<4>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
+  }
+}
+
+cudaError_t launch_apply_matrix(const double* M, int m, int lower, const double* S,
+                                const double* X, double* Y, long long n_points, cudaStream_t st) {
+  if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (m <= 16) return apply_launch<4>(M, m, lower, S, X, Y, n_points, sms, st);
+  if (m <= 32) return apply_launch<8>(M, m, lower, S, X, Y, n_points, sms, st);
+  if (m <= 64) return apply_launch<16>(M, m, lower, S, X, Y, n_points, sms, st);
+  return apply_launch<32>(M, m, lower, S, X, Y, n_points, sms, st);
+}
+
+}  // namespace itp

@@ -562,14 +562,14 @@ int orthonormalize_lane(itp_handle h);
 template <>
 int orthonormalize_lane<double>(itp_handle h) {
   Lane<double>& L = h->f64;
-  ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial<double, double, double>(
+  ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial(
                                      h->acc, h->acc, h->m, h->g.n_points, h->n_chunks,
                                      h->partial, h->st)));
   ITP_LAUNCH(h, ITP_KERNEL_GRAM_REDUCE,
              launch_gram_reduce(h->partial, h->n_chunks, h->m, h->dV, 1, h->S, h->st));
   ITP_LAUNCH(h, ITP_KERNEL_CHOLESKY, launch_cholesky_inverse(h->S, h->m, h->Mx, h->status, h->st));
-  ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix<double, double>(
-                                      h->Mx, h->m, 1, h->acc, L.psi, h->g.n_points, h->st)));
+  ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix(
+                                      h->Mx, h->m, 1, h->S, h->acc, L.psi, h->g.n_points, h->st)));
   h->launches += apply_launches(h->m, true) - 1;
   return ITP_OK;
 }
@@ -644,7 +644,7 @@ int energies_lane(itp_handle h, int flags) {
                                        g.n_points, h->n_chunks_tc, h->partial, h->status,
                                        h->st, tc_expire(h))));
   } else {
-    ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial<double, double, double>(
+    ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial(
                                        reinterpret_cast<const double*>(L.psi), h->acc, h->m,
                                        g.n_points, h->n_chunks, h->partial, h->st)));
   }
@@ -660,8 +660,8 @@ int energies_lane(itp_handle h, int flags) {
                                           h->status, h->st, tc_expire(h))));
       h->launches += apply_launches(h->m, false) - 1;
     } else {
-      ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix<double, double>(
-                                          h->Mx, h->m, 0, reinterpret_cast<const double*>(L.psi),
+      ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix(
+                                          h->Mx, h->m, 0, nullptr, reinterpret_cast<const double*>(L.psi),
                                           reinterpret_cast<double*>(L.psi_tmp), g.n_points,
                                           h->st)));
       h->launches += apply_launches(h->m, false) - 1;
@@ -930,7 +930,7 @@ int autotune_lane(itp_handle h, int k, double tau, std::string& rep) {
           e = launch_tc_gram(h->f32.psi_tmp, h->f32.psi_tmp, h->m, g.n_points, chunks,
                              h->partial, h->status, h->st);
         else
-          e = launch_gram_partial<double, double, double>(h->acc, h->acc, h->m, g.n_points,
+          e = launch_gram_partial(h->acc, h->acc, h->m, g.n_points,
                                                           chunks, h->partial, h->st);
         return e == cudaSuccess ? ITP_OK : fail(h, ITP_ERR_CUDA, "gram: %s",
                                                 cudaGetErrorString(e));

@@ -146,12 +146,10 @@ template <typename TS, typename TD>
 cudaError_t launch_transpose_planes(const TS* src, TD* dst, long long nplanes, int rows,
                                     int cols, cudaStream_t st);
 
-// ---- dense part (dense.cu) ----
-// Partial Gram sums: P[c][i][j] = sum_{p in chunk c} A[i][p] * B[j][p],
-// multiplied in precision TC (FP32 products are summed in FP32 over runs of
-// 256 points and those runs in FP64).
-template <typename TA, typename TB, typename TC>
-cudaError_t launch_gram_partial(const TA* A, const TB* B, int m, long long n_points,
+// ---- dense part (dense.cu, fx_gemm.cu, tc_gemm.cu) ----
+// Partial Gram sums P[c][i][j] = sum_{p in chunk c} A[i][p] * B[j][p] to FP64
+// accuracy, in integer arithmetic (fx_gemm.cu).
+cudaError_t launch_gram_partial(const double* A, const double* B, int m, long long n_points,
                                 int n_chunks, double* partial, cudaStream_t st);
 // G = scale * sum_c P[c] (fixed order), symmetrised if sym.
 cudaError_t launch_gram_reduce(const double* partial, int n_chunks, int m, double scale,
@@ -183,11 +181,12 @@ cudaError_t launch_axpby(double a, const R* X, double b, const R* Y, R* out, lon
 // E[j] = H[j][j]
 cudaError_t launch_diag(const double* H, int m, double* E, cudaStream_t st);
 // Y = M * X over all points: Y[i][p] = sum_k M[i][k] X[k][p]   (M lower
-// triangular if lower != 0), computed in the precision of TY.  X and Y must
-// not overlap.
-template <typename TX, typename TY>
-cudaError_t launch_apply_matrix(const double* M, int m, int lower, const TX* X, TY* Y,
-                                long long n_points, cudaStream_t st);
+// triangular if lower != 0) to FP64 accuracy, in integer arithmetic
+// (fx_gemm.cu).  S: a matrix whose diagonal holds the squared norms of the
+// rows of X up to a common factor (their overlap matrix), or null where the
+// norms are alike.  X and Y must not overlap.
+cudaError_t launch_apply_matrix(const double* M, int m, int lower, const double* S,
+                                const double* X, double* Y, long long n_points, cudaStream_t st);
 // Tensor-core (tcgen05 TF32, 3xTF32 split) versions, m <= 256; status gets
 // bit 4 if a bounded mbarrier wait expired (the kernel then leaves its
 // output unwritten).  expire_ns != 0 is the failure-detection test hook:

@@ -72,11 +72,11 @@ extern "C" int itp_orthonormalize_noalloc(const double* phi_device, double* psi_
   // the array keeps the last call's contents: the status word must start at 0
   if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return ITP_ERR_CUDA;
   using namespace itp;
-  if (launch_gram_partial<double, double, double>(phi_device, phi_device, m, n_points,
+  if (launch_gram_partial(phi_device, phi_device, m, n_points,
                                                   kNoallocChunks, partial, st) != cudaSuccess ||
       launch_gram_reduce(partial, kNoallocChunks, m, dV, 1, S, st) != cudaSuccess ||
       launch_cholesky_inverse(S, m, Minv, status, st) != cudaSuccess ||
-      launch_apply_matrix<double, double>(Minv, m, 1, phi_device, psi_device, n_points, st) !=
+      launch_apply_matrix(Minv, m, 1, S, phi_device, psi_device, n_points, st) !=
           cudaSuccess)
     return ITP_ERR_CUDA;
   int h_status = 0;
