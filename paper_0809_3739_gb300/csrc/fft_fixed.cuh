@@ -61,7 +61,23 @@ ITP_HD int fx_clz(unsigned v) {
 }
 ITP_HD int fx_max(int a, int b) { return a > b ? a : b; }
 ITP_HD int fx_min(int a, int b) { return a < b ? a : b; }
+// v >> n, n >= 0 (63 and more: the sign)
+ITP_HD long long fx_shr(long long v, int n) {
+#ifdef __CUDA_ARCH__
+  long long r;   // the instruction clamps the count
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return v >> (n > 63 ? 63 : n);
+#endif
+}
 ITP_HD long long fx_shl(long long v, int n) { return (long long)((unsigned long long)v << n); }
+// v * p for p = 2^n, n < 32: a left shift on the multiplier, which the passes
+// keep less busy than the shifter
+ITP_HD long long fx_mulp(long long v, unsigned p) {
+  const long long lo = (long long)((unsigned long long)fx_lo(v) * p);
+  return lo + ((long long)((unsigned long long)((unsigned)fx_hi(v) * p) << 32));
+}
 ITP_HD long long fx_bits(double d) {
 #ifdef __CUDA_ARCH__
   return __double_as_longlong(d);
@@ -246,9 +262,9 @@ template <int N> struct SVec<cfx, N> {
     const int top = em + kFxDrop + EXTRA;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const int s = fx_min(top - ei[i], 63);
-      v[i].x >>= s;
-      v[i].y >>= s;
+      const int s = top - ei[i];
+      v[i].x = fx_shr(v[i].x, s);
+      v[i].y = fx_shr(v[i].y, s);
     }
     e = em == kFxTop ? kFxPoison : top;
   }
@@ -278,12 +294,12 @@ template <int N> struct SVec<cfx, N> {
     const int n = fx_clz((unsigned)top_word()) - 1;
     int es = e - n;
     if (e >= kFxTop) es = kFxTop;
-    const bool under = es < 0;
-    es = under ? 0 : es;
+    const unsigned p = es < 0 ? 0u : 1u << n;   // zero below the exponent range
+    es = fx_max(es, 0);
     const unsigned ex = (unsigned)es & 63u, ey = (unsigned)es >> 6;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      long long x = under ? 0 : fx_shl(v[i].x, n), y = under ? 0 : fx_shl(v[i].y, n);
+      const long long x = fx_mulp(v[i].x, p), y = fx_mulp(v[i].y, p);
       v[i].x = (x & ~63LL) | (long long)ex;
       v[i].y = (y & ~63LL) | (long long)ey;
     }
@@ -327,8 +343,8 @@ template <int N> struct SVec<cfx, N> {
     constexpr int kDown = HASF ? 5 : 4;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      v[i].x >>= fx_min(em - ex[i] + kDown, 63);
-      v[i].y >>= fx_min(em - ey[i] + kDown, 63);
+      v[i].x = fx_shr(v[i].x, em - ex[i] + kDown);
+      v[i].y = fx_shr(v[i].y, em - ey[i] + kDown);
     }
     // a double is mant 2^(ex - 1023 - 52), here mant 2^8
     e = em - 1023 - 52 - 8 + kDown + kFxBias + (HASF ? -1023 : 0);
@@ -358,8 +374,8 @@ template <int N> struct SVec<cfx, N> {
     const int r = fx_max(0, 7 - fx_clz((unsigned)fx_max(mx, ~mn)));
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      v[i].x >>= fx_min(em - ex[i] + r, 63);
-      v[i].y >>= fx_min(em - ey[i] + r, 63);
+      v[i].x = fx_shr(v[i].x, em - ex[i] + r);
+      v[i].y = fx_shr(v[i].y, em - ey[i] + r);
     }
     e = e >= kFxPoison || em == 2047 ? kFxPoison : e + em - 1023 + r;
   }
