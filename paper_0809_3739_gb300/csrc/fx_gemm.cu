@@ -104,7 +104,7 @@ constexpr int kGramBits = 54;
 // (bi, bj) of the blocks, packed as bi * 256 + bj.
 struct GramBlocks {
   int n;
-  short ij[16];
+  short ij[64];
 };
 
 template <int TT>
@@ -115,8 +115,8 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
   constexpr int ROWS = 16 * TT;            // rows of a block
   constexpr int PITCH = ROWS + 2;          // 16-byte rows of pairs, few bank conflicts
   constexpr int PER = ROWS * kTile / 256;  // elements per thread and operand tile (TT)
-  __shared__ __align__(16) int2 sA[kTile][PITCH];
-  __shared__ __align__(16) int2 sB[kTile][PITCH];
+  __shared__ __align__(16) int2 sA[2][kTile][PITCH];   // two tiles: one barrier per tile
+  __shared__ __align__(16) int2 sB[2][kTile][PITCH];
   __shared__ int eA[ROWS], eB[ROWS];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
   const int bi = blocks.ij[blockIdx.y] >> 8, bj = blocks.ij[blockIdx.y] & 255;
@@ -174,37 +174,48 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
     double va[PER], vb[PER];
     load(A, ia, run, re, va);
     if (!one) load(B, jb, run, re, vb);
-    const int2(*tB)[PITCH] = one ? sA : sB;
-    int done = 0;
-    for (long long p0 = run; p0 < re; p0 += kTile) {
+    auto store = [&](int buf) {
 #pragma unroll
       for (int q = 0; q < PER; ++q) {
         const int i = ty + 16 * q;
-        sA[tx][i] = to_halves<kGramBits>(va[q], eA[i]);
-        if (!one) sB[tx][i] = to_halves<kGramBits>(vb[q], eB[i]);
+        sA[buf][tx][i] = to_halves<kGramBits>(va[q], eA[i]);
+        if (!one) sB[buf][tx][i] = to_halves<kGramBits>(vb[q], eB[i]);
+      }
+    };
+    store(0);
+    const int ntile = (int)((re - run + kTile - 1) / kTile);
+    for (int t = 0; t < ntile; ++t) {
+      const bool more = t + 1 < ntile;
+      if (more) {   // the next tile's loads are in flight meanwhile
+        const long long p0 = run + (long long)(t + 1) * kTile;
+        load(A, ia, p0, re, va);
+        if (!one) load(B, jb, p0, re, vb);
       }
       __syncthreads();
-      if (p0 + kTile < re) {   // the next tile's loads are in flight meanwhile
-        load(A, ia, p0 + kTile, re, va);
-        if (!one) load(B, jb, p0 + kTile, re, vb);
-      }
+      const int2(*tA)[PITCH] = sA[t & 1];
+      const int2(*tB)[PITCH] = one ? sA[t & 1] : sB[t & 1];
 #pragma unroll 2
       for (int k = 0; k < kTile; ++k) {
         int2 a[TT], b[TT];
-        load_pairs(&sA[k][ty * TT], a);
+        load_pairs(&tA[k][ty * TT], a);
         load_pairs(&tB[k][tx * TT], b);
 #pragma unroll
         for (int q = 0; q < TT; ++q)
 #pragma unroll
-          for (int r = 0; r < TT; ++r) {
+          for (int r = 0; r < TT; ++r)
             hh[q][r] = fx_wide(a[q].x, b[r].x, hh[q][r]);   // <= 512 * 2^52
+#pragma unroll
+        for (int q = 0; q < TT; ++q)
+#pragma unroll
+          for (int r = 0; r < TT; ++r)
             hl[q][r] = fx_wide(a[q].x, b[r].y, hl[q][r]);   // <= 256 * 2^54, see below
-            hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
-          }
+#pragma unroll
+        for (int q = 0; q < TT; ++q)
+#pragma unroll
+          for (int r = 0; r < TT; ++r) hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
       }
-      __syncthreads();
-      done += kTile;
-      if (done == kRun / 2) {   // keep the middle sums within 64 bits
+      if (more) store((t + 1) & 1);
+      if ((t + 1) * kTile == kRun / 2) {   // keep the middle sums within 64 bits
 #pragma unroll
         for (int q = 0; q < TT; ++q)
 #pragma unroll
@@ -233,49 +244,82 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
 
 // ---------------------------------------------------------------------------
 // Y[r0 + i] (=|+=) sum_k M[r0 + i][k0 + k] X[k0 + k] for i < nr, k < nk (both
-// <= 4 RG): one block of Y = M X.  Persistent CTAs of 256 threads over tiles
+// <= 4 RG): one block of Y = M X.  Persistent CTAs of 512 threads over tiles
 // of PT = 1024 / RG points.  State k is scaled by the power of two nearest
 // to its norm, from the diagonal of its overlap matrix S (null: all states of
 // norm one), and column k of M by the inverse; the rows of that M, scaled by
-// their largest entry to 55 bits, stay in shared memory as halves [k][i], a
+// their largest entry to 55 bits, stay in shared memory as halves [k][i]; a
 // tile of X, each point scaled by its largest value over the states, comes
-// as halves [k][point].
-// A thread holds 4 rows x 4 points.  lower: M[i][k] = 0 for k > i (global
-// indices), so a row group stops there; warps w and w + 4, which share a
-// sub-partition, take row groups that add up to the same work.
+// as halves [k][point] into one of two buffers while the other one is
+// multiplied (one barrier per tile).  A thread holds 4 rows x 2 points.
+// lower: M[i][k] = 0 for k > i (global indices), so a row group stops there;
+// the four warps that share a sub-partition take row groups that add up to
+// the same work.
 //
 // Precision: products are exact in 110 bits, so a sum is off by the rounding
 // of its operands, 2^-56 of the largest |M_ik| times the point's largest
 // |X_k| (both scaled) per term with random signs, and the rounding to a double;
 // an FP64 sum rounds by up to 2^-53 of the same size.
 constexpr int kApplyBits = 55;
+constexpr int kApplyThreads = 512;
+
+// hh 2^56 + hl 2^28 + ll as a double, times 2^k (k far below: 0; poison: NaN).
+__device__ __forceinline__ double sum_to_double(long long hh, long long hl, long long ll, int k,
+                                                bool poison) {
+  const long long mid = hl + (ll >> kHalf);
+  const long long top = hh + (mid >> kHalf);   // value = (top + low 2^-32) 2^56
+  unsigned w2 = (unsigned)(top >> 32), w1 = (unsigned)top, w0 = (unsigned)mid << (32 - kHalf);
+  const unsigned s = (unsigned)((int)w2 >> 31);
+  w2 ^= s;   // magnitude, to one unit of 2^24
+  w1 ^= s;
+  w0 ^= s;
+  const bool far = w2 == 0;   // cancelled by 2^-32 or more: the lower words
+  const int z = __clz(far ? w1 : w2);
+  const unsigned hi = __funnelshift_l(far ? w0 : w1, far ? w1 : w2, z);
+  const unsigned lo = __funnelshift_l(far ? 0u : w0, far ? w0 : w1, z);
+  // hi:lo is normalised (bit 63 set) unless the value is zero
+  const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+  const long long q = (long long)(m >> 11) + (long long)((m >> 10) & 1ull);
+  const int be = 1023 + 56 + 63 - z - (far ? 32 : 0) + k;
+  double r = be > 0 && be < 2047 ? __longlong_as_double(q + ((long long)(be - 1) << 52))
+                                 : (be >= 2047 ? __longlong_as_double(0x7ff0000000000000LL) : 0.0);
+  if (hi == 0) r = 0.0;
+  if (poison) r = __longlong_as_double(0x7ff8000000000000LL);
+  return s ? -r : r;
+}
 
 template <int RG>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kApplyThreads)
     fx_apply_kernel(const double* __restrict__ M, int m, int lower, const double* __restrict__ S,
-                    const double* __restrict__ X, double* __restrict__ Y, long long N, int r0, int nr, int k0, int nk, int add) {
-  constexpr int ROWS = 4 * RG, TX = 256 / RG, PT = 4 * TX;
+                    const double* __restrict__ X, double* __restrict__ Y, long long N, int r0,
+                    int nr, int k0, int nk, int add) {
+  constexpr int NP = 2;                           // points per thread
+  constexpr int ROWS = 4 * RG, TX = kApplyThreads / RG, PT = NP * TX;
   constexpr int MP = ROWS + 2;                    // pitch of sM (16-byte rows)
-  constexpr int STEP = PT >= 256 ? 1 : 256 / PT;  // threads per point of a tile load
+  constexpr int STEP = kApplyThreads / PT;        // threads per point of a tile load
   constexpr int PER = ROWS / STEP;
-  static_assert(PT <= 256, "at least four row groups");
+  static_assert(PT <= 256 && STEP >= 2, "four to thirty-two row groups");
   extern __shared__ __align__(16) unsigned char smraw[];
   int2* sM = reinterpret_cast<int2*>(smraw);      // [ROWS k][MP]
-  int2* sX = sM + ROWS * MP;                      // [ROWS k][PT]
-  int* eM = reinterpret_cast<int*>(sX + ROWS * PT);   // [ROWS]
+  int2* sX = sM + ROWS * MP;                      // [2][ROWS k][PT]
+  int* eM = reinterpret_cast<int*>(sX + 2 * ROWS * PT);   // [ROWS]
   int* xs = eM + ROWS;                            // [ROWS] scales of the states
-  int* eX = xs + ROWS;                            // [STEP][PT]
+  int* eX = xs + ROWS;                            // [3][STEP][PT]: tile t in slot t % 3, as
+                                                  // slower warps still read tile t - 1's
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // thread -> (row group, point): the warps of the upper half in reverse
-  int ty = tid / TX;
-  const int tx = tid - ty * TX;
-  if (tid >= 128) ty = RG / 2 + (RG - 1 - ty);
-  for (int k = tid; k < ROWS; k += 256) {
+  // thread -> (row group, point).  Warps w, w + 4, w + 8, w + 12 share a
+  // sub-partition: every other group of four warps is taken in reverse.
+  constexpr int WPG = TX >= 32 ? TX / 32 : 1;     // warps per row group
+  const int wr = (warp & 4) ? (warp ^ 3) : warp;
+  const int vt = TX > 32 ? tid : wr * 32 + lane;  // (row groups wider than a warp: as they come)
+  const int ty = vt / TX, tx = vt - ty * TX;
+  (void)WPG;
+  for (int k = tid; k < ROWS; k += kApplyThreads) {
     const int e = S && k < nk ? exponent(S[(long long)(k0 + k) * (m + 1)]) : 0;
     xs[k] = e > 0 && e < 2047 ? (e - 1023) >> 1 : 0;
   }
   __syncthreads();
-  for (int i = warp; i < ROWS; i += 8) {
+  for (int i = warp; i < ROWS; i += kApplyThreads / 32) {
     int e = kNone;
     if (i < nr)
       for (int k = lane; k < nk; k += 32)
@@ -289,81 +333,91 @@ __global__ void __launch_bounds__(256)
   }
   const long long ntiles = (N + PT - 1) / PT;
   const int lp = tid & (PT - 1), lk = tid / PT;   // tile load: point, first state
-  auto load = [&](long long tile, double (&v)[PER]) {
+  double v[PER];
+  auto load = [&](long long tile) {
     const long long p = tile * PT + lp;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       const int k = lk + STEP * q;
-      v[q] = (k < nk && p < N) ? X[(long long)(k0 + k) * N + p] : 0.0;
+      v[q] = (tile < ntiles && k < nk && p < N) ? X[(long long)(k0 + k) * N + p] : 0.0;
     }
   };
-  double v[PER];
-  if ((long long)blockIdx.x < ntiles) load(blockIdx.x, v);
-  const int kmax = lower ? fx_max(0, fx_min(nk, r0 + 4 * ty + 4 - k0)) : nk;
-  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  auto put_exponent = [&](int slot) {
     int e = kNone;
 #pragma unroll
     for (int q = 0; q < PER; ++q) e = fx_max(e, scaled_exponent(v[q], -xs[lk + STEP * q]));
-    __syncthreads();   // the previous tile is consumed (and M is stored)
-    eX[lk * PT + lp] = e;
-    __syncthreads();
+    eX[(slot * STEP + lk) * PT + lp] = e;
+  };
+  auto point_exponent = [&](int slot, int p) {
+    int e = kNone;
 #pragma unroll
-    for (int s = 0; s < STEP; ++s) e = fx_max(e, eX[s * PT + lp]);
+    for (int s = 0; s < STEP; ++s) e = fx_max(e, eX[(slot * STEP + s) * PT + p]);
+    return e;
+  };
+  auto convert = [&](int buf, int slot) {
+    const int e = point_exponent(slot, lp);
 #pragma unroll
     for (int q = 0; q < PER; ++q)
-      sX[(lk + STEP * q) * PT + lp] = to_halves<kApplyBits>(v[q], e + xs[lk + STEP * q]);
-    __syncthreads();
-    if (tile + gridDim.x < ntiles) load(tile + gridDim.x, v);   // in flight meanwhile
-    long long hh[4][4], hl[4][4], ll[4][4];
+      sX[(buf * ROWS + lk + STEP * q) * PT + lp] =
+          to_halves<kApplyBits>(v[q], e + xs[lk + STEP * q]);
+  };
+  load(blockIdx.x);
+  put_exponent(0);
+  __syncthreads();
+  convert(0, 0);
+  load((long long)blockIdx.x + gridDim.x);
+  const int kmax = lower ? fx_max(0, fx_min(nk, r0 + 4 * ty + 4 - k0)) : nk;
+  int buf = 0, slot = 0;
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int next = slot == 2 ? 0 : slot + 1;
+    put_exponent(next);
+    __syncthreads();   // this tile is stored, the other buffer's last reader done
+    convert(buf ^ 1, next);
+    load(tile + 2LL * gridDim.x);   // in flight meanwhile
+    long long hh[4][NP], hl[4][NP], ll[4][NP];
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) hh[q][r] = hl[q][r] = ll[q][r] = 0;
-#pragma unroll 2
+      for (int r = 0; r < NP; ++r) hh[q][r] = hl[q][r] = ll[q][r] = 0;
+    const int2* xb = sX + buf * ROWS * PT + tx;
+#pragma unroll 4
     for (int k = 0; k < kmax; ++k) {
-      int2 a[4], b[4];
+      int2 a[4], b[NP];
       load_pairs(&sM[k * MP + 4 * ty], a);
 #pragma unroll
-      for (int r = 0; r < 4; ++r) b[r] = sX[k * PT + tx + TX * r];
+      for (int r = 0; r < NP; ++r) b[r] = xb[k * PT + TX * r];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {   // 128 terms: <= 2^61, 2^62, 2^61
+        for (int r = 0; r < NP; ++r) {   // 128 terms: <= 2^61, 2^62, 2^61
           hh[q][r] = fx_wide(a[q].x, b[r].x, hh[q][r]);
           hl[q][r] = fx_wide(a[q].x, b[r].y, hl[q][r]);
-          hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
           ll[q][r] = fx_wide(a[q].y, b[r].y, ll[q][r]);
         }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < NP; ++r) hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < NP; ++r) {
       const long long p = tile * PT + tx + TX * r;
       if (p >= N) continue;
-      int ex = kNone;
-#pragma unroll
-      for (int s = 0; s < STEP; ++s) ex = fx_max(ex, eX[s * PT + tx + TX * r]);
+      const int ex = point_exponent(slot, tx + TX * r);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int i = 4 * ty + q;
         if (i >= nr) continue;
-        // hh 2^56 + hl 2^28 + ll, normalised to 62 bits
-        const long long mid = hl[q][r] + (ll[q][r] >> kHalf);
-        const long long top = hh[q][r] + (mid >> kHalf);
-        const long long low = (long long)((unsigned long long)mid << (64 - kHalf));
-        const int th = fx_hi(top);
-        const int n = fx_max(0, fx_clz((unsigned)(th ^ (th >> 31))) - 2);
-        const long long w = n == 0 ? top
-                                   : (long long)(((unsigned long long)top << n) |
-                                                 ((unsigned long long)low >> (64 - n)));
         const int em = eM[i];
-        const int ev = em == kNotFinite || ex == kNotFinite
-                           ? kFxPoison
-                           : em + ex - 2 * (1022 + kApplyBits) + 2 * kHalf - n + kFxBias;
+        const double d = sum_to_double(hh[q][r], hl[q][r], ll[q][r],
+                                       em + ex - 2 * (1022 + kApplyBits),
+                                       em == kNotFinite || ex == kNotFinite);
         double* y = Y + (long long)(r0 + i) * N + p;
-        const double d = fx_to_double(w, ev);
         *y = add ? *y + d : d;
       }
     }
+    buf ^= 1;
+    slot = next;
   }
 }
 
@@ -379,9 +433,9 @@ cudaError_t gram_launch(const double* A, const double* B, int m, long long N, lo
 template <int RG>
 cudaError_t apply_launch(const double* M, int m, int lower, const double* S, const double* X,
                          double* Y, long long N, int sms, cudaStream_t st) {
-  constexpr int ROWS = 4 * RG, PT = 1024 / RG, STEP = PT >= 256 ? 1 : 256 / PT;
-  const size_t smem = ((size_t)ROWS * (ROWS + 2) + (size_t)ROWS * PT) * sizeof(int2) +
-                      ((size_t)2 * ROWS + (size_t)STEP * PT) * sizeof(int);
+  constexpr int ROWS = 4 * RG, PT = 2 * kApplyThreads / RG, STEP = kApplyThreads / PT;
+  const size_t smem = ((size_t)ROWS * (ROWS + 2) + 2 * (size_t)ROWS * PT) * sizeof(int2) +
+                      (2 * (size_t)ROWS + 3 * (size_t)STEP * PT) * sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(fx_apply_kernel<RG>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -393,7 +447,7 @@ cudaError_t apply_launch(const double* M, int m, int lower, const double* S, con
     const int nr = m - r0 < kBlk ? m - r0 : kBlk;
     for (int k0 = 0; k0 < m && (!lower || k0 <= r0 + nr - 1); k0 += kBlk) {
       const int nk = m - k0 < kBlk ? m - k0 : kBlk;
-      fx_apply_kernel<RG><<<grid, 256, smem, st>>>(M, m, lower, S, X, Y, N, r0, nr, k0, nk, k0 > 0);
+      fx_apply_kernel<RG><<<grid, kApplyThreads, smem, st>>>(M, m, lower, S, X, Y, N, r0, nr, k0, nk, k0 > 0);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
@@ -409,10 +463,19 @@ cudaError_t launch_gram_partial(const double* A, const double* B, int m, long lo
   long long chunk = (n_points + n_chunks - 1) / n_chunks;
   chunk = (chunk + kTile - 1) / kTile * kTile;
   // blocks of at most 64 rows, as few as that takes and then as small; A A^T:
-  // the lower blocks, mirrored
+  // the lower blocks, mirrored.  Smaller blocks where that leaves SMs idle
+  // (few chunks: a caller's scratch limits them).
   const bool same = A == B;
-  const int nb = (m + 63) / 64, tt = (m + 16 * nb - 1) / (16 * nb);
   GramBlocks blocks{};
+  int tt = 4;
+  for (int cap = 64; cap >= 32; cap -= 16) {
+    const int nb = (m + cap - 1) / cap;
+    tt = (m + 16 * nb - 1) / (16 * nb);
+    blocks.n = same ? nb * (nb + 1) / 2 : nb * nb;
+    if (blocks.n * (long long)n_chunks >= 304) break;
+  }
+  const int nb = (m + 16 * tt - 1) / (16 * tt);
+  blocks.n = 0;
   for (int bi = 0; bi < nb; ++bi)
     for (int bj = 0; bj < nb; ++bj)
       if (!same || bj <= bi) blocks.ij[blocks.n++] = (short)(bi * 256 + bj);

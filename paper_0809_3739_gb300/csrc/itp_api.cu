@@ -80,7 +80,8 @@ struct itp_grid {
   bool cur64 = true;          // which lane holds the states
   bool have_V = false, have_states = false, have_phi = false;
   int n_chunks = 0;           // Gram partial sums (CUDA-core kernels)
-  int n_chunks_tc = 0;        // Gram partial sums (tensor-core kernel, one CTA per SM)
+  int n_chunks_tc = 0;        // Gram partial sums (tensor-core kernel: one CTA per SM, FP32
+                              // cores: two)
   double* partial = nullptr;  // [n_chunks][m][m]
   double* S = nullptr;        // [m][m]
   double* Mx = nullptr;       // [m][m]
@@ -1515,7 +1516,7 @@ int itp_create_grid(itp_handle* out, int nx, int ny, int nz, double lx, double l
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   h->n_chunks = 2 * sms;
-  h->n_chunks_tc = sms;
+  h->n_chunks_tc = h->m <= kF32MaxM ? 2 * sms : sms;
   const size_t N = (size_t)g.n_points, m = (size_t)h->m;
   int rc;
 #define ITP_CREATE(expr)           \

@@ -203,6 +203,13 @@ template <typename TX, typename TY>
 cudaError_t launch_tc_apply(const double* M, int m, const TX* X, TY* Y, long long n_points,
                             int* status, cudaStream_t st, unsigned long long expire_ns = 0,
                             int lower = 0);
+// The same on the FP32 cores for few states (f32_gemm.cu): m <= kF32MaxM,
+// n_points a multiple of 4, A, B, X and Y 16-byte aligned.
+constexpr int kF32MaxM = 64;
+cudaError_t launch_f32_gram(const float* A, const float* B, int m, long long n_points,
+                            int n_chunks, double* partial, cudaStream_t st);
+cudaError_t launch_f32_apply(const double* M, int m, int lower, const float* X, float* Y,
+                             long long n_points, cudaStream_t st);
 // Precision conversion of whole state blocks.
 template <typename TS, typename TD>
 cudaError_t launch_convert(const TS* src, TD* dst, long long count, cudaStream_t st);

@@ -19,7 +19,7 @@
 namespace {
 
 constexpr int kNoallocMaxM = 128;                // states per call at most
-constexpr int kNoallocChunks = 32;               // partial sums of the overlap
+constexpr int kNoallocChunks = 32;               // partial sums of the overlap at 128 states
 constexpr size_t kPartialDoubles = (size_t)kNoallocChunks * kNoallocMaxM * kNoallocMaxM;
 constexpr size_t kMatDoubles = (size_t)kNoallocMaxM * kNoallocMaxM;
 // partials (4 MiB) | S (128 KiB) | L^{-1} (128 KiB) | status (256 B)
@@ -72,9 +72,11 @@ extern "C" int itp_orthonormalize_noalloc(const double* phi_device, double* psi_
   // the array keeps the last call's contents: the status word must start at 0
   if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return ITP_ERR_CUDA;
   using namespace itp;
-  if (launch_gram_partial(phi_device, phi_device, m, n_points,
-                                                  kNoallocChunks, partial, st) != cudaSuccess ||
-      launch_gram_reduce(partial, kNoallocChunks, m, dV, 1, S, st) != cudaSuccess ||
+  // fewer states leave room for more partial sums, up to two CTAs per SM
+  const int room = (int)(kPartialDoubles / ((size_t)m * m));
+  const int chunks = room < 304 ? room : 304;
+  if (launch_gram_partial(phi_device, phi_device, m, n_points, chunks, partial, st) != cudaSuccess ||
+      launch_gram_reduce(partial, chunks, m, dV, 1, S, st) != cudaSuccess ||
       launch_cholesky_inverse(S, m, Minv, status, st) != cudaSuccess ||
       launch_apply_matrix(Minv, m, 1, S, phi_device, psi_device, n_points, st) !=
           cudaSuccess)

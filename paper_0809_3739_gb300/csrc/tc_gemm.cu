@@ -531,6 +531,10 @@ cudaError_t launch_tc_gram(const float* A, const float* B, int m, long long n_po
   if (m > 256 || m < 1 || (n_points % 8) || n_points >= (1LL << 31)) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15)
     return cudaErrorInvalidValue;
+  // few states: the FP32 cores (a tile here is 128 rows whatever m is); the
+  // expiry test hook needs these kernels
+  if (m <= kF32MaxM && !expire_ns)
+    return launch_f32_gram(A, B, m, n_points, n_chunks, partial, st);
   long long chunk = (n_points + n_chunks - 1) / n_chunks;
   chunk = (chunk + kGramKT - 1) / kGramKT * kGramKT;
   const bool same = A == B;
@@ -574,6 +578,8 @@ cudaError_t launch_tc_apply(const double* M, int m, const TX* X, TY* Y, long lon
                             int* status, cudaStream_t st, unsigned long long expire_ns,
                             int lower) {
   if (m > 256 || m < 1) return cudaErrorInvalidValue;
+  if (m <= kF32MaxM && !expire_ns && (n_points & 3) == 0)
+    return launch_f32_apply(M, m, lower, X, Y, n_points, st);
   // M hi/lo 128 KB, two X stages 64 KB, output staging 18 KB
   const size_t smem = 2 * (size_t)kMBytes + 4 * (size_t)kXTileBytes + 128 * (kApplyNT + 4) * 4;
   cudaError_t e = cudaFuncSetAttribute(tc_apply_kernel<TX, TY>,
