@@ -48,9 +48,25 @@ constexpr int kFxPoison = 1 << 20;     // exponent of a poisoned open vector
 
 ITP_HD int fx_hi(long long v) { return (int)(v >> 32); }
 ITP_HD unsigned fx_lo(long long v) { return (unsigned)v; }
-ITP_HD long long fx_wide(int a, int b, long long c) { return (long long)a * b + c; }
+// a * b + c as one instruction (the compiler made two or three of the C form:
+// FP64 merged pass of 48 states at 128^3 2.15 -> 1.74 ms)
+ITP_HD long long fx_wide(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return (long long)a * b + c;
+#endif
+}
 ITP_HD long long fx_wideu(unsigned a, unsigned b, long long c) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
   return (long long)((unsigned long long)a * b + (unsigned long long)c);
+#endif
 }
 ITP_HD int fx_clz(unsigned v) {
 #ifdef __CUDA_ARCH__
