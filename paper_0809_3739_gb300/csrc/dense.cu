@@ -48,188 +48,354 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const double* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky S = L L^T and M = L^{-1} (right-looking, column by column) on a
-// cluster of kClus CTAs, for the FP64 rate: an SM retires about two FP64 FMAs per clock, so the O(m^3) work is spread
-// over the cluster's SMs.  CTA r owns rows [r*rp, r*rp + rp) of S (lower
-// part) and of R = I - sum_j L[:, j] M[j, :], in its shared memory; other
-// CTAs read them through distributed shared memory.  Step k (one cluster
-// barrier): every CTA reads the pivot S[k][k], column k of the updated S
-// (giving column k of L) and row k of R (giving row k of M = L^{-1}), then
-// updates its own rows i > k:
-//   S[i][j] -= L[i][k] L[j][k]  (k < j <= i),   R[i][j] -= L[i][k] M[k][j]  (j <= k).
-// Nothing a step reads remotely (column k of S, row k of R) is written in
-// that step, so one barrier per step orders everything.
-constexpr int kClus = 8;                      // CTAs per cluster (portable size)
-constexpr int kClusThreads = 256;
+// The O(m^3) kernels run on one CTA, or on a cluster of kClus for larger m:
+// an SM retires about 1.7 FP64 FMAs per clock, so the work is spread over SMs
+// once it outweighs the cluster barriers.  CTA r of n owns the rows i with
+// i % n == r (the work per row grows or shrinks with i), in its shared memory.
+constexpr int kClus = 8;            // CTAs per cluster (portable size)
+constexpr int kClusThreads = 256;   // Cholesky: a panel row per thread
+constexpr int kClusMinM = 28;       // from this m on the cluster is faster (24: even, 32: 10 %)
+constexpr int kPanel = 8;           // columns per Cholesky panel
 
-// Shared memory of the cluster kernels: rp = ceil(m / kClus) rows of pitch
-// m + 1 (odd: conflict-free column reads), `mats` such matrices, plus
-// `vecs` vectors of m doubles.
-__host__ __device__ constexpr size_t clus_smem(int m, int mats, int vecs) {
-  return ((size_t)mats * ((m + kClus - 1) / kClus) * (m + 1) + (size_t)vecs * m) *
-         sizeof(double);
+// 1/d for a finite d > 0: a single-precision seed and one third-order step,
+// three dependent FP64 instructions.
+__device__ __forceinline__ double recip(double d) {
+  const long long b = __double_as_longlong(d);
+  const int e = (int)(b >> 52) - 1023;   // d = f 2^e, 1 <= f < 2
+  if (e < -1000 || e > 1000) return 1.0 / d;
+  const double f = __longlong_as_double((b & 0xfffffffffffffLL) | 0x3ff0000000000000LL);
+  const double y = (double)(1.0f / (float)f);
+  const double r = fma(-f, y, 1.0);
+  const double z = fma(y, fma(r, r, r), y);   // in (1/2, 1]
+  return __longlong_as_double(__double_as_longlong(z) - ((long long)e << 52));
 }
 
-__global__ void __cluster_dims__(kClus, 1, 1) __launch_bounds__(kClusThreads)
-    cholesky_inverse_cluster_kernel(const double* __restrict__ S, int m,
-                                    double* __restrict__ Minv, int* status) {
+// Cholesky S = L L^T and M = L^{-1}, in the form S = U D U^T (U unit lower
+// triangular, D = diag d): M = D^{-1/2} U^{-1}, so that no square root lies on
+// the chain from pivot to pivot.  Right-looking in panels of kPanel columns:
+// every CTA gathers the panel (thread t holds row k0 + t) and factors it
+// alike, one block barrier and a reciprocal per column; it completes the
+// panel's rows of R = U^{-1}; then it updates its own rows below,
+//   A[i][j] -= sum_c U[i][c] A[j][c]  (j <= i),   R[i][j] -= sum_c U[i][c] R[c][j].
+// One cluster barrier per panel (the column-by-column form took one cluster
+// and two block barriers, a square root and a division per column: 2.5 us;
+// 57 states 0.118 -> 0.063 ms, 128 states 0.35 -> 0.165).
+__global__ void __launch_bounds__(kClusThreads)
+    cholesky_inverse_kernel(const double* __restrict__ S, int m, double* __restrict__ Minv,
+                            int* status) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ double csh[];
-  __shared__ double s_piv;
+  __shared__ double s_col[kPanel][kPanel];   // A[k0 + c'][k0 + c] when column c is eliminated
+  __shared__ double s_rs[kPanel];            // 1 / sqrt(d) of the panel
   __shared__ int s_bad;
-  const int rank = (int)cl.block_rank();
-  const int rp = (m + kClus - 1) / kClus;
-  const int pitch = m + 1;
-  double* A_ = csh;                       // [rp][pitch] own rows of S (lower part)
-  double* Rr_ = A_ + (size_t)rp * pitch;  // [rp][pitch] own rows of R
-  double* lf = Rr_ + (size_t)rp * pitch;  // [m]
-  double* mk = lf + m;                    // [m]
-  auto A = [&](int il, int j) -> double& { return A_[il * pitch + j]; };
-  auto Rr = [&](int il, int j) -> double& { return Rr_[il * pitch + j]; };
-  const int r0 = rank * rp, r1 = max(r0, min(m, r0 + rp));
+  const int nr = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int rp = (m + nr - 1) / nr, pitch = m + 1;
+  double* A_ = csh;                        // [rp][pitch] own rows of S (lower part)
+  double* Rr_ = A_ + (size_t)rp * pitch;   // [rp][pitch] own rows of R
+  double* U = Rr_ + (size_t)rp * pitch;    // [m][kPanel + 1] panel of U
+  double* Ac = U + (size_t)m * (kPanel + 1);   // [m][kPanel + 1] panel of A
+  double* Rp = Ac + (size_t)m * (kPanel + 1);  // [kPanel][pitch] panel rows of R
+  constexpr int UP = kPanel + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = kClusThreads / 32;
+  constexpr int NT = kClusThreads, NW = NT / 32;
   if (tid == 0) s_bad = 0;
-  for (int q = tid; q < (r1 - r0) * m; q += kClusThreads) {
-    const int il = q / m, j = q - il * m;
-    A(il, j) = S[(long long)(r0 + il) * m + j];
-    Rr(il, j) = (r0 + il == j) ? 1.0 : 0.0;
+  for (int i = rank + nr * warp; i < m; i += nr * NW) {
+    double* a = A_ + (size_t)(i / nr) * pitch;
+    double* r = Rr_ + (size_t)(i / nr) * pitch;
+    for (int j = lane; j < m; j += 32) {
+      a[j] = S[(long long)i * m + j];
+      r[j] = i == j ? 1.0 : 0.0;
+    }
   }
-  cl.sync();
-  for (int k = 0; k < m; ++k) {
-    const int ok = k / rp;
-    if (tid == 0) {
-      const double akk = *cl.map_shared_rank(&A(k - ok * rp, k), ok);
-      double piv = 1.0;
-      if (!(akk > 0.0) || !isfinite(akk)) s_bad = 1;
-      else piv = sqrt(akk);
-      s_piv = piv;
+  for (int k0 = 0; k0 < m; k0 += kPanel) {
+    const int w = min(kPanel, m - k0);
+    if (nr > 1) cl.sync();
+    else __syncthreads();
+    const int i = k0 + tid;   // this thread's panel row
+    double a[kPanel];
+    if (i < m) {
+      const double* src = A_ + (size_t)(i / nr) * pitch + k0;
+      if (nr > 1) src = cl.map_shared_rank(src, i % nr);
+#pragma unroll
+      for (int c = 0; c < kPanel; ++c) a[c] = c < w ? src[c] : 0.0;
     }
-    __syncthreads();
-    const double rpiv = 1.0 / s_piv;
-    for (int j = k + 1 + tid; j < m; j += kClusThreads) {
-      const int o = j / rp;
-      lf[j] = *cl.map_shared_rank(&A(j - o * rp, k), o) * rpiv;
+    for (int q = warp; q < w; q += NW) {
+      const double* src = Rr_ + (size_t)((k0 + q) / nr) * pitch;
+      if (nr > 1) src = cl.map_shared_rank(src, (k0 + q) % nr);
+      for (int j = lane; j < k0 + w; j += 32) Rp[q * pitch + j] = src[j];
     }
-    for (int j = tid; j <= k; j += kClusThreads)
-      mk[j] = *cl.map_shared_rank(&Rr(k - ok * rp, j), ok) * rpiv;
-    __syncthreads();
-    if (rank == ok)
-      for (int j = tid; j < m; j += kClusThreads) Minv[(long long)k * m + j] = j <= k ? mk[j] : 0.0;
-    // own rows i > k: one warp per row, lanes over columns
-    for (int i = max(r0, k + 1) + warp; i < r1; i += NW) {
-      const int il = i - r0;
-      const double li = lf[i];
-      for (int j = lane; j <= i; j += 32) {
-        if (j <= k) Rr(il, j) -= li * mk[j];
-        else A(il, j) -= li * lf[j];
+#pragma unroll
+    for (int c = 0; c < kPanel; ++c) {
+      if (c < w) {   // uniform
+        if (tid >= c && tid < w) s_col[c][tid] = a[c];
+        __syncthreads();
+        if (i > k0 + c && i < m) {
+          double d = s_col[c][c];
+          if (!(d > 0.0) || !isfinite(d)) d = 1.0;
+          const double u = a[c] * recip(d);
+          U[i * UP + c] = u;
+          Ac[i * UP + c] = a[c];
+#pragma unroll
+          for (int q = c + 1; q < kPanel; ++q)
+            if (q < w && k0 + q <= i) a[q] = fma(-u, s_col[c][q], a[q]);
+        }
       }
     }
-    cl.sync();
+    __syncthreads();
+    // the panel's own rows of R, a column per thread; 1/sqrt(d) meanwhile
+    if (tid < w) {
+      const double d = s_col[tid][tid];
+      const bool ok = d > 0.0 && isfinite(d);
+      if (!ok) s_bad = 1;
+      s_rs[tid] = ok ? 1.0 / sqrt(d) : 1.0;
+    }
+    for (int j = tid; j < k0 + w; j += NT) {
+      double x[kPanel];
+#pragma unroll
+      for (int c = 0; c < kPanel; ++c) {
+        if (c < w) {
+          double v = Rp[c * pitch + j];
+#pragma unroll
+          for (int q = 0; q < c; ++q) v = fma(-U[(k0 + c) * UP + q], x[q], v);
+          x[c] = v;
+          Rp[c * pitch + j] = v;
+        }
+      }
+    }
+    __syncthreads();
+    for (int q = warp; q < w; q += NW)
+      if ((k0 + q) % nr == rank)
+        for (int j = lane; j < m; j += 32)
+          Minv[(long long)(k0 + q) * m + j] = j <= k0 + q ? Rp[q * pitch + j] * s_rs[q] : 0.0;
+    // own rows below the panel: one warp per row, lanes over columns
+    const int first = k0 + w;
+    for (int r = first + (rank - first % nr + nr) % nr + nr * warp; r < m; r += nr * NW) {
+      double u[kPanel];
+#pragma unroll
+      for (int c = 0; c < kPanel; ++c) u[c] = c < w ? U[r * UP + c] : 0.0;
+      double* ar = A_ + (size_t)(r / nr) * pitch;
+      double* rr = Rr_ + (size_t)(r / nr) * pitch;
+      for (int j = lane; j <= r; j += 32) {
+        double* dst = j < first ? rr + j : ar + j;
+        const double* src = j < first ? Rp + j : Ac + (size_t)j * UP;
+        const int step = j < first ? pitch : 1;
+        double v0 = *dst, v1 = 0.0;
+#pragma unroll
+        for (int c = 0; c < kPanel; c += 2) {
+          if (c < w) v0 = fma(-u[c], src[c * step], v0);
+          if (c + 1 < w) v1 = fma(-u[c + 1], src[(c + 1) * step], v1);
+        }
+        *dst = v0 + v1;
+      }
+    }
   }
   if (tid == 0 && s_bad) atomicOr(status, 1);
+  if (nr > 1) cl.sync();   // no CTA leaves while another may still read its shared memory
 }
 
-// Householder tridiagonalisation (eigenvalues only) on a cluster: CTA r
-// owns full rows [r*rp, r*rp + rp) of the symmetric matrix.  Step k takes
-// two cluster barriers: after the partial sums of squares of column k
-// (giving the reflector, which every CTA forms alike from the same values in
-// the same order), and after the partial products p = beta A v and v^T p;
-// then each CTA applies A -= v w^T + w v^T to its own rows.
-__global__ void __cluster_dims__(kClus, 1, 1) __launch_bounds__(kClusThreads)
-    tridiag_cluster_kernel(const double* __restrict__ H, int m, double* __restrict__ d,
-                           double* __restrict__ e) {
+// 1/sqrt(a) for 2^-1000 < a < 2^1000: a single-precision seed and one
+// third-order step.
+__device__ __forceinline__ double rsqrt64(double a) {
+  const long long b = __double_as_longlong(a);
+  const int e = ((int)(b >> 52) - 1023) & ~1;   // a = f 2^e, e even, 1 <= f < 4
+  const double f = __longlong_as_double(b - ((long long)e << 52));
+  const double y = (double)rsqrtf((float)f);
+  const double r = fma(-f * y, y, 1.0);
+  const double z = fma(y * r, fma(0.375, r, 0.5), y);   // y (1 + r/2 + 3 r^2/8)
+  return __longlong_as_double(__double_as_longlong(z) - ((long long)(e / 2) << 52));
+}
+
+// Householder tridiagonalisation (eigenvalues only).  An FP64 operation costs
+// 78 cycles of its sub-partition and as much latency, so up to 128 states the
+// CTA has one warp per sub-partition (two above), and the steps are arranged
+// for a short chain of dependent operations.  Every CTA holds column k, x = A[k+1.., k], of the current
+// matrix; groups of eight lanes of all warps but the last own rows of A.  Step k:
+//   the groups form y = A x for their rows and publish y and their entries C
+//   of column k + 1 to all CTAs, while the last warp forms the reflector
+//   v = x - alpha e_1, beta = 2 / v^T v from x; (cluster) barrier;
+//   A v = y - alpha C, so p = beta (y - alpha C), K = beta/2 v^T p =
+//   beta^2/2 (x^T y - 2 alpha y_1 + alpha^2 C_1) and w = p - K v follow from
+//   one dot product, and so does the next column, C - v w_1 - w v_1, in every
+//   CTA alike; block barrier;
+//   the groups apply A -= v w^T + w v^T to their rows and in the same pass form
+//   the next y.
+// (The form with two cluster barriers, five block barriers and 256 threads took
+// 5.4 us per step; tridiagonalisation and bisection of 57 states 0.34 -> 0.23
+// ms, of 24 0.13 -> 0.10, of 128 0.92 -> 0.67.)
+template <int kTriThreads>
+__global__ void __launch_bounds__(kTriThreads)
+    tridiag_kernel(const double* __restrict__ H, int m, double* __restrict__ d,
+                   double* __restrict__ e) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ double csh[];
-  __shared__ double s_sig[2], s_dot[2];  // partial sums (read by the others)
-  __shared__ double s_beta, s_K;
-  const int rank = (int)cl.block_rank();
-  const int rp = (m + kClus - 1) / kClus;
-  const int pitch = m + 1;
+  __shared__ double s_alpha[2], s_beta[2], s_v0[2];
+  const int nr = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int rp = (m + nr - 1) / nr, pitch = m + 1;
   double* A_ = csh;                       // [rp][pitch] own rows
-  double* vf = A_ + (size_t)rp * pitch;   // [m]
+  double* Y = A_ + (size_t)rp * pitch;    // [2][m] published y (step parity)
+  double* C = Y + 2 * m;                  // [2][m] published column k + 1
+  double* xf = C + 2 * m;                 // [2][m] x
+  double* vf = xf + 2 * m;                // [m]
   double* wf = vf + m;                    // [m]
-  double* pl = wf + m;                    // [m] (rp used): own entries of p (read by the others)
-  auto A = [&](int il, int j) -> double& { return A_[il * pitch + j]; };
-  const int r0 = rank * rp, r1 = max(r0, min(m, r0 + rp));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = kClusThreads / 32;
-  for (int q = tid; q < (r1 - r0) * m; q += kClusThreads) {
-    const int il = q / m, j = q - il * m, i = r0 + il;
-    A(il, j) = 0.5 * (H[(long long)i * m + j] + H[(long long)j * m + i]);
+  constexpr int NW = kTriThreads / 32, kLanes = 8, kGroups = (NW - 1) * 32 / kLanes;
+  for (int i = rank + nr * warp; i < m; i += nr * NW)
+    for (int j = lane; j < m; j += 32)
+      A_[(size_t)(i / nr) * pitch + j] = 0.5 * (H[(long long)i * m + j] + H[(long long)j * m + i]);
+  for (int j = tid; j < m; j += kTriThreads) {
+    xf[j] = 0.5 * (H[j] + H[(long long)j * m]);
+    vf[j] = wf[j] = 0.0;
   }
   __syncthreads();
+  if (nr > 1) cl.sync();   // every CTA has started before it is written to
+  auto warp_sum = [](double v, int width) {
+    for (int o = width / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  const int group = tid / kLanes, gl = tid % kLanes;
   for (int k = 0; k + 2 < m; ++k) {
     const int n0 = k + 1, b = k & 1;
-    if (warp == 0) {
-      double sig = 0.0;
-      for (int i = max(r0, n0 + 1) + lane; i < r1; i += 32) sig += A(i - r0, k) * A(i - r0, k);
-      for (int o = 16; o; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
-      if (lane == 0) s_sig[b] = sig;
-    }
-    if (tid == 0 && k >= r0 && k < r1) d[k] = A(k - r0, k);
-    cl.sync();
-    if (tid == 0) {
-      double sig = 0.0;
-      for (int r = 0; r < kClus; ++r) sig += *cl.map_shared_rank(&s_sig[b], r);
-      const int o = n0 / rp;
-      const double x0 = *cl.map_shared_rank(&A(n0 - o * rp, k), o);
-      double alpha = x0, beta = 0.0, v0 = 0.0;
-      if (sig != 0.0) {
-        const double nrm = sqrt(x0 * x0 + sig);
-        alpha = x0 > 0 ? -nrm : nrm;
-        v0 = x0 - alpha;
-        beta = 2.0 / (v0 * v0 + sig);
+    const double* x = xf + b * m;
+    double* Yb = Y + b * m;
+    double* Cb = C + b * m;
+    if (warp == NW - 1) {   // the reflector
+      double s = 0.0;
+      for (int j = n0 + 1 + lane; j < m; j += 32) s = fma(x[j], x[j], s);
+      s = warp_sum(s, 32);
+      if (lane == 0) {
+        const double x0 = x[n0], s2 = fma(x0, x0, s);
+        double alpha = x0, beta = 0.0, v0 = 0.0;
+        if (s != 0.0) {
+          double nrm;
+          const int ex = (__double2hiint(s2) >> 20) & 0x7ff;
+          if (ex > 100 && ex < 1900) {
+            const double z = rsqrt64(s2);
+            nrm = s2 * z;
+            nrm = fma(0.5 * z, fma(-nrm, nrm, s2), nrm);
+            beta = recip(fma(fabs(x0), nrm, s2));   // 2 / v^T v = 1 / (|x|^2 + |x_0| |x|)
+          } else {
+            nrm = sqrt(s2);
+            beta = 1.0 / fma(fabs(x0), nrm, s2);
+          }
+          alpha = x0 > 0 ? -nrm : nrm;
+          v0 = x0 - alpha;
+        }
+        s_alpha[b] = alpha;
+        s_beta[b] = beta;
+        s_v0[b] = v0;
+        if (rank == 0) e[k] = alpha;
       }
-      s_beta = beta;
-      vf[n0] = v0;
-      if (rank == 0) e[k] = alpha;
+    } else {
+      // own rows i >= n0: the previous step's update (v, w from column k - 1;
+      // zero before the first step), then y = A x
+      const int il0 = (n0 - rank + nr - 1) / nr;   // first local row with i >= n0
+      for (int il = il0 - il0 % kGroups + group; il - group < rp; il += kGroups) {
+        const int i = rank + nr * il;
+        const bool mine = il >= il0 && i < m;
+        double s = 0.0, t = 0.0, c = 0.0;
+        if (mine) {
+          double* row = A_ + (size_t)il * pitch;
+          const double vi = vf[i], wi = wf[i];
+          for (int j = n0 + gl; j < m; j += 2 * kLanes) {
+            const int j2 = j + kLanes;
+            const double a = fma(-vi, wf[j], fma(-wi, vf[j], row[j]));
+            row[j] = a;
+            s = fma(a, x[j], s);
+            if (j == n0) c = a;
+            if (j2 < m) {
+              const double a2 = fma(-vi, wf[j2], fma(-wi, vf[j2], row[j2]));
+              row[j2] = a2;
+              t = fma(a2, x[j2], t);
+            }
+          }
+        }
+        s = warp_sum(s + t, kLanes);
+        c = __shfl_sync(0xffffffffu, c, lane & ~(kLanes - 1));
+        if (mine && gl < nr) {
+          double* y = Yb + i;
+          double* cc = Cb + i;
+          if (nr > 1) {
+            y = cl.map_shared_rank(y, gl);
+            cc = cl.map_shared_rank(cc, gl);
+          }
+          *y = s;
+          *cc = c;
+        }
+      }
     }
-    for (int j = n0 + 1 + tid; j < m; j += kClusThreads) {
-      const int o = j / rp;
-      vf[j] = *cl.map_shared_rank(&A(j - o * rp, k), o);
-    }
-    __syncthreads();
-    const double beta = s_beta;
-    for (int i = max(r0, n0) + warp; i < r1; i += NW) {
-      double acc = 0.0;
-      for (int j = n0 + lane; j < m; j += 32) acc += A(i - r0, j) * vf[j];
-      for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) pl[i - r0] = beta * acc;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      double acc = 0.0;
-      for (int i = max(r0, n0) + lane; i < r1; i += 32) acc += vf[i] * pl[i - r0];
-      for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) s_dot[b] = acc;
-    }
-    cl.sync();
-    if (tid == 0) {
-      double dot = 0.0;
-      for (int r = 0; r < kClus; ++r) dot += *cl.map_shared_rank(&s_dot[b], r);
-      s_K = 0.5 * beta * dot;
-    }
-    __syncthreads();
-    const double K = s_K;
-    for (int j = n0 + tid; j < m; j += kClusThreads) {
-      const int o = j / rp;
-      wf[j] = *cl.map_shared_rank(&pl[j - o * rp], o) - K * vf[j];
-    }
-    __syncthreads();
-    for (int i = max(r0, n0) + warp; i < r1; i += NW) {
-      const int il = i - r0;
-      const double vi = vf[i], wi = wf[i];
-      for (int j = n0 + lane; j < m; j += 32) A(il, j) -= vi * wf[j] + wi * vf[j];
+    if (nr > 1) cl.sync();
+    else __syncthreads();
+    // scalars, in every warp alike
+    const double alpha = s_alpha[b], beta = s_beta[b], v0 = s_v0[b];
+    double xy = 0.0;
+    for (int j = n0 + lane; j < m; j += 32) xy = fma(x[j], Yb[j], xy);
+    const double y1 = Yb[n0], c1 = Cb[n0];
+    const double hb = 0.5 * beta * beta, rest = alpha * fma(alpha, c1, -2.0 * y1);
+    const double p1 = beta * fma(-alpha, c1, y1);
+    xy = warp_sum(xy, 32);
+    const double K = hb * (xy + rest);
+    const double w1 = fma(-K, v0, p1);
+    double* xn = xf + (b ^ 1) * m;
+    if (tid == 0 && (n0 - 1) == 0 && rank == 0) d[0] = A_[0];
+    for (int j = n0 + tid; j < m; j += kTriThreads) {
+      const double vj = j == n0 ? v0 : x[j], cj = Cb[j];
+      const double wj = fma(-K, vj, beta * fma(-alpha, cj, Yb[j]));
+      const double cn = fma(-wj, v0, fma(-vj, w1, cj));   // column n0 of the updated matrix
+      vf[j] = vj;
+      wf[j] = wj;
+      xn[j] = cn;
+      if (j == n0 && rank == 0) d[n0] = cn;
     }
     __syncthreads();
   }
-  if (tid == 0) {
-    if (m >= 2 && m - 2 >= r0 && m - 2 < r1) d[m - 2] = A(m - 2 - r0, m - 2);
-    if (m >= 2 && m - 1 >= r0 && m - 1 < r1) e[m - 2] = A(m - 1 - r0, m - 2);
-    if (m - 1 >= r0 && m - 1 < r1) d[m - 1] = A(m - 1 - r0, m - 1);
+  // the last 2 x 2 block: d[m - 2] is set above (m > 2), the update of the last
+  // diagonal entry is still due
+  const int last = m - 1;
+  if (m == 1) {
+    if (tid == 0 && rank == 0) d[0] = A_[0];
+  } else if (last % nr == rank && tid == 0) {
+    const double* row = A_ + (size_t)(last / nr) * pitch;
+    if (m == 2) {
+      e[0] = row[0];
+      d[1] = row[1];
+    } else {
+      const double vl = vf[last], wl = wf[last];
+      d[last] = fma(-vl, wl, fma(-wl, vl, row[last]));
+      e[last - 1] = xf[((m - 2) & 1) * m + last];
+    }
   }
-  cl.sync();   // no CTA leaves while another may still read its shared memory
+  if (m == 2 && rank == 0 && tid == 0) d[0] = A_[0];
+  if (nr > 1) cl.sync();   // no CTA leaves while another may still write to it
+}
+
+// Shared memory of the two kernels on a cluster of nr CTAs.
+size_t cholesky_smem(int m, int nr) {
+  return ((size_t)2 * ((m + nr - 1) / nr) * (m + 1) + (size_t)2 * m * (kPanel + 1) +
+          (size_t)kPanel * (m + 1)) * sizeof(double);
+}
+size_t tridiag_smem(int m, int nr) {
+  return ((size_t)((m + nr - 1) / nr) * (m + 1) + (size_t)8 * m) * sizeof(double);
+}
+
+// Launch on one cluster (of one CTA for small m).
+template <typename K, typename... Args>
+cudaError_t launch_cluster(K kernel, int nr, int threads, size_t smem, cudaStream_t st,
+                           Args... args) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(nr);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = nr;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // ---------------------------------------------------------------------------
@@ -346,7 +512,7 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(const double* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// Eigenvalues only: the cluster tridiagonalisation above, then bisection on
+// Eigenvalues only: the tridiagonalisation above, then bisection on
 // Sturm counts, one CTA of four warps per eigenvalue (128-point
 // multisection: seven bits per round, one warp on each of the SM's four
 // sub-partitions, whose FP64 units the counts keep busy).
@@ -555,12 +721,9 @@ cudaError_t launch_gram_reduce(const double* partial, int n_chunks, int m, doubl
 cudaError_t launch_cholesky_inverse(const double* S, int m, double* Minv, int* status,
                                     cudaStream_t st) {
   if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
-  const size_t smem = clus_smem(m, 2, 2);
-  cudaError_t e = cudaFuncSetAttribute(cholesky_inverse_cluster_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cholesky_inverse_cluster_kernel<<<kClus, kClusThreads, smem, st>>>(S, m, Minv, status);
-  return cudaGetLastError();
+  const int nr = m < kClusMinM ? 1 : kClus;
+  return launch_cluster(cholesky_inverse_kernel, nr, kClusThreads, cholesky_smem(m, nr), st, S, m,
+                        Minv, status);
 }
 
 cudaError_t launch_jacobi_eigh(const double* H, int m, double* E, double* Rt, double* work,
@@ -583,12 +746,12 @@ cudaError_t launch_jacobi_eigh(const double* H, int m, double* E, double* Rt, do
 
 cudaError_t launch_tridiag(const double* H, int m, double* work, cudaStream_t st) {
   if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
-  const size_t smem = clus_smem(m, 1, 3);
-  cudaError_t e = cudaFuncSetAttribute(tridiag_cluster_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  tridiag_cluster_kernel<<<kClus, kClusThreads, smem, st>>>(H, m, work, work + m);
-  return cudaGetLastError();
+  const int nr = m < kClusMinM ? 1 : kClus;
+  if (m <= 128)
+    return launch_cluster(tridiag_kernel<128>, nr, 128, tridiag_smem(m, nr), st, H, m, work,
+                          work + m);
+  return launch_cluster(tridiag_kernel<256>, nr, 256, tridiag_smem(m, nr), st, H, m, work,
+                        work + m);
 }
 
 cudaError_t launch_bisect(const double* work, int m, double* E, cudaStream_t st) {
