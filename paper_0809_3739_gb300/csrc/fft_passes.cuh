@@ -40,7 +40,8 @@ namespace cg = cooperative_groups;
 namespace itp {
 
 template <int NX, int NY>
-cudaError_t plane64_dispatch(const GridDesc& g, int mode, const PlaneArgs<double>& a,
+cudaError_t plane64_dispatch(const GridDesc& g, int mode,
+                             const TermPack<PlaneArgs<double>>& p,
                              const PlaneArgs<double>* args, const int2* rows, int nrows,
                              size_t smem, cudaStream_t st);
 
@@ -993,22 +994,24 @@ template <typename R, int NX, int NY, int MODE>
 __global__ void __launch_bounds__(launch_threads(kThreads),
                                   min_blocks(plane_smem_ct(NX, NY, sizeof(R)),
                                              sizeof(R) == 4 ? 3 : 2))
-    plane_kernel(const GridDesc g, const PlaneArgs<R> a) {
-  plane_body<R, NX, NY, MODE>(g, a, blockIdx.x, blockIdx.y);
+    plane_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<R>> p) {
+  const int t = blockIdx.y / p.a[0].m;   // term
+  plane_body<R, NX, NY, MODE>(g, p.a[t], blockIdx.x, blockIdx.y - t * p.a[0].m);
 }
 
 // Grouped plane pass: one launch over the states of several problems with
 // the same grid (a batch of independent problems).  CTA row y of the grid
 // is state rows[y].y of problem rows[y].x, whose arguments are args[rows[y].x].
-// (FP64: one kernel for both forms, to halve the compile time; rows null: the
-// arguments are `a`.)
+// (FP64: one kernel for both forms, to halve the compile time; rows null: CTA
+// row y is a state of one of the terms p.)
 template <int NX, int NY, int MODE>
 __global__ void __launch_bounds__(launch_threads(plane64_threads(NX)),
                                   min_blocks(plane_smem_ct(NX, NY, 8), 2))
-    plane64_kernel(const GridDesc g, const PlaneArgs<double> a,
+    plane64_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<double>> p,
                    const PlaneArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
-  const int2 r = rows ? rows[blockIdx.y] : make_int2(0, (int)blockIdx.y);
-  const PlaneArgs<double> la = rows ? args[r.x] : a;
+  const int t = rows ? 0 : blockIdx.y / p.a[0].m;
+  const int2 r = rows ? rows[blockIdx.y] : make_int2(t, (int)blockIdx.y - t * p.a[0].m);
+  const PlaneArgs<double> la = rows ? args[r.x] : p.a[t];
   plane_body<double, NX, NY, MODE>(g, la, blockIdx.x, r.y);
 }
 
@@ -1396,7 +1399,9 @@ struct RowGeo : PlaneGeo<R, NX, 2 * TB, kThreads> {
 
 template <typename R, int NX, int TB, int MODE>
 __global__ void __launch_bounds__(kThreads)
-    rowpass_kernel(const GridDesc g, const PlaneArgs<R> a) {
+    rowpass_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<R>> p) {
+  const int term = blockIdx.y / p.a[0].m;
+  const PlaneArgs<R>& a = p.a[term];
   using C = typename SpecOf<R>::type;
   using CR = typename CplxOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1405,7 +1410,8 @@ __global__ void __launch_bounds__(kThreads)
   C* twx = sm + TB * G.pp;
   for (int i = threadIdx.x; i < G.nx; i += blockDim.x) twx[i] = static_cast<const C*>(a.twx)[i];
   const int nb = (g.ny / 2) / TB;   // TB divides ny / 2
-  const int z = blockIdx.x / nb, blk = blockIdx.x - z * nb, s = blockIdx.y;
+  const int z = blockIdx.x / nb, blk = blockIdx.x - z * nb,
+            s = blockIdx.y - term * p.a[0].m;
   const int t0 = blk * TB;
   const long long plane_pts = (long long)G.nx * g.ny;
   const long long real_off = (long long)s * g.n_points + (long long)z * plane_pts;
@@ -1508,8 +1514,7 @@ __device__ __forceinline__ void col_invB_load_r(nt_tag<NT>, C* sm, const C* __re
 
 template <typename R, int NY, int W, int DIR>
 __global__ void __launch_bounds__(launch_threads(task_threads(W)))
-    colpass_kernel(const GridDesc g, void* spec, const void* twy_g, int pw_rt,
-                   const KinFac<R> kin) {
+    colpass_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<R>> p, int pw_rt) {
   constexpr int NT = task_threads(W);
   using C = typename SpecOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1518,18 +1523,20 @@ __global__ void __launch_bounds__(launch_threads(task_threads(W)))
   const int ny = NY ? NY : g.ny;
   const int pw = W ? W : pw_rt;
   C* twy = sm + ny * pw;
-  for (int i = threadIdx.x; i < ny; i += blockDim.x) twy[i] = static_cast<const C*>(twy_g)[i];
-  const long long plane = blockIdx.y;
+  const int planes = p.a[0].m * g.nz, term = blockIdx.y / planes;
+  const PlaneArgs<R>& a = p.a[term];
+  for (int i = threadIdx.x; i < ny; i += blockDim.x) twy[i] = static_cast<const C*>(a.twy)[i];
+  const long long plane = blockIdx.y - term * planes;
   const int kx0 = blockIdx.x * pw;
   const int w = min(pw, g.nxh - kx0);
-  C* base = static_cast<C*>(spec) + plane * (long long)ny * g.nxh + kx0;
+  C* base = static_cast<C*>(a.spec) + plane * (long long)ny * g.nxh + kx0;
   __syncthreads();
   if constexpr (DIR < 0) {
     ITP_WITH_RADIX(ay.r2, (outlined<C, NY>), pencil_fwdA_r, nt_tag<NT>(), sm, base, twy, (long long)g.nxh, w, pw,
                    ay.r1)
     __syncthreads();
     ITP_WITH_RADIX(ay.r1, (outlined<C, NY>), col_fwdB_store_r, nt_tag<NT>(), sm, base, (long long)g.nxh, w, pw,
-                   ay.r2, kin, kx0)
+                   ay.r2, a.kin, kx0)
   } else {
     ITP_WITH_RADIX(ay.r1, (outlined<C, NY>), col_invB_load_r, nt_tag<NT>(), sm, base, twy, (long long)g.nxh, w, pw,
                    ay.r2)
@@ -1572,18 +1579,20 @@ template <typename R, int NZ, int W, int MODE>
 __global__ void __launch_bounds__(launch_threads(task_threads(W)),
                                   min_blocks(pencil_smem_ct(NZ, W, sizeof(R)),
                                              pencil_min_ctas(NZ, sizeof(R))))
-    pencil_kernel(const GridDesc g, const PencilArgs<R> a) {
-  pencil_body<R, NZ, W, MODE>(g, a, blockIdx.x, blockIdx.y);
+    pencil_kernel(const GridDesc g, const __grid_constant__ TermPack<PencilArgs<R>> p) {
+  const int t = blockIdx.y / p.a[0].m;   // term
+  pencil_body<R, NZ, W, MODE>(g, p.a[t], blockIdx.x, blockIdx.y - t * p.a[0].m);
 }
 
 // FP64 pencil pass, single or grouped (rows set) launches, either mode.
 template <int NZ, int W>
 __global__ void __launch_bounds__(launch_threads(task_threads(W)),
                                   min_blocks(pencil_smem_ct(NZ, W, 8), pencil_min_ctas(NZ, 8)))
-    pencil64_kernel(const GridDesc g, const PencilArgs<double> a,
+    pencil64_kernel(const GridDesc g, const __grid_constant__ TermPack<PencilArgs<double>> p,
                     const PencilArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
-  const int2 r = rows ? rows[blockIdx.y] : make_int2(0, (int)blockIdx.y);
-  const PencilArgs<double> la = rows ? args[r.x] : a;
+  const int t = rows ? 0 : blockIdx.y / p.a[0].m;
+  const int2 r = rows ? rows[blockIdx.y] : make_int2(t, (int)blockIdx.y - t * p.a[0].m);
+  const PencilArgs<double> la = rows ? args[r.x] : p.a[t];
   pencil_body<double, NZ, W, -1>(g, la, blockIdx.x, r.y);
 }
 
@@ -1695,25 +1704,34 @@ __global__ void transpose_planes_kernel(const TS* __restrict__ src, TD* __restri
   }
 }
 
+template <typename A>
+TermPack<A> pack_terms(const A* a, int n) {
+  TermPack<A> p{};
+  for (int i = 0; i < n; ++i) p.a[i] = a[i];
+  return p;
+}
+
 template <typename K>
 cudaError_t set_smem(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 template <typename R, int NX, int NY>
-cudaError_t plane_dispatch(const GridDesc& g, const PlaneArgs<R>& a, size_t smem, cudaStream_t st) {
+cudaError_t plane_dispatch(const GridDesc& g, const PlaneArgs<R>* a, int n, size_t smem,
+                           cudaStream_t st) {
+  const TermPack<PlaneArgs<R>> p = pack_terms(a, n);
   if constexpr (sizeof(R) == 8) {
-    return plane64_dispatch<NX, NY>(g, a.mode, a, nullptr, nullptr, a.m, smem, st);
+    return plane64_dispatch<NX, NY>(g, a->mode, p, nullptr, nullptr, n * a->m, smem, st);
   } else {
-    dim3 grid(g.nz, a.m);
+    dim3 grid(g.nz, n * a->m);
     const int nthr = kThreads;
     cudaError_t e;
-    switch (a.mode) {
+    switch (a->mode) {
 #define ITP_PLANE_CASE(M)                                                   \
     case M:                                                                 \
       e = set_smem(plane_kernel<R, NX, NY, M>, smem);                       \
       if (e != cudaSuccess) return e;                                       \
-      plane_kernel<R, NX, NY, M><<<grid, nthr, smem, st>>>(g, a);           \
+      plane_kernel<R, NX, NY, M><<<grid, nthr, smem, st>>>(g, p);           \
       break;
       ITP_PLANE_CASE(PLANE_FWD_REAL)
       ITP_PLANE_CASE(PLANE_MERGED)
@@ -1729,24 +1747,25 @@ cudaError_t plane_dispatch(const GridDesc& g, const PlaneArgs<R>& a, size_t smem
 }
 
 template <typename R, int NZ, int W>
-cudaError_t pencil_dispatch(const GridDesc& g, const PencilArgs<R>& a, size_t smem,
+cudaError_t pencil_dispatch(const GridDesc& g, const PencilArgs<R>* a, int n, size_t smem,
                             cudaStream_t st) {
+  const TermPack<PencilArgs<R>> p = pack_terms(a, n);
   const int chunks = (g.nxh + g.pencil_w - 1) / g.pencil_w;
-  dim3 grid(g.ny * chunks, a.m);
+  dim3 grid(g.ny * chunks, n * a->m);
   const int nthr = launch_threads(task_threads(W));
   cudaError_t e;
   if constexpr (sizeof(R) == 8) {
     e = set_smem(pencil64_kernel<NZ, W>, smem);
     if (e != cudaSuccess) return e;
-    pencil64_kernel<NZ, W><<<grid, nthr, smem, st>>>(g, a, nullptr, nullptr);
-  } else if (a.mode == PENCIL_PROPAGATE) {
+    pencil64_kernel<NZ, W><<<grid, nthr, smem, st>>>(g, p, nullptr, nullptr);
+  } else if (a->mode == PENCIL_PROPAGATE) {
     e = set_smem(pencil_kernel<R, NZ, W, PENCIL_PROPAGATE>, smem);
     if (e != cudaSuccess) return e;
-    pencil_kernel<R, NZ, W, PENCIL_PROPAGATE><<<grid, nthr, smem, st>>>(g, a);
+    pencil_kernel<R, NZ, W, PENCIL_PROPAGATE><<<grid, nthr, smem, st>>>(g, p);
   } else {
     e = set_smem(pencil_kernel<R, NZ, W, PENCIL_KINETIC>, smem);
     if (e != cudaSuccess) return e;
-    pencil_kernel<R, NZ, W, PENCIL_KINETIC><<<grid, nthr, smem, st>>>(g, a);
+    pencil_kernel<R, NZ, W, PENCIL_KINETIC><<<grid, nthr, smem, st>>>(g, p);
   }
   return cudaGetLastError();
 }
@@ -1754,10 +1773,11 @@ cudaError_t pencil_dispatch(const GridDesc& g, const PencilArgs<R>& a, size_t sm
 }  // namespace
 
 // The FP64 plane passes of one plane size, instantiated by translation units
-// of their own: over the a.m states of `a`, or nrows rows of a table (no
-// PLANE_TERM: FP64 terms are accumulated).
+// of their own: over the states of the terms `p`, or the rows of a table (nrows
+// in all; no PLANE_TERM: FP64 terms are accumulated).
 template <int NX, int NY>
-cudaError_t plane64_dispatch(const GridDesc& g, int mode, const PlaneArgs<double>& a,
+cudaError_t plane64_dispatch(const GridDesc& g, int mode,
+                             const TermPack<PlaneArgs<double>>& p,
                              const PlaneArgs<double>* args, const int2* rows, int nrows,
                              size_t smem, cudaStream_t st) {
   dim3 grid(g.nz, nrows);
@@ -1768,7 +1788,7 @@ cudaError_t plane64_dispatch(const GridDesc& g, int mode, const PlaneArgs<double
     e = set_smem(plane64_kernel<NX, NY, M>, smem);                              \
     if (e != cudaSuccess) return e;                                             \
     plane64_kernel<NX, NY, M>                                                   \
-        <<<grid, launch_threads(plane64_threads(NX)), smem, st>>>(g, a, args, rows); \
+        <<<grid, launch_threads(plane64_threads(NX)), smem, st>>>(g, p, args, rows); \
     break;
     ITP_PLANE64_CASE(PLANE_FWD_REAL)
     ITP_PLANE64_CASE(PLANE_MERGED)
@@ -1781,25 +1801,26 @@ cudaError_t plane64_dispatch(const GridDesc& g, int mode, const PlaneArgs<double
   return cudaGetLastError();
 }
 #ifndef ITP_PLANE64_UNIT   // units that instantiate a size define this
-extern template cudaError_t plane64_dispatch<0, 0>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
-extern template cudaError_t plane64_dispatch<32, 32>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
-extern template cudaError_t plane64_dispatch<48, 48>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
-extern template cudaError_t plane64_dispatch<64, 64>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
-extern template cudaError_t plane64_dispatch<96, 96>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
-extern template cudaError_t plane64_dispatch<128, 128>(const GridDesc&, int, const PlaneArgs<double>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<0, 0>(const GridDesc&, int, const TermPack<PlaneArgs<double>>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<32, 32>(const GridDesc&, int, const TermPack<PlaneArgs<double>>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<48, 48>(const GridDesc&, int, const TermPack<PlaneArgs<double>>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<64, 64>(const GridDesc&, int, const TermPack<PlaneArgs<double>>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<96, 96>(const GridDesc&, int, const TermPack<PlaneArgs<double>>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
+extern template cudaError_t plane64_dispatch<128, 128>(const GridDesc&, int, const TermPack<PlaneArgs<double>>&, const PlaneArgs<double>*, const int2*, int, size_t, cudaStream_t);
 #endif
 
 template <typename R, int NX, int TB>
-cudaError_t rowpass_dispatch(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_t st) {
+cudaError_t rowpass_dispatch(const GridDesc& g, const PlaneArgs<R>* a, int n, cudaStream_t st) {
+  const TermPack<PlaneArgs<R>> p = pack_terms(a, n);
   const size_t smem = ((size_t)TB * g.pp + g.nx) * 2 * sizeof(R);
-  dim3 grid(g.nz * ((g.ny / 2) / TB), a.m);
+  dim3 grid(g.nz * ((g.ny / 2) / TB), n * a->m);
   cudaError_t e;
-  switch (a.mode) {
+  switch (a->mode) {
 #define ITP_ROW_CASE(M)                                                     \
   case M:                                                                   \
     e = set_smem(rowpass_kernel<R, NX, TB, M>, smem);                       \
     if (e != cudaSuccess) return e;                                         \
-    rowpass_kernel<R, NX, TB, M><<<grid, kThreads, smem, st>>>(g, a);       \
+    rowpass_kernel<R, NX, TB, M><<<grid, kThreads, smem, st>>>(g, p);       \
     break;
     ITP_ROW_CASE(PLANE_FWD_REAL)
     ITP_ROW_CASE(PLANE_MERGED)
@@ -1813,45 +1834,55 @@ cudaError_t rowpass_dispatch(const GridDesc& g, const PlaneArgs<R>& a, cudaStrea
 }
 
 template <typename R>
-cudaError_t rowpass_launch(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_t st) {
+cudaError_t rowpass_launch(const GridDesc& g, const PlaneArgs<R>* a, int n, cudaStream_t st) {
   const int tb = g.row_tb[sizeof(R) == 4 ? 0 : 1];
   if (g.nx == 256 && g.pp == row_pitch(256) && tb == (sizeof(R) == 4 ? 32 : 16)) {
-    if constexpr (sizeof(R) == 4) return rowpass_dispatch<R, 256, 32>(g, a, st);
-    else return rowpass_dispatch<R, 256, 16>(g, a, st);
+    if constexpr (sizeof(R) == 4) return rowpass_dispatch<R, 256, 32>(g, a, n, st);
+    else return rowpass_dispatch<R, 256, 16>(g, a, n, st);
   }
   if constexpr (sizeof(R) == 4)
-    if (tb == 32) return rowpass_dispatch<R, 0, 32>(g, a, st);
-  if (tb == 16) return rowpass_dispatch<R, 0, 16>(g, a, st);
-  if (tb == 8) return rowpass_dispatch<R, 0, 8>(g, a, st);
+    if (tb == 32) return rowpass_dispatch<R, 0, 32>(g, a, n, st);
+  if (tb == 16) return rowpass_dispatch<R, 0, 16>(g, a, n, st);
+  if (tb == 8) return rowpass_dispatch<R, 0, 8>(g, a, n, st);
   return cudaErrorInvalidValue;
 }
 
 template <typename R, int NY, int W, int DIR>
-cudaError_t colpass_one(const GridDesc& g, void* spec, const void* twy, int m,
-                        const KinFac<R>& kin, cudaStream_t st) {
+cudaError_t colpass_one(const GridDesc& g, const PlaneArgs<R>* a, int n, cudaStream_t st) {
   const int cw = g.col_w[sizeof(R) == 4 ? 0 : 1];
   const size_t smem = ((size_t)g.ny * cw + g.ny) * 2 * sizeof(R);
   cudaError_t e = set_smem(colpass_kernel<R, NY, W, DIR>, smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((g.nxh + cw - 1) / cw, (unsigned)((long long)m * g.nz));
-  colpass_kernel<R, NY, W, DIR><<<grid, launch_threads(task_threads(W)), smem, st>>>(
-      g, spec, twy, cw, kin);
+  dim3 grid((g.nxh + cw - 1) / cw, (unsigned)((long long)n * a->m * g.nz));
+  colpass_kernel<R, NY, W, DIR>
+      <<<grid, launch_threads(task_threads(W)), smem, st>>>(g, pack_terms(a, n), cw);
   return cudaGetLastError();
 }
 
 template <typename R, int DIR>
-cudaError_t colpass_launch(const GridDesc& g, void* spec, const void* twy, int m,
-                           const KinFac<R>& kin, cudaStream_t st) {
+cudaError_t colpass_launch(const GridDesc& g, const PlaneArgs<R>* a, int n, cudaStream_t st) {
   if (g.ny == 256 && g.col_w[sizeof(R) == 4 ? 0 : 1] == (sizeof(R) == 4 ? 33 : 17)) {
-    if constexpr (sizeof(R) == 4) return colpass_one<R, 256, 33, DIR>(g, spec, twy, m, kin, st);
-    else return colpass_one<R, 256, 17, DIR>(g, spec, twy, m, kin, st);
+    if constexpr (sizeof(R) == 4) return colpass_one<R, 256, 33, DIR>(g, a, n, st);
+    else return colpass_one<R, 256, 17, DIR>(g, a, n, st);
   }
-  return colpass_one<R, 0, 0, DIR>(g, spec, twy, m, kin, st);
+  return colpass_one<R, 0, 0, DIR>(g, a, n, st);
 }
 
 template <typename R>
-cudaError_t launch_plane(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_t st, int* nlaunch) {
+cudaError_t launch_plane(const GridDesc& g, const PlaneArgs<R>* ap, int n, cudaStream_t st,
+                         int* nlaunch) {
+  if (n < 1 || n > kMaxTermsK) return cudaErrorInvalidValue;
+  const PlaneArgs<R>& a = *ap;
   if (nlaunch) *nlaunch = 1;
+  // cluster planes take one term per launch
+  if (n > 1 && g.split_planes[sizeof(R) == 4 ? 0 : 1] >= 2) {
+    for (int i = 0; i < n; ++i) {
+      const cudaError_t e = launch_plane<R>(g, ap + i, 1, st, nullptr);
+      if (e != cudaSuccess) return e;
+    }
+    if (nlaunch) *nlaunch = n;
+    return cudaSuccess;
+  }
   // FP32 H psi passes write FP32 (potential and output in R)
   if (a.mode == PLANE_HPSI && sizeof(R) == 4 && (!a.V_r || !a.phi_out))
     return cudaErrorInvalidValue;
@@ -1914,63 +1945,64 @@ cudaError_t launch_plane(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_t 
   if (g.split_planes[sizeof(R) == 4 ? 0 : 1]) {
     // planes too large for one CTA: column passes for y, row passes for x
     cudaError_t e = cudaSuccess;
-    int n = 0;
+    int nl = 0;
     if (a.mode != PLANE_FWD_REAL) {
-      e = colpass_launch<R, 1>(g, a.spec, a.twy, a.m, KinFac<R>{}, st);
-      ++n;
+      e = colpass_launch<R, 1>(g, ap, n, st);
+      ++nl;
       if (e != cudaSuccess) return e;
     }
-    e = rowpass_launch<R>(g, a, st);
-    ++n;
+    e = rowpass_launch<R>(g, ap, n, st);
+    ++nl;
     if (e != cudaSuccess) return e;
     if (a.mode == PLANE_FWD_REAL || a.mode == PLANE_MERGED) {
-      e = colpass_launch<R, -1>(g, a.spec, a.twy, a.m, a.kin, st);
-      ++n;
+      e = colpass_launch<R, -1>(g, ap, n, st);
+      ++nl;
     }
-    if (nlaunch) *nlaunch = n;
+    if (nlaunch) *nlaunch = nl;
     return e;
   }
   const size_t smem = plane_smem_bytes(g, sizeof(R));
   if (g.nx == g.ny && g.pp == row_pitch(g.nx)) {
     switch (g.nx) {
-      case 32: return plane_dispatch<R, 32, 32>(g, a, smem, st);
-      case 48: return plane_dispatch<R, 48, 48>(g, a, smem, st);
-      case 64: return plane_dispatch<R, 64, 64>(g, a, smem, st);
-      case 96: return plane_dispatch<R, 96, 96>(g, a, smem, st);
-      case 128: return plane_dispatch<R, 128, 128>(g, a, smem, st);
+      case 32: return plane_dispatch<R, 32, 32>(g, ap, n, smem, st);
+      case 48: return plane_dispatch<R, 48, 48>(g, ap, n, smem, st);
+      case 64: return plane_dispatch<R, 64, 64>(g, ap, n, smem, st);
+      case 96: return plane_dispatch<R, 96, 96>(g, ap, n, smem, st);
+      case 128: return plane_dispatch<R, 128, 128>(g, ap, n, smem, st);
       default: break;
     }
   }
-  return plane_dispatch<R, 0, 0>(g, a, smem, st);
+  return plane_dispatch<R, 0, 0>(g, ap, n, smem, st);
 }
 
 template <typename R>
-cudaError_t launch_pencil(const GridDesc& g, const PencilArgs<R>& a, cudaStream_t st) {
+cudaError_t launch_pencil(const GridDesc& g, const PencilArgs<R>* a, int n, cudaStream_t st) {
+  if (n < 1 || n > kMaxTermsK) return cudaErrorInvalidValue;
   if (g.pencil_w == 0) {
     if constexpr (sizeof(R) == 4) {
-      return launch_pencil_tm(g, a, st);
+      return launch_pencil_tm(g, a, n, st);
     } else {
       // the FP64 passes of a mixed handle: the default slab width
       GridDesc g2 = g;
       const size_t full = (size_t)g.nz * g.nxh * 2 * sizeof(R), budget = 72 * 1024;
       const int chunks = (int)((full + budget - 1) / budget);
       g2.pencil_w = g2.pencil_pitch = (g.nxh + chunks - 1) / chunks;
-      return launch_pencil(g2, a, st);
+      return launch_pencil(g2, a, n, st);
     }
   }
   const size_t smem = pencil_smem_bytes(g, sizeof(R));
   switch (g.nz * 1000 + g.pencil_w) {
-    case 32 * 1000 + 17: return pencil_dispatch<R, 32, 17>(g, a, smem, st);
-    case 48 * 1000 + 25: return pencil_dispatch<R, 48, 25>(g, a, smem, st);
-    case 64 * 1000 + 33: return pencil_dispatch<R, 64, 33>(g, a, smem, st);
-    case 96 * 1000 + 49: return pencil_dispatch<R, 96, 49>(g, a, smem, st);
-    case 96 * 1000 + 25: return pencil_dispatch<R, 96, 25>(g, a, smem, st);
-    case 128 * 1000 + 65: return pencil_dispatch<R, 128, 65>(g, a, smem, st);
-    case 128 * 1000 + 33: return pencil_dispatch<R, 128, 33>(g, a, smem, st);
-    case 256 * 1000 + 33: return pencil_dispatch<R, 256, 33>(g, a, smem, st);
+    case 32 * 1000 + 17: return pencil_dispatch<R, 32, 17>(g, a, n, smem, st);
+    case 48 * 1000 + 25: return pencil_dispatch<R, 48, 25>(g, a, n, smem, st);
+    case 64 * 1000 + 33: return pencil_dispatch<R, 64, 33>(g, a, n, smem, st);
+    case 96 * 1000 + 49: return pencil_dispatch<R, 96, 49>(g, a, n, smem, st);
+    case 96 * 1000 + 25: return pencil_dispatch<R, 96, 25>(g, a, n, smem, st);
+    case 128 * 1000 + 65: return pencil_dispatch<R, 128, 65>(g, a, n, smem, st);
+    case 128 * 1000 + 33: return pencil_dispatch<R, 128, 33>(g, a, n, smem, st);
+    case 256 * 1000 + 33: return pencil_dispatch<R, 256, 33>(g, a, n, smem, st);
     default: break;
   }
-  return pencil_dispatch<R, 0, 0>(g, a, smem, st);
+  return pencil_dispatch<R, 0, 0>(g, a, n, smem, st);
 }
 
 template <typename R>
@@ -2004,7 +2036,8 @@ template <typename R, int NX, int NY>
 cudaError_t plane_group_dispatch(const GridDesc& g, int mode, const PlaneArgs<R>* args,
                                  const int2* rows, int nrows, size_t smem, cudaStream_t st) {
   if constexpr (sizeof(R) == 8) {
-    return plane64_dispatch<NX, NY>(g, mode, PlaneArgs<double>{}, args, rows, nrows, smem, st);
+    return plane64_dispatch<NX, NY>(g, mode, TermPack<PlaneArgs<double>>{}, args, rows, nrows,
+                                    smem, st);
   } else {
     dim3 grid(g.nz, nrows);
     cudaError_t e;
@@ -2056,7 +2089,7 @@ cudaError_t pencil_group_dispatch(const GridDesc& g, int mode, const PencilArgs<
   if constexpr (sizeof(R) == 8) {   // (the mode is in the arguments)
     e = set_smem(pencil64_kernel<NZ, W>, smem);
     if (e != cudaSuccess) return e;
-    pencil64_kernel<NZ, W><<<grid, nthr, smem, st>>>(g, PencilArgs<double>{}, args, rows);
+    pencil64_kernel<NZ, W><<<grid, nthr, smem, st>>>(g, TermPack<PencilArgs<double>>{}, args, rows);
   } else if (mode == PENCIL_PROPAGATE) {
     e = set_smem(pencil_group_kernel<R, NZ, W, PENCIL_PROPAGATE>, smem);
     if (e != cudaSuccess) return e;

@@ -6,6 +6,7 @@
 
 namespace itp {
 
-template cudaError_t launch_pencil<float>(const GridDesc&, const PencilArgs<float>&, cudaStream_t);
+template cudaError_t launch_pencil<float>(const GridDesc&, const PencilArgs<float>*, int,
+                                          cudaStream_t);
 
 }  // namespace itp

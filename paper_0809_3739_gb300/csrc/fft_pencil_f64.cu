@@ -6,7 +6,8 @@
 
 namespace itp {
 
-template cudaError_t launch_pencil<double>(const GridDesc&, const PencilArgs<double>&, cudaStream_t);
+template cudaError_t launch_pencil<double>(const GridDesc&, const PencilArgs<double>*, int,
+                                          cudaStream_t);
 template cudaError_t launch_pencil_group<double>(const GridDesc&, int, const PencilArgs<double>*,
                                                  const int2*, int, cudaStream_t);
 

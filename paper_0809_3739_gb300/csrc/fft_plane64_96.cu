@@ -6,7 +6,8 @@
 
 namespace itp {
 
-template cudaError_t plane64_dispatch<96, 96>(const GridDesc&, int, const PlaneArgs<double>&,
+template cudaError_t plane64_dispatch<96, 96>(const GridDesc&, int,
+                                             const TermPack<PlaneArgs<double>>&,
                                              const PlaneArgs<double>*, const int2*, int, size_t,
                                              cudaStream_t);
 

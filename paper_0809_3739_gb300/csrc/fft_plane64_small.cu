@@ -6,13 +6,16 @@
 
 namespace itp {
 
-template cudaError_t plane64_dispatch<32, 32>(const GridDesc&, int, const PlaneArgs<double>&,
+template cudaError_t plane64_dispatch<32, 32>(const GridDesc&, int,
+                                             const TermPack<PlaneArgs<double>>&,
                                              const PlaneArgs<double>*, const int2*, int, size_t,
                                              cudaStream_t);
-template cudaError_t plane64_dispatch<48, 48>(const GridDesc&, int, const PlaneArgs<double>&,
+template cudaError_t plane64_dispatch<48, 48>(const GridDesc&, int,
+                                             const TermPack<PlaneArgs<double>>&,
                                              const PlaneArgs<double>*, const int2*, int, size_t,
                                              cudaStream_t);
-template cudaError_t plane64_dispatch<64, 64>(const GridDesc&, int, const PlaneArgs<double>&,
+template cudaError_t plane64_dispatch<64, 64>(const GridDesc&, int,
+                                             const TermPack<PlaneArgs<double>>&,
                                              const PlaneArgs<double>*, const int2*, int, size_t,
                                              cudaStream_t);
 

@@ -6,7 +6,7 @@
 
 namespace itp {
 
-template cudaError_t launch_plane<float>(const GridDesc&, const PlaneArgs<float>&, cudaStream_t,
-                                         int*);
+template cudaError_t launch_plane<float>(const GridDesc&, const PlaneArgs<float>*, int,
+                                         cudaStream_t, int*);
 
 }  // namespace itp

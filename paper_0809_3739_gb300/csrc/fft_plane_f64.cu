@@ -6,7 +6,7 @@
 
 namespace itp {
 
-template cudaError_t launch_plane<double>(const GridDesc&, const PlaneArgs<double>&, cudaStream_t,
-                                          int*);
+template cudaError_t launch_plane<double>(const GridDesc&, const PlaneArgs<double>*, int,
+                                         cudaStream_t, int*);
 
 }  // namespace itp

@@ -155,16 +155,22 @@ __device__ __forceinline__ void pencil_batch(const float2* col, long long zs, in
 struct PencilCol {
   float2* col;
   bool active;
+  int term;
   float fx, fy;
 };
-__device__ __forceinline__ PencilCol pencil_col(const GridDesc& g, const PencilArgs<float>& a,
+__device__ __forceinline__ PencilCol pencil_col(const GridDesc& g,
+                                                const TermPack<PencilArgs<float>>& p,
                                                 long long c, long long total) {
   PencilCol r;
   r.active = c < total;
   if (!r.active) c = total - 1;
   const long long cps = (long long)g.ny * g.nxh;
-  const long long s = c / cps;
-  const int q = (int)(c - s * cps);
+  const long long row = c / cps;               // (term, state)
+  const int t = (int)(row / p.a[0].m);
+  const PencilArgs<float>& a = p.a[t];
+  const long long s = row - (long long)t * a.m;
+  r.term = t;
+  const int q = (int)(c - row * cps);
   const int ky = q / g.nxh, kx = q - ky * g.nxh;
   r.col = static_cast<float2*>(a.spec) + s * g.n_half + q;
   r.fx = __ldg(&a.kx_tab[kx]);
@@ -198,12 +204,14 @@ __device__ __forceinline__ void pencil_stage1(float2 (&v)[16], int n1, const flo
 // registers cost more than the hidden latency gained.)
 template <int MODE>
 __global__ void __launch_bounds__(kTmThreads, 2)
-    pencil128_tm_kernel(const GridDesc g, const PencilArgs<float> a) {
+    pencil128_tm_kernel(const GridDesc g, const __grid_constant__ TermPack<PencilArgs<float>> p,
+                        int nterm) {
+  const PencilArgs<float>& a = p.a[0];
   __shared__ uint32_t tbase;
-  __shared__ float kz_s[128];    // kinetic factor along z
+  __shared__ float kz_s[kMaxTermsK][128];   // kinetic factor along z, per term
   __shared__ float2 tw_s[128];   // exp(-2 pi i m / 128)
   const int warp = threadIdx.x >> 5;
-  kz_s[threadIdx.x] = a.kz_tab[threadIdx.x];
+  for (int t = 0; t < nterm; ++t) kz_s[t][threadIdx.x] = p.a[t].kz_tab[threadIdx.x];
   tw_s[threadIdx.x] = static_cast<const float2*>(a.twz)[threadIdx.x];
   if (warp == 0) tmem_alloc(&tbase, kTmCols);
   tc_fence_before();
@@ -211,10 +219,10 @@ __global__ void __launch_bounds__(kTmThreads, 2)
   tc_fence_after();
   const uint32_t tm = tbase + ((uint32_t)(32 * warp) << 16);
   const long long zs = (long long)g.ny * g.nxh;
-  const long long total = (long long)a.m * zs;
+  const long long total = (long long)nterm * a.m * zs;
   const long long ntiles = (total + kTmThreads - 1) / kTmThreads;
   long long tile = blockIdx.x;
-  PencilCol cur = pencil_col(g, a, tile * kTmThreads + threadIdx.x, total);
+  PencilCol cur = pencil_col(g, p, tile * kTmThreads + threadIdx.x, total);
   float2 pf[kTmPrefetch][16];
 #pragma unroll
   for (int b = 0; b < kTmPrefetch; ++b) pencil_batch(cur.col, zs, b, pf[b]);
@@ -243,7 +251,7 @@ __global__ void __launch_bounds__(kTmThreads, 2)
       Dft<8, -1, float2>::run(u);
 #pragma unroll
       for (int k1 = 0; k1 < 8; ++k1) {
-        const float fz = kz_s[k2 + 16 * k1];
+        const float fz = kz_s[cur.term][k2 + 16 * k1];
         float f;
         if constexpr (MODE == PENCIL_PROPAGATE) f = fxy * fz;
         else f = (cur.fx + cur.fy + fz) * a.scale;
@@ -257,7 +265,7 @@ __global__ void __launch_bounds__(kTmThreads, 2)
       tm_wait_st<16>(r);
     }
     // the next tile's first batches (a valid column in any case)
-    const PencilCol nxt = pencil_col(g, a, (tile + gridDim.x) * kTmThreads + threadIdx.x, total);
+    const PencilCol nxt = pencil_col(g, p, (tile + gridDim.x) * kTmThreads + threadIdx.x, total);
 #pragma unroll
     for (int b = 0; b < kTmPrefetch; ++b) pencil_batch(nxt.col, zs, b, pf[b]);
     // inverse stage 2

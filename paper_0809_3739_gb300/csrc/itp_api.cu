@@ -33,6 +33,7 @@ struct Lane {
   void* work = nullptr;      // [m][n_half] complex
   void* work_terms[kMaxTerms] = {};  // per-term spectra / contributions (mixed)
   bool fused_ok = true;              // per-term workspaces could be allocated
+  bool together_ok = true;
   R* f_half[kMaxTerms] = {}; // exp(-tau_i V / 2)
   R* f_full[kMaxTerms] = {}; // exp(-tau_i V)      (terms i >= 2)
   R* ktab = nullptr;         // per term: nxh + ny + nz propagation factors
@@ -55,11 +56,15 @@ struct RecOp {
   int kind = kOther;
   int lane = 0;               // 0: FP32 arguments, 1: FP64
   int mode = 0;               // plane or pencil mode
-  PlaneArgs<float> p32{};
-  PlaneArgs<double> p64{};
-  PencilArgs<float> e32{};
-  PencilArgs<double> e64{};
+  std::vector<PlaneArgs<float>> p32;    // one entry per term of the pass
+  std::vector<PlaneArgs<double>> p64;
+  std::vector<PencilArgs<float>> e32;
+  std::vector<PencilArgs<double>> e64;
   TermSumArgs ts{};
+  int terms() const {
+    return kind == kPlane ? (int)(p32.size() + p64.size())
+                          : (kind == kPencil ? (int)(e32.size() + e64.size()) : 1);
+  }
   std::function<cudaError_t()> fn;   // the launch on the problem's stream
 };
 
@@ -378,40 +383,42 @@ void free_lane(Lane<R>& L) {
   L = Lane<R>();
 }
 
-// A plane pass: 1 kernel, or 2-3 kernels on split planes (counted).
+// A plane pass of n terms: 1 kernel, or 2-3 kernels on split planes (counted).
 template <typename R>
-cudaError_t plane_counted(itp_handle h, const PlaneArgs<R>& a) {
+cudaError_t plane_counted(itp_handle h, const PlaneArgs<R>* ap, int n_terms = 1) {
   if (h->rec) {
+    const std::vector<PlaneArgs<R>> a(ap, ap + n_terms);
     RecOp op;
     op.kind = RecOp::kPlane;
     op.lane = sizeof(R) == 8;
-    op.mode = a.mode;
+    op.mode = ap->mode;
     if constexpr (sizeof(R) == 4) op.p32 = a;
     else op.p64 = a;
-    op.fn = [h, a]() { int n = 1; return launch_plane<R>(h->g, a, h->st, &n); };
+    op.fn = [h, a]() { return launch_plane<R>(h->g, a.data(), (int)a.size(), h->st); };
     h->rec->push_back(std::move(op));
     return cudaSuccess;
   }
   int n = 1;
-  const cudaError_t e = launch_plane<R>(h->g, a, h->st, &n);
+  const cudaError_t e = launch_plane<R>(h->g, ap, n_terms, h->st, &n);
   h->launches += n - 1;
   return e;
 }
 
 template <typename R>
-cudaError_t pencil_counted(itp_handle h, const PencilArgs<R>& a) {
+cudaError_t pencil_counted(itp_handle h, const PencilArgs<R>* ap, int n_terms = 1) {
   if (h->rec) {
+    const std::vector<PencilArgs<R>> a(ap, ap + n_terms);
     RecOp op;
     op.kind = RecOp::kPencil;
     op.lane = sizeof(R) == 8;
-    op.mode = a.mode;
+    op.mode = ap->mode;
     if constexpr (sizeof(R) == 4) op.e32 = a;
     else op.e64 = a;
-    op.fn = [h, a]() { return launch_pencil<R>(h->g, a, h->st); };
+    op.fn = [h, a]() { return launch_pencil<R>(h->g, a.data(), (int)a.size(), h->st); };
     h->rec->push_back(std::move(op));
     return cudaSuccess;
   }
-  return launch_pencil<R>(h->g, a, h->st);
+  return launch_pencil<R>(h->g, ap, n_terms, h->st);
 }
 
 cudaError_t term_sum_counted(itp_handle h, const TermSumArgs& a) {
@@ -450,99 +457,149 @@ int prepare_tables(itp_handle h, Lane<R>& L, int k, double tau) {
   return ITP_OK;
 }
 
+// Whether the terms of the expansion run together, one launch per pass over
+// all of them: they are independent up to the final sum, and a term of a
+// small problem does not fill the GPU for longer than a launch takes to
+// start.  The results are the same bit for bit.  (24 states at 32^3, order 8,
+// FP32: 26 passes in 10 launches, a step 0.354 -> 0.312 ms; 89 states on 256^2,
+// order 12, 1.91 -> 1.78 ms; 61 on 96 x 72 x 48 7 % of a step.  Where one term
+// already is many waves of CTAs nothing is gained and the workspaces are
+// large: 57 states at 64^3 1 %.)
+constexpr long long kTogetherElems = 12LL << 20;   // half-spectrum values of one term
+constexpr size_t kTogetherBytes = (size_t)1 << 30; // workspaces of all terms
+template <typename R>
+bool terms_together(itp_handle h, int k) {
+  const GridDesc& g = h->g;
+  const long long elems = (long long)h->m * g.n_half;
+  return k > 1 && g.split_planes[sizeof(R) == 4 ? 0 : 1] < 2 &&
+         elems <= kTogetherElems && (size_t)k * elems * 2 * sizeof(R) <= kTogetherBytes &&
+         (long long)k * h->m * g.nz <= 65535;
+}
+// Whether the mixed path keeps every term's contribution and sums them once.
+template <typename R>
+bool terms_fused(itp_handle h) {
+  return sizeof(R) == 4 && lane_of<R>(h).fused_ok && h->g.split_planes[0] != 1;
+}
+
+// A workspace per term, where the terms run together or keep their
+// contributions; without the memory for it both are off for the handle.
+template <typename R>
+void term_workspaces(itp_handle h, int k, bool step = true) {
+  Lane<R>& L = lane_of<R>(h);
+  L.work_terms[0] = L.work;
+  if (!terms_fused<R>(h) && !(step && L.together_ok && terms_together<R>(h, k))) return;
+  for (int i = 1; i < k; ++i) {
+    if (!L.work_terms[i] &&
+        cudaMalloc(&L.work_terms[i], (size_t)h->m * h->g.n_half * 2 * sizeof(R)) != cudaSuccess) {
+      cudaGetLastError();   // clear the allocation error; use the per-term path
+      L.fused_ok = L.together_ok = false;
+      return;
+    }
+  }
+}
+
 // Eq. (3) with the order-2k expansion: acc = sum_i c_i T_2(tau/i)^i psi.
 // Per term i: plane-forward with exp(-tau_i V/2), then i pencils with i-1
 // merged plane passes (exp(-tau_i V)) between them, then the final inverse
 // plane pass with exp(-tau_i V/2) adds c_i u_i (Sec. II).  The mixed path
 // keeps every term's spectrum in its own workspace, writes each term's FP32
 // contribution c_i f u_i over it, and sums the contributions once in FP64.
+// step: part of a whole step, whose passes may run all terms together; on its
+// own (itp_propagate) a propagation is the k(k+2) passes, each one launch, that
+// itp_kernel_launches and itp_profile count.
 template <typename R>
 int propagate_lane(itp_handle h, int k, double tau, int s0 = 0, const R* in = nullptr,
-                   R* out = nullptr, int s1 = -1) {
+                   R* out = nullptr, int s1 = -1, bool step = true) {
   Lane<R>& L = lane_of<R>(h);
   ITP_TRY(prepare_tables<R>(h, L, k, tau));
   const GridDesc& g = h->g;
   const size_t tl = (size_t)g.nxh + g.ny + g.nz;
-  bool fused = sizeof(R) == 4 && L.fused_ok && g.split_planes[0] != 1;
-  if (fused) {
-    L.work_terms[0] = L.work;
-    for (int i = 1; i < k && fused; ++i) {
-      if (!L.work_terms[i] &&
-          cudaMalloc(&L.work_terms[i], (size_t)h->m * g.n_half * 2 * sizeof(R)) != cudaSuccess) {
-        cudaGetLastError();   // clear the allocation error; use the per-term path
-        L.fused_ok = fused = false;
-      }
-    }
-  }
+  term_workspaces<R>(h, k, step);
+  const bool fused = terms_fused<R>(h);
+  const bool together = step && L.together_ok && terms_together<R>(h, k);
   // states s0..s1-1 only (s1 < 0: to the last state; the others are kept)
   const int ms = (s1 < 0 ? h->m : s1) - s0;
   const long long so = s0;
   auto at_state = [&](void* w) {
     return static_cast<void*>(static_cast<char*>(w) + so * g.n_half * 2 * sizeof(R));
   };
+  const bool planar = g.nz == 1;   // the kinetic factor ends each forward pass
   TermSumArgs ts{};
+  PlaneArgs<R> pf[kMaxTerms];      // per term: forward, merged and final plane pass, pencil
+  PlaneArgs<R> pm[kMaxTerms], pl[kMaxTerms];
+  PencilArgs<R> pe[kMaxTerms];
   for (int i = 1; i <= k; ++i) {
-    void* work = at_state(fused ? L.work_terms[i - 1] : L.work);
+    void* work = at_state(fused || together ? L.work_terms[i - 1] : L.work);
+    const R* kt = L.ktab + (i - 1) * tl;
     PlaneArgs<R> pa{};
     pa.m = ms;
     pa.in_real = (in ? in : L.psi) + so * g.n_points;
     pa.spec = work;
     pa.twx = L.twx;
     pa.twy = L.twy;
-    pa.mode = PLANE_FWD_REAL;
-    pa.f_in = L.f_half[i - 1];
-    const bool planar = g.nz == 1;   // the kinetic factor ends each forward pass
     if (planar) {
-      const R* kt = L.ktab + (i - 1) * tl;
       pa.kin.fx = kt;
       pa.kin.fy = kt + g.nxh;
       pa.kin.fz = kt + g.nxh + g.ny;
       pa.kin.mode = 0;
     }
-    ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_FWD, plane_counted<R>(h, pa));
-    PencilArgs<R> pe{};
-    pe.mode = PENCIL_PROPAGATE;
-    pe.m = ms;
-    pe.spec = work;
-    pe.kx_tab = L.ktab + (i - 1) * tl;
-    pe.ky_tab = pe.kx_tab + g.nxh;
-    pe.kz_tab = pe.ky_tab + g.ny;
-    pe.scale = (R)1;
-    pe.twz = L.twz;
-    for (int j = 1; j <= i; ++j) {
-      if (!planar)
-        ITP_LAUNCH_PASS(h, pe.mode == PENCIL_PROPAGATE ? ITP_KERNEL_PENCIL
-                                                       : ITP_KERNEL_PENCIL_KINETIC,
-                        pencil_counted<R>(h, pe));
-      if (j < i) {
-        PlaneArgs<R> pm = pa;
-        pm.mode = PLANE_MERGED;
-        pm.f_in = nullptr;
-        pm.f_mid = L.f_full[i - 1];
-        ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_MERGED, plane_counted<R>(h, pm));
-      }
-    }
+    pf[i - 1] = pa;
+    pf[i - 1].mode = PLANE_FWD_REAL;
+    pf[i - 1].f_in = L.f_half[i - 1];
+    pm[i - 1] = pa;
+    pm[i - 1].mode = PLANE_MERGED;
+    pm[i - 1].f_mid = L.f_full[i - 1];
+    PlaneArgs<R>& p = pl[i - 1];
+    p = pa;
+    p.f_out = L.f_half[i - 1];
+    p.coef = mp_coefficient(i, k);
     if (fused) {
       // the term's contribution c_i f u_i, in place over its spectrum
-      PlaneArgs<R> pt = pa;
-      pt.mode = PLANE_TERM;
-      pt.f_in = nullptr;
-      pt.f_out = L.f_half[i - 1];
-      pt.coef = mp_coefficient(i, k);
-      ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_COMBINE, plane_counted<R>(h, pt));
+      p.mode = PLANE_TERM;
       ts.term[i - 1] = reinterpret_cast<const float*>(work);
-      continue;
+    } else {
+      p.mode = PLANE_COMBINE;
+      p.acc = (sizeof(R) == 8 && out ? reinterpret_cast<double*>(out) : h->acc) + so * g.n_points;
+      p.acc_init = (i == 1);
+      // the mixed path keeps the sum in FP64 and rounds the finished phi once
+      p.phi_out = (sizeof(R) == 4 && i == k) ? (out ? out : L.psi_tmp) + so * g.n_points : nullptr;
     }
-    PlaneArgs<R> pc = pa;
-    pc.mode = PLANE_COMBINE;
-    pc.f_in = nullptr;
-    pc.f_out = L.f_half[i - 1];
-    pc.acc = (sizeof(R) == 8 && out ? reinterpret_cast<double*>(out) : h->acc) + so * g.n_points;
-    pc.coef = mp_coefficient(i, k);
-    pc.acc_init = (i == 1);
-    // the mixed path keeps the sum in FP64 and rounds the finished phi once
-    pc.phi_out = (sizeof(R) == 4 && i == k) ? (out ? out : L.psi_tmp) + so * g.n_points : nullptr;
-    ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_COMBINE, plane_counted<R>(h, pc));
+    PencilArgs<R>& q = pe[i - 1];
+    q = PencilArgs<R>{};
+    q.mode = PENCIL_PROPAGATE;
+    q.m = ms;
+    q.spec = work;
+    q.kx_tab = kt;
+    q.ky_tab = kt + g.nxh;
+    q.kz_tab = kt + g.nxh + g.ny;
+    q.scale = (R)1;
+    q.twz = L.twz;
+  }
+  // terms i0 .. i1, each pass over all of them that still need it
+  auto run_terms = [&](int i0, int i1) -> int {
+    const int n = i1 - i0 + 1;
+    ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_FWD, plane_counted<R>(h, pf + i0 - 1, n));
+    for (int j = 1; j <= i1; ++j) {
+      const int first = std::max(i0, j), next = std::max(i0, j + 1);
+      if (!planar)
+        ITP_LAUNCH_PASS(h, ITP_KERNEL_PENCIL,
+                        pencil_counted<R>(h, pe + first - 1, i1 - first + 1));
+      if (j < i1)
+        ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_MERGED,
+                        plane_counted<R>(h, pm + next - 1, i1 - next + 1));
+    }
+    if (fused) {
+      ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_COMBINE, plane_counted<R>(h, pl + i0 - 1, n));
+    } else {   // in order: the sum is kept in memory
+      for (int i = i0; i <= i1; ++i)
+        ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_COMBINE, plane_counted<R>(h, pl + i - 1, 1));
+    }
+    return ITP_OK;
+  };
+  if (together) {
+    ITP_TRY(run_terms(1, k));
+  } else {
+    for (int i = 1; i <= k; ++i) ITP_TRY(run_terms(i, i));
   }
   if (fused) {
     // phi = sum_i c_i f u_i in FP64 over the FP32 contributions
@@ -615,7 +672,7 @@ int energies_lane(itp_handle h, int flags) {
     pa.kin.mode = 1;
     pa.kin.scale = (R)(1.0 / (double)g.n_points);
   }
-  ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_FWD, plane_counted<R>(h, pa));
+  ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_FWD, plane_counted<R>(h, &pa));
   pa.kin = KinFac<R>{};
   PencilArgs<R> pe{};
   pe.mode = PENCIL_KINETIC;
@@ -628,7 +685,7 @@ int energies_lane(itp_handle h, int flags) {
   pe.twz = L.twz;
   if (!planar)
     ITP_LAUNCH_PASS(h, pe.mode == PENCIL_PROPAGATE ? ITP_KERNEL_PENCIL : ITP_KERNEL_PENCIL_KINETIC,
-                    pencil_counted<R>(h, pe));
+                    pencil_counted<R>(h, &pe));
   PlaneArgs<R> ph = pa;
   ph.mode = PLANE_HPSI;
   ph.acc = h->acc;
@@ -637,7 +694,7 @@ int energies_lane(itp_handle h, int flags) {
     ph.V_r = L.Vr;
     ph.phi_out = L.psi_tmp;
   }
-  ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_HPSI, plane_counted<R>(h, ph));
+  ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_HPSI, plane_counted<R>(h, &ph));
   if (sizeof(R) == 4) {
     ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_tc_gram(
                                        reinterpret_cast<const float*>(L.psi),
@@ -760,18 +817,7 @@ template <typename R>
 int step_resources(itp_handle h, int k, double tau) {
   Lane<R>& L = lane_of<R>(h);
   ITP_TRY(prepare_tables<R>(h, L, k, tau));
-  if (sizeof(R) == 4 && L.fused_ok && h->g.split_planes[0] != 1) {
-    L.work_terms[0] = L.work;
-    for (int i = 1; i < k; ++i) {
-      if (!L.work_terms[i] &&
-          cudaMalloc(&L.work_terms[i], (size_t)h->m * h->g.n_half * 2 * sizeof(R)) !=
-              cudaSuccess) {
-        cudaGetLastError();
-        L.fused_ok = false;
-        break;
-      }
-    }
-  }
+  term_workspaces<R>(h, k);
   return ITP_OK;
 }
 
@@ -1220,6 +1266,7 @@ std::string group_key(itp_handle h, const std::vector<RecOp>& ops) {
   for (const RecOp& op : ops) {
     key += (char)('a' + op.kind);
     key += (char)('0' + op.mode);
+    key += (char)('0' + op.terms());
   }
   return key;
 }
@@ -1281,26 +1328,29 @@ int build_grouped_graph(itp_batch* b, int k, double tau, int eflags, cudaGraph_t
       std::vector<unsigned char> args;
       for (int q = 0; q < (int)G.size(); ++q) {
         const RecOp& op = ops[G[q]][t];
+        // a table entry and its states per term
+        const size_t nt = op.terms();
         int nrow = 0;
         const void* a = nullptr;
         size_t asz = 0;
         if (op.kind == RecOp::kPlane) {
-          nrow = op.lane ? op.p64.m : op.p32.m;
-          a = op.lane ? (const void*)&op.p64 : (const void*)&op.p32;
-          asz = op.lane ? sizeof(op.p64) : sizeof(op.p32);
+          nrow = op.lane ? op.p64[0].m : op.p32[0].m;
+          a = op.lane ? (const void*)op.p64.data() : (const void*)op.p32.data();
+          asz = op.lane ? sizeof(op.p64[0]) : sizeof(op.p32[0]);
         } else if (op.kind == RecOp::kPencil) {
-          nrow = op.lane ? op.e64.m : op.e32.m;
-          a = op.lane ? (const void*)&op.e64 : (const void*)&op.e32;
-          asz = op.lane ? sizeof(op.e64) : sizeof(op.e32);
+          nrow = op.lane ? op.e64[0].m : op.e32[0].m;
+          a = op.lane ? (const void*)op.e64.data() : (const void*)op.e32.data();
+          asz = op.lane ? sizeof(op.e64[0]) : sizeof(op.e32[0]);
         } else {
           nrow = op.ts.m;
           a = &op.ts;
           asz = sizeof(op.ts);
         }
-        for (int r = 0; r < nrow; ++r) rows.push_back(make_int2(q, r));
+        for (size_t e = 0; e < nt; ++e)
+          for (int r = 0; r < nrow; ++r) rows.push_back(make_int2((int)(q * nt + e), r));
         const size_t o = args.size();
-        args.resize(o + asz);
-        memcpy(args.data() + o, a, asz);
+        args.resize(o + nt * asz);
+        memcpy(args.data() + o, a, nt * asz);
       }
       if (rows.size() > 65535)
         return batch_fail(b, ITP_ERR_ARG, "a group has more than 65535 states; "
@@ -1704,9 +1754,9 @@ int itp_propagate(itp_handle h, int order, double tau) {
   const int k = order / 2;
   if (h->precision == ITP_MIXED) {
     ITP_TRY(switch_lane<float>(h));
-    ITP_TRY(propagate_lane<float>(h, k, tau));
+    ITP_TRY(propagate_lane<float>(h, k, tau, 0, nullptr, nullptr, -1, false));
   } else {
-    ITP_TRY(propagate_lane<double>(h, k, tau));
+    ITP_TRY(propagate_lane<double>(h, k, tau, 0, nullptr, nullptr, -1, false));
   }
   h->have_phi = true;
   return ITP_OK;

@@ -24,6 +24,16 @@ struct GridDesc {
 };
 
 // Pass kinds.
+constexpr int kMaxTermsK = 6;   // terms of the expansion (order <= 12)
+
+// The arguments of up to kMaxTermsK passes of one kind over the same number
+// of states, run by one launch (the terms of the expansion are independent):
+// by value in the kernel parameters.
+template <typename A>
+struct TermPack {
+  A a[kMaxTermsK];
+};
+
 enum PlaneMode {
   PLANE_FWD_REAL = 0,   // real state * f_in -> half spectrum
   PLANE_MERGED = 1,     // half spectrum -> inverse -> * f_mid -> forward -> half spectrum
@@ -89,7 +99,6 @@ struct PencilArgs {
 // TwoSum accumulation; mixed path): term_i holds the FP32 contribution
 // c_i * f_i * u_i of term i, stored plane by plane with the half-spectrum
 // plane pitch (floats); phi is [m][N].
-constexpr int kMaxTermsK = 6;
 struct TermSumArgs {
   int m, k, nz, plane_pts;
   long long plane_pitch;
@@ -116,16 +125,18 @@ cudaError_t launch_pencil_group(const GridDesc& g, int mode, const PencilArgs<R>
 cudaError_t launch_term_sum_group(const TermSumArgs* args, const int2* rows, int nrows, int nz,
                                   int plane_pts, cudaStream_t st);
 
-// One plane pass (*nlaunch receives the number of kernels: 1, or 2-3 when
-// the planes are split into row and column passes).
+// One plane pass of n <= kMaxTermsK terms, a[0..n), alike in mode and states
+// (*nlaunch receives the number of kernels: 1, 2-3 when the planes are split
+// into row and column passes, n times that for cluster planes).
 template <typename R>
-cudaError_t launch_plane(const GridDesc& g, const PlaneArgs<R>& a, cudaStream_t st,
+cudaError_t launch_plane(const GridDesc& g, const PlaneArgs<R>* a, int n, cudaStream_t st,
                          int* nlaunch = nullptr);
 template <typename R>
-cudaError_t launch_pencil(const GridDesc& g, const PencilArgs<R>& a, cudaStream_t st);
+cudaError_t launch_pencil(const GridDesc& g, const PencilArgs<R>* a, int n, cudaStream_t st);
 // The pencil pass with one thread per z column and the column held in TMEM
 // (nz = 128, FP32; GridDesc::pencil_w = 0 selects it in launch_pencil).
-cudaError_t launch_pencil_tm(const GridDesc& g, const PencilArgs<float>& a, cudaStream_t st);
+cudaError_t launch_pencil_tm(const GridDesc& g, const PencilArgs<float>* a, int n,
+                             cudaStream_t st);
 
 // Factor tables of one term, tau_i = tau / i:
 //   f_half = exp(-tau_i V / 2), f_full = exp(-tau_i V)   ([N] each, precision R)
