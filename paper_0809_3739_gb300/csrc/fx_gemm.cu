@@ -10,6 +10,7 @@
 //   Gram:   h h', and h l' + l h' (l l' is below the precision, see there);
 //   update: h h', h l' + l h', and l l',
 // accumulated exactly in 64-bit integers over up to 512 terms.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -26,9 +27,9 @@ constexpr int kHalf = 28;    // bits of the lower half
 
 // The double d as an integer of scale 2^(BITS - 1) at the biased exponent e
 // (|d| < 2^(e - 1022)): |result| <= 2^BITS, rounded to nearest, 0 for
-// subnormal d; as halves (h, l) with l in [-2^27, 2^27).
+// subnormal d; to_halves: as halves (h, l) with l in [-2^27, 2^27).
 template <int BITS>
-__device__ __forceinline__ int2 to_halves(double d, int e) {
+__device__ __forceinline__ long long to_integer(double d, int e) {
   const long long b = __double_as_longlong(d);
   const int ex = (int)((b >> 52) & 0x7ff);
   constexpr int kUp = 9;   // 53-bit mantissa to 62 bits: room to round
@@ -37,7 +38,11 @@ __device__ __forceinline__ int2 to_halves(double d, int e) {
   m = (m + ((1LL << s) >> 1)) >> s;
   m = ex == 0 ? 0 : m;
   const long long sg = b >> 63;
-  m = (m ^ sg) - sg;
+  return (m ^ sg) - sg;
+}
+template <int BITS>
+__device__ __forceinline__ int2 to_halves(double d, int e) {
+  const long long m = to_integer<BITS>(d, e);
   int2 r;
   r.x = (int)((m + (1LL << (kHalf - 1))) >> kHalf);
   r.y = (int)((unsigned)m << (32 - kHalf)) >> (32 - kHalf);
@@ -100,6 +105,10 @@ __device__ __forceinline__ void load_pairs(const int2* p, int2 (&v)[N]) {
 constexpr int kRun = 512;
 constexpr int kTile = 16;   // (32 points needed more registers for the tile in flight)
 constexpr int kGramBits = 54;
+// More states than this: the tensor-core form below.  57 states at 64^3: 0.50 ms
+// here, 0.27 there; 128: 1.74, 1.00; 48 at 128^3: 2.30, 1.92; but 32 at 24^3
+// 0.019 here, 0.037 there.
+constexpr int kGramMmaMin = 32;
 
 // (bi, bj) of the blocks, packed as bi * 256 + bj.
 struct GramBlocks {
@@ -239,6 +248,217 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
       }
     }
     __syncthreads();   // the exponents are rewritten by the next run
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same sums for more than kGramMmaMin states on the tensor cores: elements
+// as 55-bit integers in seven signed base-256 digits d_0 .. d_6, each exact in
+// FP16; the products of digits a and b belong to level a + b, and the levels
+// 0 .. 6 (28 digit products per element product) are accumulated apart, in
+// FP32: up to 7 * 128 products of at most 2^14 stay below 2^24, so the sums
+// over 128 points are exact whatever the rounding.  They are then moved to
+// 64-bit integers in shared memory (levels 0-3 and 4-6), and the run's sums to
+// FP64.  The levels above 6 are below the precision: about 2^-56 of the two
+// largest values per product, with random signs.
+//
+// mma.sync reaches 1000 FMAs per clock and SM here, a quarter of tcgen05, but
+// its sums are in registers: the seven accumulators of a 128 x 128 tile would
+// not fit TMEM, and would have to be read back every 128 points.  A CTA
+// of 16 warps sums a 64 x 64 block, 16 x 16 per warp.  (Against the IMAD.WIDE
+// form, 3.2 cycles per multiply-add: see kGramMmaMin.)
+constexpr int kMmaThreads = 512;
+constexpr int kMmaRows = 64;             // rows and columns of a block
+constexpr int kMmaTile = 32;             // points per tile
+constexpr int kMmaPitch = kMmaTile + 8;  // halves; rows 80 bytes apart: conflict-free ldmatrix
+constexpr int kDigits = 7;
+constexpr int kMmaBits = 55;
+constexpr int kMmaDrain = 128 / kMmaTile;   // tiles between drains
+constexpr size_t kMmaOperand = (size_t)kDigits * kMmaRows * kMmaPitch;   // halves
+constexpr size_t kMmaSmem = 2 * 2 * kMmaOperand * 2 + (size_t)16 * kMmaThreads * 8;
+
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                        uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},"
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Two FP16 digits from 10-bit fields u = digit + 128 in the halves of x: FP16
+// 1024 + u has the bits 0x6400 + u.
+__device__ __forceinline__ uint32_t digits_f16(uint32_t x, uint32_t mask) {
+  uint32_t r = (x & mask) | 0x64006400u;
+  asm("add.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0xe480e480u));   // - 1152
+  return r;
+}
+// The digits of two integers: pair l = (digit l of v0, digit l of v1).
+__device__ __forceinline__ void digit_pairs(long long v0, long long v1, uint32_t (&d)[kDigits]) {
+  constexpr long long kBias = 0x0080808080808080LL;   // every digit + 128, no borrows
+  v0 += kBias;
+  v1 += kBias;
+  const uint32_t l0 = (uint32_t)v0, h0 = (uint32_t)(v0 >> 32);
+  const uint32_t l1 = (uint32_t)v1, h1 = (uint32_t)(v1 >> 32);
+  d[0] = digits_f16(__byte_perm(h0, h1, 0x7632), 0x01ff01ffu);
+  d[1] = digits_f16(__byte_perm(h0, h1, 0x0501), 0x00ff00ffu);
+  d[2] = digits_f16(__byte_perm(h0, h1, 0x0400), 0x00ff00ffu);
+  d[3] = digits_f16(__byte_perm(l0, l1, 0x0703), 0x00ff00ffu);
+  d[4] = digits_f16(__byte_perm(l0, l1, 0x0602), 0x00ff00ffu);
+  d[5] = digits_f16(__byte_perm(l0, l1, 0x0501), 0x00ff00ffu);
+  d[6] = digits_f16(__byte_perm(l0, l1, 0x0400), 0x00ff00ffu);
+}
+
+__global__ void __launch_bounds__(kMmaThreads, 1)
+    fx_gram_mma_kernel(const double* __restrict__ A, const double* __restrict__ B, int m,
+                       long long N, long long chunk, double* __restrict__ partial,
+                       const GramBlocks blocks, int same) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __half* sD = reinterpret_cast<__half*>(smraw);   // [2 buffers][2 operands][digit][row][pitch]
+  long long* sacc = reinterpret_cast<long long*>(smraw + 2 * 2 * kMmaOperand * 2);   // [16][tid]
+  __shared__ int eA[kMmaRows], eB[kMmaRows];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int bi = blocks.ij[blockIdx.y] >> 8, bj = blocks.ij[blockIdx.y] & 255;
+  const bool one = same && bi == bj;       // a diagonal block: one operand
+  const int ia = kMmaRows * bi, jb = kMmaRows * bj;
+  const long long p_begin = (long long)blockIdx.x * chunk;
+  const long long p_end = p_begin + chunk < N ? p_begin + chunk : N;
+  double* out = partial + (long long)blockIdx.x * m * m;
+  // this warp's 16 x 16 part, and this thread's entry c of its column tile n
+  const int wi = 16 * (warp >> 2), wj = 16 * (warp & 3);
+  auto row_of = [&](int c) { return wi + (lane >> 2) + 8 * (c >> 1); };
+  auto col_of = [&](int n, int c) { return wj + 8 * n + 2 * (lane & 3) + (c & 1); };
+  auto add_sum = [&](int i, int j, double v, bool first) {
+    if (i >= m || j >= m) return;
+    if (!first) v += out[i * m + j];
+    out[i * m + j] = v;
+    if (same && bi != bj) out[j * m + i] = v;
+  };
+  if (p_begin >= p_end) {
+    for (int q = 0; q < 8; ++q) add_sum(ia + row_of(q & 3), jb + col_of(q >> 2, q & 3), 0.0, true);
+    return;
+  }
+  // ldmatrix addresses: A 16 rows x 16 points, B 16 columns x 16 points
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(sD);
+  const uint32_t offA = (uint32_t)(((wi + (lane & 7) + 8 * ((lane >> 3) & 1)) * kMmaPitch +
+                                    8 * (lane >> 4)) * 2);
+  const uint32_t offB = (uint32_t)(((wj + (lane & 7) + 8 * (lane >> 4)) * kMmaPitch +
+                                    8 * ((lane >> 3) & 1)) * 2);
+  constexpr uint32_t kSlice = kMmaRows * kMmaPitch * 2, kOp = kMmaOperand * 2;
+  const int lr = tid >> 3, lp = 4 * (tid & 7);   // tile load: row, first of four points
+  double va[4], vb[4];
+  auto load = [&](const double* X, int r0, long long p0, long long pe, double (&v)[4]) {
+    const double* src = X + (long long)(r0 + lr) * N + p0 + lp;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = (r0 + lr < m && p0 + lp + q < pe) ? src[q] : 0.0;
+  };
+  auto store = [&](int buf, int op, const double (&v)[4], int e) {
+    uint32_t d0[kDigits], d1[kDigits];
+    digit_pairs(to_integer<kMmaBits>(v[0], e), to_integer<kMmaBits>(v[1], e), d0);
+    digit_pairs(to_integer<kMmaBits>(v[2], e), to_integer<kMmaBits>(v[3], e), d1);
+    __half* dst = sD + (size_t)(buf * 2 + op) * kMmaOperand + lr * kMmaPitch + lp;
+#pragma unroll
+    for (int l = 0; l < kDigits; ++l)
+      *reinterpret_cast<uint2*>(dst + (size_t)l * kMmaRows * kMmaPitch) = make_uint2(d0[l], d1[l]);
+  };
+  for (long long run = p_begin; run < p_end; run += kRun) {
+    const long long re = run + kRun < p_end ? run + kRun : p_end;
+    for (int op = 0; op < (one ? 1 : 2); ++op) {   // largest exponents, one warp per row
+      const double* X = op == 0 ? A : B;
+      const int r0 = op == 0 ? ia : jb;
+      for (int i = warp; i < kMmaRows; i += kMmaThreads / 32) {
+        int e = 0;
+        if (r0 + i < m) {
+          const double* row = X + (long long)(r0 + i) * N + run;
+#pragma unroll 8
+          for (int k = lane; k < (int)(re - run); k += 32) e = fx_max(e, exponent(row[k]));
+        }
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) (op == 0 ? eA : eB)[i] = e;
+      }
+    }
+    load(A, ia, run, re, va);
+    if (!one) load(B, jb, run, re, vb);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) sacc[q * kMmaThreads + tid] = 0;
+    __syncthreads();
+    store(0, 0, va, eA[lr]);
+    if (!one) store(0, 1, vb, eB[lr]);
+    float acc[kDigits][2][4];
+#pragma unroll
+    for (int l = 0; l < kDigits; ++l)
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[l][n][c] = 0.f;
+    const int ntile = (int)((re - run + kMmaTile - 1) / kMmaTile);
+    for (int t = 0; t < ntile; ++t) {
+      const bool more = t + 1 < ntile;
+      if (more) {   // the next tile's loads are in flight meanwhile
+        const long long p0 = run + (long long)(t + 1) * kMmaTile;
+        load(A, ia, p0, re, va);
+        if (!one) load(B, jb, p0, re, vb);
+      }
+      __syncthreads();
+      const uint32_t tA = base + (uint32_t)(t & 1) * 2 * kOp + offA;
+      const uint32_t tB = base + (uint32_t)(t & 1) * 2 * kOp + (one ? 0 : kOp) + offB;
+#pragma unroll 1
+      for (int k = 0; k < kMmaTile; k += 16) {
+        uint32_t b[kDigits][4];
+#pragma unroll
+        for (int l = 0; l < kDigits; ++l) ldmatrix4(b[l], tB + l * kSlice + 2 * k);
+#pragma unroll
+        for (int l = 0; l < kDigits; ++l) {
+          uint32_t a[4];
+          ldmatrix4(a, tA + l * kSlice + 2 * k);
+#pragma unroll
+          for (int q = 0; q + l < kDigits; ++q) {
+            mma_f16(acc[l + q][0], a, b[q][0], b[q][1]);
+            mma_f16(acc[l + q][1], a, b[q][2], b[q][3]);
+          }
+        }
+      }
+      if (more) {
+        store((t + 1) & 1, 0, va, eA[lr]);
+        if (!one) store((t + 1) & 1, 1, vb, eB[lr]);
+      }
+      if (!more || (t + 1) % kMmaDrain == 0) {
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            int v[kDigits];
+#pragma unroll
+            for (int l = 0; l < kDigits; ++l) {
+              v[l] = __float2int_rn(acc[l][n][c]);
+              acc[l][n][c] = 0.f;
+            }
+            const int q = n * 4 + c;
+            long long hi = sacc[q * kMmaThreads + tid], lo = sacc[(8 + q) * kMmaThreads + tid];
+            hi += fx_wide(v[0], 1 << 24, fx_wide(v[1], 1 << 16, fx_wide(v[2], 1 << 8, v[3])));
+            lo += fx_wide(v[4], 1 << 16, fx_wide(v[5], 1 << 8, v[6]));
+            sacc[q * kMmaThreads + tid] = hi;
+            sacc[(8 + q) * kMmaThreads + tid] = lo;
+          }
+      }
+    }
+    // (hi 2^72 + lo 2^48) 2^(ea + eb - 2 * (1022 + 55))
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = row_of(q & 3), j = col_of(q >> 2, q & 3);
+      const int ea = eA[i], eb = (one ? eA : eB)[j];
+      const double sum = fma((double)sacc[q * kMmaThreads + tid], (double)(1 << 24),
+                             (double)sacc[(8 + q) * kMmaThreads + tid]);
+      double v = scale2(sum, ea + eb - 2 * (1022 + kMmaBits) + 48);
+      if (ea == 2047 || eb == 2047) v = __longlong_as_double(0x7ff8000000000000LL);
+      add_sum(ia + i, jb + j, v, run == p_begin);
+    }
+    __syncthreads();   // the exponents and buffers are rewritten by the next run
   }
 }
 
@@ -467,6 +687,20 @@ cudaError_t launch_gram_partial(const double* A, const double* B, int m, long lo
   // (few chunks: a caller's scratch limits them).
   const bool same = A == B;
   GramBlocks blocks{};
+  if (m > kGramMmaMin) {
+    const int nb = (m + kMmaRows - 1) / kMmaRows;
+    chunk = (chunk + kMmaTile - 1) / kMmaTile * kMmaTile;
+    for (int bi = 0; bi < nb; ++bi)
+      for (int bj = 0; bj < nb; ++bj)
+        if (!same || bj <= bi) blocks.ij[blocks.n++] = (short)(bi * 256 + bj);
+    cudaError_t e = cudaFuncSetAttribute(fx_gram_mma_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kMmaSmem);
+    if (e != cudaSuccess) return e;
+    fx_gram_mma_kernel<<<dim3(n_chunks, blocks.n), kMmaThreads, kMmaSmem, st>>>(
+        A, B, m, n_points, chunk, partial, blocks, same);
+    return cudaGetLastError();
+  }
   int tt = 4;
   for (int cap = 64; cap >= 32; cap -= 16) {
     const int nb = (m + cap - 1) / cap;
