@@ -48,6 +48,13 @@ cudaError_t plane64_dispatch(const GridDesc& g, int mode,
 namespace {
 
 constexpr int kThreads = 256;
+// Threads per SM that the generic plane instantiations (run-time sizes) are
+// compiled for, FP64 (128 registers) and FP32 (80), in CTAs of any size up to
+// that; one CTA of 256 threads with up to 255 registers left most of the SM
+// idle: FP64 merged pass at 72 x 48 90 -> 58 ps per value, FP32 at 96 x 72 19.2
+// -> 10.4 ps.
+constexpr int kGenericThreads64 = 512, kGenericThreads32 = 768;
+constexpr int kGenericCtas64 = 2;   // FP64 pencils of run-time sizes
 
 __host__ __device__ constexpr bool is_radix(int r) {
   return r == 1 || r == 2 || r == 3 || r == 4 || r == 6 || r == 8 || r == 12 || r == 16;
@@ -90,6 +97,37 @@ __host__ __device__ constexpr int launch_threads(int nt) { return (nt + 31) / 32
 // of 256 (0.268 ms against 0.289).
 __host__ __device__ constexpr int plane64_threads(int nx) {
   return nx == 128 ? 512 : nx == 64 ? 264 : kThreads;
+}
+
+// Threads per CTA of a plane kernel, and of its launch bounds.
+template <typename R>
+__host__ __device__ constexpr int plane_threads(int nx) {
+  return nx == 0 ? (sizeof(R) == 8 ? kGenericThreads64 : kGenericThreads32)
+                 : (sizeof(R) == 8 ? launch_threads(plane64_threads(nx)) : kThreads);
+}
+// Threads of a generic plane pass: the count that leaves the fewest of them
+// idle over the x and y stages of an nx x ny plane (a 24 x 48 plane has 78 to 144
+// tasks per stage), as long as the CTAs that shared memory admits fill the SM.
+template <typename R>
+int generic_threads(const GridDesc& g, size_t smem) {
+  const int nxh = g.nx / 2 + 1, np = g.ny / 2;
+  const int tasks[4] = {np * g.rx1, np * g.rx2, nxh * g.ry1, nxh * g.ry2};
+  const int radix[4] = {g.rx2, g.rx1, g.ry2, g.ry1};
+  const int full = plane_threads<R>(0);
+  int best = kThreads;
+  double least = -1;
+  for (int nt = 512; nt >= 96; nt -= 32) {
+    double cost = 0;   // thread-rounds, by the values of a task
+    for (int s = 0; s < 4; ++s) cost += (double)((tasks[s] + nt - 1) / nt) * nt * radix[s];
+    const int ctas = (int)(227 * 1024 / (smem + 1024));
+    const int resident = nt * (ctas < full / nt ? (ctas < 1 ? 1 : ctas) : full / nt);
+    cost *= (double)full / resident;
+    if (least < 0 || cost < least) {
+      least = cost;
+      best = nt;
+    }
+  }
+  return best;
 }
 
 // Shared-memory pitch of a row pair: room for the padded packed row
@@ -140,12 +178,13 @@ __device__ __forceinline__ void scale_by(SVec<C, N>& a, F&& f) {
 // the strided reads of the split/merge free of bank conflicts.
 __device__ __forceinline__ int swz(int p) { return p + (p >> 4); }
 
-// Task loop over NT threads: task = t + ntr * q, t fastest across lanes.
+// Task loop over NT threads (0: the whole CTA): task = t + ntr * q, t fastest
+// across lanes.
 template <int NT, typename F>
 __device__ __forceinline__ void for_tasks(int ntr, int nq, F&& f) {
   const int total = ntr * nq;
-  if (threadIdx.x >= NT) return;
-  for (int task = threadIdx.x; task < total; task += NT) {
+  if (NT > 0 && threadIdx.x >= NT) return;
+  for (int task = threadIdx.x; task < total; task += (NT > 0 ? NT : blockDim.x)) {
     const int q = task / ntr;
     const int t = task - q * ntr;
     f(t, q);
@@ -416,7 +455,8 @@ template <typename R, int NX, int NY, int NTT>
 __device__ __forceinline__ void x_split(const PlaneGeo<R, NX, NY, NTT>& G, typename SpecOf<R>::type* sm) {
   using C = typename SpecOf<R>::type;
   constexpr int MAXQ = NX ? (NX / 2 + 32) / 32 : 5;
-  constexpr int NW = (PlaneGeo<R, NX, NY, NTT>::NT + 31) / 32;
+  const int NW = (PlaneGeo<R, NX, NY, NTT>::NT > 0 ? PlaneGeo<R, NX, NY, NTT>::NT + 31
+                                                    : blockDim.x) / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int half = G.nx >> 1;
   const Axis ax{G.ax.L, G.ax.r1, G.ax.r2};
@@ -465,7 +505,8 @@ template <typename R, int NX, int NY, int NTT>
 __device__ __forceinline__ void x_merge(const PlaneGeo<R, NX, NY, NTT>& G, typename SpecOf<R>::type* sm) {
   using C = typename SpecOf<R>::type;
   constexpr int MAXQ = NX ? (NX / 2 + 32) / 32 : 5;
-  constexpr int NW = (PlaneGeo<R, NX, NY, NTT>::NT + 31) / 32;
+  const int NW = (PlaneGeo<R, NX, NY, NTT>::NT > 0 ? PlaneGeo<R, NX, NY, NTT>::NT + 31
+                                                    : blockDim.x) / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int half = G.nx >> 1;
   const Axis ax{G.ax.L, G.ax.r1, G.ax.r2};
@@ -512,7 +553,8 @@ __device__ __forceinline__ void x_merge(const PlaneGeo<R, NX, NY, NTT>& G, typen
 // lane (r2 - b) % r2 of the same group and arrive by warp shuffles.
 template <int R1, typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void xB_fwd_split_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm) {
-  constexpr int NW = (PlaneGeo<R, NX, NY, NTT>::NT + 31) / 32;
+  const int NW = (PlaneGeo<R, NX, NY, NTT>::NT > 0 ? PlaneGeo<R, NX, NY, NTT>::NT + 31
+                                                    : blockDim.x) / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp >= NW) return;
   const int r2 = G.ax.r2, rpw = 32 / r2;
@@ -586,7 +628,8 @@ __device__ __forceinline__ void xB_fwd_split_r(const PlaneGeo<R, NX, NY, NTT>& G
 // self-conjugate bins dropped), the row's lanes synchronise, then stage B'.
 template <int R1, typename R, int NX, int NY, int NTT, typename C>
 __device__ __forceinline__ void xB_inv_merge_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
-  constexpr int NW = (PlaneGeo<R, NX, NY, NTT>::NT + 31) / 32;
+  const int NW = (PlaneGeo<R, NX, NY, NTT>::NT > 0 ? PlaneGeo<R, NX, NY, NTT>::NT + 31
+                                                    : blockDim.x) / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp >= NW) return;
   const int r2 = G.ax.r2, rpw = 32 / r2;
@@ -927,7 +970,7 @@ __device__ __forceinline__ void plane_body(const GridDesc& g, const PlaneArgs<R>
   using C = typename SpecOf<R>::type;
   using CR = typename CplxOf<R>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int NTT = sizeof(R) == 8 ? plane64_threads(NX) : kThreads;
+  constexpr int NTT = NX == 0 ? 0 : (sizeof(R) == 8 ? plane64_threads(NX) : kThreads);
   const PlaneGeo<R, NX, NY, NTT> G(g);
   C* sm = reinterpret_cast<C*>(smraw);
   C* twx = sm + G.npair * G.pp;   // nx roots
@@ -991,7 +1034,7 @@ __device__ __forceinline__ void plane_body(const GridDesc& g, const PlaneArgs<R>
 }
 
 template <typename R, int NX, int NY, int MODE>
-__global__ void __launch_bounds__(launch_threads(kThreads),
+__global__ void __launch_bounds__(plane_threads<R>(NX),
                                   min_blocks(plane_smem_ct(NX, NY, sizeof(R)),
                                              sizeof(R) == 4 ? 3 : 2))
     plane_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<R>> p) {
@@ -1005,7 +1048,7 @@ __global__ void __launch_bounds__(launch_threads(kThreads),
 // (FP64: one kernel for both forms, to halve the compile time; rows null: CTA
 // row y is a state of one of the terms p.)
 template <int NX, int NY, int MODE>
-__global__ void __launch_bounds__(launch_threads(plane64_threads(NX)),
+__global__ void __launch_bounds__(plane_threads<double>(NX),
                                   min_blocks(plane_smem_ct(NX, NY, 8), 2))
     plane64_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<double>> p,
                    const PlaneArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
@@ -1016,7 +1059,7 @@ __global__ void __launch_bounds__(launch_threads(plane64_threads(NX)),
 }
 
 template <typename R, int NX, int NY, int MODE>
-__global__ void __launch_bounds__(launch_threads(kThreads),
+__global__ void __launch_bounds__(plane_threads<R>(NX),
                                   min_blocks(plane_smem_ct(NX, NY, sizeof(R)),
                                              sizeof(R) == 4 ? 3 : 2))
     plane_group_kernel(const GridDesc g, const PlaneArgs<R>* __restrict__ args,
@@ -1587,7 +1630,7 @@ __global__ void __launch_bounds__(launch_threads(task_threads(W)),
 // FP64 pencil pass, single or grouped (rows set) launches, either mode.
 template <int NZ, int W>
 __global__ void __launch_bounds__(launch_threads(task_threads(W)),
-                                  min_blocks(pencil_smem_ct(NZ, W, 8), pencil_min_ctas(NZ, 8)))
+                                  NZ ? min_blocks(pencil_smem_ct(NZ, W, 8), pencil_min_ctas(NZ, 8)) : kGenericCtas64)
     pencil64_kernel(const GridDesc g, const __grid_constant__ TermPack<PencilArgs<double>> p,
                     const PencilArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
   const int t = rows ? 0 : blockIdx.y / p.a[0].m;
@@ -1724,7 +1767,7 @@ cudaError_t plane_dispatch(const GridDesc& g, const PlaneArgs<R>* a, int n, size
     return plane64_dispatch<NX, NY>(g, a->mode, p, nullptr, nullptr, n * a->m, smem, st);
   } else {
     dim3 grid(g.nz, n * a->m);
-    const int nthr = kThreads;
+    const int nthr = NX ? kThreads : generic_threads<R>(g, smem);
     cudaError_t e;
     switch (a->mode) {
 #define ITP_PLANE_CASE(M)                                                   \
@@ -1781,6 +1824,7 @@ cudaError_t plane64_dispatch(const GridDesc& g, int mode,
                              const PlaneArgs<double>* args, const int2* rows, int nrows,
                              size_t smem, cudaStream_t st) {
   dim3 grid(g.nz, nrows);
+  const int nthr = NX ? plane_threads<double>(NX) : generic_threads<double>(g, smem);
   cudaError_t e;
   switch (mode) {
 #define ITP_PLANE64_CASE(M)                                                     \
@@ -1788,7 +1832,7 @@ cudaError_t plane64_dispatch(const GridDesc& g, int mode,
     e = set_smem(plane64_kernel<NX, NY, M>, smem);                              \
     if (e != cudaSuccess) return e;                                             \
     plane64_kernel<NX, NY, M>                                                   \
-        <<<grid, launch_threads(plane64_threads(NX)), smem, st>>>(g, p, args, rows); \
+        <<<grid, nthr, smem, st>>>(g, p, args, rows);                           \
     break;
     ITP_PLANE64_CASE(PLANE_FWD_REAL)
     ITP_PLANE64_CASE(PLANE_MERGED)
@@ -2040,13 +2084,14 @@ cudaError_t plane_group_dispatch(const GridDesc& g, int mode, const PlaneArgs<R>
                                     smem, st);
   } else {
     dim3 grid(g.nz, nrows);
+    const int nthr = NX ? kThreads : generic_threads<R>(g, smem);
     cudaError_t e;
     switch (mode) {
 #define ITP_PLANE_GROUP_CASE(M)                                             \
     case M:                                                                 \
       e = set_smem(plane_group_kernel<R, NX, NY, M>, smem);                 \
       if (e != cudaSuccess) return e;                                       \
-      plane_group_kernel<R, NX, NY, M><<<grid, kThreads, smem, st>>>(g, args, rows); \
+      plane_group_kernel<R, NX, NY, M><<<grid, nthr, smem, st>>>(g, args, rows); \
       break;
       ITP_PLANE_GROUP_CASE(PLANE_FWD_REAL)
       ITP_PLANE_GROUP_CASE(PLANE_MERGED)

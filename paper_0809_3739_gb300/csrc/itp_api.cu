@@ -285,8 +285,9 @@ void roots_table(int L, std::vector<float>& out) {
 
 // cos(2 pi j / L) * 2^61 (sine: j - L/4), rounded; by reduction to at most an
 // eighth of a turn and the Taylor series in integers with 2^-120 units, so
-// that every machine gets the same table.
-__int128 fx_cos61(int j, int L) {
+// that every machine gets the same table.  memo: the distinct values so far, one
+// table per L.
+__int128 fx_cos61(int j, int L, std::vector<__int128> (&memo)[2]) {
   j = ((j % L) + L) % L;
   if (2 * j > L) j = L - j;                       // cos(-x) = cos(x)
   bool neg = false;
@@ -294,6 +295,9 @@ __int128 fx_cos61(int j, int L) {
   const bool sine = 8 * j > L;                    // cos(x) = sin(pi/2 - x)
   // angle = 2 pi num / den with num/den <= 1/8
   const int num = sine ? L - 4 * j : j, den = sine ? 4 * L : L;
+  std::vector<__int128>& known = memo[sine ? 1 : 0];   // by num (0: not computed)
+  if (known.size() <= (size_t)num) known.resize(num + 1, 0);
+  if (known[num]) return neg ? -known[num] : known[num];
   const __int128 one = (__int128)1 << 120;
   auto mul = [](__int128 a, __int128 b) {   // a b 2^-120, 0 <= a, b <= 2^120
     const __int128 ah = a >> 60, al = a & (((__int128)1 << 60) - 1);
@@ -305,20 +309,23 @@ __int128 fx_cos61(int j, int L) {
   const __int128 x = pi4 * 8 / den * num;         // 2 pi num / den <= pi/4
   const __int128 x2 = mul(x, x);
   __int128 term = sine ? x : one, sum = term;
-  for (int k = sine ? 2 : 1; k < 40; k += 2) {
+  for (int k = sine ? 2 : 1; k < 40 && term != 0; k += 2) {
     term = -mul(term < 0 ? -term : term, x2) / (k * (k + 1)) * (term < 0 ? -1 : 1);
     sum += term;
   }
   const __int128 r = (sum + ((__int128)1 << 58)) >> 59;
+  known[num] = r;
   return neg ? -r : r;
 }
 
 void roots_table(int L, std::vector<double>& out) {
   out.resize(2 * (size_t)L);
+  std::vector<__int128> memo[2];
   for (int j = 0; j < L; ++j) {
     int w[4];
     for (int part = 0; part < 2; ++part) {
-      const __int128 v = part == 0 ? fx_cos61(4 * j, 4 * L) : -fx_cos61(4 * j - L, 4 * L);
+      const __int128 v = part == 0 ? fx_cos61(4 * j, 4 * L, memo)
+                                  : -fx_cos61(4 * j - L, 4 * L, memo);
       const __int128 h = (v + ((__int128)1 << 31)) >> 32;
       const __int128 l = v - (h << 32);
       w[2 * part] = (int)h;
