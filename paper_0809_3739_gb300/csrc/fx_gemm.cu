@@ -32,11 +32,11 @@ template <int BITS>
 __device__ __forceinline__ long long to_integer(double d, int e) {
   const long long b = __double_as_longlong(d);
   const int ex = (int)((b >> 52) & 0x7ff);
-  constexpr int kUp = 9;   // 53-bit mantissa to 62 bits: room to round
-  long long m = ((b & 0xfffffffffffffLL) | 0x10000000000000LL) << kUp;
-  const int s = fx_max(1, fx_min(e - ex + (53 + kUp - BITS), 63));   // >= 7 for finite d != 0
-  m = (m + ((1LL << s) >> 1)) >> s;
-  m = ex == 0 ? 0 : m;
+  // the 53-bit mantissa, shifted so that one more bit than wanted is left
+  constexpr int kUp = BITS + 1 - 53;
+  static_assert(kUp >= 1 && kUp <= 9, "54 to 61 bits");
+  long long m = fx_shr(((b & 0xfffffffffffffLL) | 0x10000000000000LL) << kUp, fx_max(0, e - ex));
+  m = ex == 0 ? 0 : (m + 1) >> 1;   // (the magnitude: no bias towards or from zero)
   const long long sg = b >> 63;
   return (m ^ sg) - sg;
 }
@@ -641,6 +641,162 @@ __global__ void __launch_bounds__(kApplyThreads)
   }
 }
 
+// ---------------------------------------------------------------------------
+// The update for more than kApplyMmaMin states in the digits of the tensor-
+// core Gram: a CTA multiplies 64 rows of M (its digits stay in shared memory)
+// with up to 128 states, 32 points per tile; a warp holds 16 rows x 8 points
+// in eight FP32 accumulators, exact over the 128 states, and turns each sum
+// into a double.  lower: the 16-state steps beyond a warp's rows are skipped.
+// Scaling and precision as in the integer form.
+// (One level more than the Gram, 34 digit products: a sum over few states has
+// no averaging over the grid, and without level 7 its error, about 2^-53 of
+// the largest product, was that of the FP64 form instead of below it.)
+// 57 states at 64^3 0.40 ms in integers, 128 1.44, 48 at 128^3 2.92; up to 32
+// states both forms take the same time.
+constexpr int kApplyMmaMin = 32;
+constexpr int kApplyMmaPts = 32;
+constexpr int kApplyLevels = 8;
+
+// (hi 2^72 + lo 2^40) 2^k as a double, |hi|, |lo| < 2^62.
+__device__ __forceinline__ double levels_to_double(long long hi, long long lo, int k, bool poison) {
+  return sum_to_double(hi + (lo >> 32), (long long)((unsigned)lo >> (32 - kHalf)), 0, k + 16,
+                       poison);   // which takes the two in 2^56 and 2^28
+}
+
+__device__ __forceinline__ void ldmatrix2(uint32_t (&r)[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"(addr)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(kMmaThreads, 1)
+    fx_apply_mma_kernel(const double* __restrict__ M, int m, int lower,
+                        const double* __restrict__ S, const double* __restrict__ X,
+                        double* __restrict__ Y, long long N, int k0, int nk, int rb0, int add) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int eM[kMmaRows], xs[128], eX[kMmaThreads / 32][kApplyMmaPts], sE[kApplyMmaPts];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = kMmaRows * (rb0 + blockIdx.y), nr = m - r0 < kMmaRows ? m - r0 : kMmaRows;
+  const int kk = lower ? fx_min(nk, r0 + kMmaRows - k0) : nk;   // states used, at most 128
+  const int KB = (kk + 63) / 64, K = 64 * KB, pitch = K + 8;
+  __half* sM = reinterpret_cast<__half*>(smraw);               // [digit][row][pitch]
+  __half* sX = sM + (size_t)kDigits * kMmaRows * pitch;         // [digit][point][pitch]
+  if (tid < 128) {
+    const int e = S && tid < kk ? exponent(S[(long long)(k0 + tid) * (m + 1)]) : 0;
+    xs[tid] = e > 0 && e < 2047 ? (e - 1023) >> 1 : 0;
+  }
+  __syncthreads();
+  for (int i = warp; i < kMmaRows; i += kMmaThreads / 32) {   // rows of M
+    const double* row = M + (long long)(r0 + i) * m + k0;
+    int e = kNone;
+    if (i < nr)
+      for (int k = lane; k < kk; k += 32) e = fx_max(e, scaled_exponent(row[k], xs[k]));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) eM[i] = e;
+    for (int k = 2 * lane; k < K; k += 64) {
+      const double v0 = i < nr && k < kk ? row[k] : 0.0, v1 = i < nr && k + 1 < kk ? row[k + 1] : 0.0;
+      uint32_t d[kDigits];
+      digit_pairs(to_integer<kMmaBits>(v0, e - xs[k]), to_integer<kMmaBits>(v1, e - xs[k + 1]), d);
+#pragma unroll
+      for (int l = 0; l < kDigits; ++l)
+        *reinterpret_cast<uint32_t*>(sM + ((size_t)l * kMmaRows + i) * pitch + k) = d[l];
+    }
+  }
+  const long long ntiles = (N + kApplyMmaPts - 1) / kApplyMmaPts;
+  // tile load: point = lane, states 4 warp .. + 3 of each 64
+  double v[2][4];
+  auto load = [&](long long tile) {
+    const long long p = tile * kApplyMmaPts + lane;
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int k = 64 * b + 4 * warp + q;
+        v[b][q] = (tile < ntiles && k < kk && p < N) ? X[(long long)(k0 + k) * N + p] : 0.0;
+      }
+  };
+  const int wi = 16 * (warp >> 2), wp = 8 * (warp & 3);
+  int steps = (kk + 15) / 16;   // 16-state steps of this warp's rows
+  if (lower) steps = fx_max(0, fx_min(steps, (r0 + wi + 16 - k0 + 15) / 16));
+  const uint32_t rowM = kMmaRows * pitch * 2, rowX = kApplyMmaPts * pitch * 2;   // digit strides
+  const uint32_t adA = (uint32_t)__cvta_generic_to_shared(sM) +
+                       (uint32_t)(((wi + (lane & 7) + 8 * ((lane >> 3) & 1)) * pitch +
+                                   8 * (lane >> 4)) * 2);
+  const uint32_t adB = (uint32_t)__cvta_generic_to_shared(sX) +
+                       (uint32_t)(((wp + (lane & 7)) * pitch + 8 * ((lane >> 3) & 1)) * 2);
+  load(blockIdx.x);
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    int e = kNone;
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        e = fx_max(e, scaled_exponent(v[b][q], -xs[64 * b + 4 * warp + q]));
+    eX[warp][lane] = e;
+    __syncthreads();   // the previous tile is multiplied, the exponents are here
+#pragma unroll
+    for (int w = 0; w < kMmaThreads / 32; ++w) e = fx_max(e, eX[w][lane]);
+    if (warp == 0) sE[lane] = e;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      if (b < KB) {
+        const int k = 64 * b + 4 * warp;
+        long long n[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) n[q] = to_integer<kMmaBits>(v[b][q], e + xs[k + q]);
+        uint32_t d0[kDigits], d1[kDigits];
+        digit_pairs(n[0], n[1], d0);
+        digit_pairs(n[2], n[3], d1);
+#pragma unroll
+        for (int l = 0; l < kDigits; ++l)
+          *reinterpret_cast<uint2*>(sX + ((size_t)l * kApplyMmaPts + lane) * pitch + k) =
+              make_uint2(d0[l], d1[l]);
+      }
+    }
+    load(tile + gridDim.x);   // in flight meanwhile
+    __syncthreads();
+    float acc[kApplyLevels][4];
+#pragma unroll
+    for (int l = 0; l < kApplyLevels; ++l)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[l][c] = 0.f;
+#pragma unroll 1
+    for (int s = 0; s < steps; ++s) {
+      uint32_t b[kDigits][2];
+#pragma unroll
+      for (int l = 0; l < kDigits; ++l) ldmatrix2(b[l], adB + l * rowX + 32 * s);
+#pragma unroll
+      for (int l = 0; l < kDigits; ++l) {
+        uint32_t a[4];
+        ldmatrix4(a, adA + l * rowM + 32 * s);
+#pragma unroll
+        for (int q = 0; q < kDigits && q + l < kApplyLevels; ++q)
+          mma_f16(acc[l + q], a, b[q][0], b[q][1]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = wi + (lane >> 2) + 8 * (c >> 1), pt = wp + 2 * (lane & 3) + (c & 1);
+      const long long p = tile * kApplyMmaPts + pt;
+      if (i < nr && p < N) {
+        int u[kApplyLevels];
+#pragma unroll
+        for (int l = 0; l < kApplyLevels; ++l) u[l] = __float2int_rn(acc[l][c]);
+        const long long hi =
+            fx_wide(u[0], 1 << 24, fx_wide(u[1], 1 << 16, fx_wide(u[2], 1 << 8, u[3])));
+        const long long lo =
+            fx_wide(u[4], 1 << 24, fx_wide(u[5], 1 << 16, fx_wide(u[6], 1 << 8, u[7])));
+        const int em = eM[i], ex = sE[pt];
+        const double d = levels_to_double(hi, lo, em + ex - 2 * (1022 + kMmaBits),
+                                          em == kNotFinite || ex == kNotFinite);
+        double* y = Y + (long long)(r0 + i) * N + p;
+        *y = add ? *y + d : d;
+      }
+    }
+  }
+}
+
 template <int TT>
 cudaError_t gram_launch(const double* A, const double* B, int m, long long N, long long chunk,
                         int n_chunks, double* partial, const GramBlocks& blocks, int same,
@@ -727,6 +883,27 @@ cudaError_t launch_apply_matrix(const double* M, int m, int lower, const double*
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (m > kApplyMmaMin) {
+    // Y = sum over blocks of 128 states, in stream order; each launch has a CTA
+    // row per 64 rows that the block reaches
+    const int nb = (m + kMmaRows - 1) / kMmaRows;
+    const long long ntiles = (n_points + kApplyMmaPts - 1) / kApplyMmaPts;
+    for (int k0 = 0; k0 < m; k0 += 128) {
+      const int nk = m - k0 < 128 ? m - k0 : 128, rb0 = lower ? k0 / kMmaRows : 0;
+      const int pitch = (nk > 64 ? 128 : 64) + 8;
+      const size_t smem = (size_t)kDigits * (kMmaRows + kApplyMmaPts) * pitch * 2;
+      cudaError_t e = cudaFuncSetAttribute(fx_apply_mma_kernel,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      const int per = sms / (nb - rb0) > 0 ? (sms + nb - rb0 - 1) / (nb - rb0) : 1;
+      const int grid = (int)(ntiles < per ? ntiles : per);
+      fx_apply_mma_kernel<<<dim3(grid, nb - rb0), kMmaThreads, smem, st>>>(
+          M, m, lower, S, X, Y, n_points, k0, nk, rb0, k0 > 0);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   if (m <= 16) return apply_launch<4>(M, m, lower, S, X, Y, n_points, sms, st);
   if (m <= 32) return apply_launch<8>(M, m, lower, S, X, Y, n_points, sms, st);
   if (m <= 64) return apply_launch<16>(M, m, lower, S, X, Y, n_points, sms, st);
