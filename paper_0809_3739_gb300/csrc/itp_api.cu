@@ -627,11 +627,11 @@ int orthonormalize_lane(itp_handle h);
 template <>
 int orthonormalize_lane<double>(itp_handle h) {
   Lane<double>& L = h->f64;
-  ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial(
-                                     h->acc, h->acc, h->m, h->g.n_points, h->n_chunks,
-                                     h->partial, h->st)));
+  const int chunks = gram_chunks(h->m, true, h->g.n_points, h->n_chunks);
+  ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial(h->acc, h->acc, h->m, h->g.n_points, chunks,
+                                                      h->partial, h->st)));
   ITP_LAUNCH(h, ITP_KERNEL_GRAM_REDUCE,
-             launch_gram_reduce(h->partial, h->n_chunks, h->m, h->dV, 1, h->S, h->st));
+             launch_gram_reduce(h->partial, chunks, h->m, h->dV, 1, h->S, h->st));
   ITP_LAUNCH(h, ITP_KERNEL_CHOLESKY, launch_cholesky_inverse(h->S, h->m, h->Mx, h->status, h->st));
   ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix(
                                       h->Mx, h->m, 1, h->S, h->acc, L.psi, h->g.n_points, h->st)));
@@ -702,6 +702,8 @@ int energies_lane(itp_handle h, int flags) {
     ph.phi_out = L.psi_tmp;
   }
   ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_HPSI, plane_counted<R>(h, &ph));
+  const int chunks = sizeof(R) == 4 ? h->n_chunks_tc
+                                    : gram_chunks(h->m, false, g.n_points, h->n_chunks);
   if (sizeof(R) == 4) {
     ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_tc_gram(
                                        reinterpret_cast<const float*>(L.psi),
@@ -711,9 +713,8 @@ int energies_lane(itp_handle h, int flags) {
   } else {
     ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial(
                                        reinterpret_cast<const double*>(L.psi), h->acc, h->m,
-                                       g.n_points, h->n_chunks, h->partial, h->st)));
+                                       g.n_points, chunks, h->partial, h->st)));
   }
-  const int chunks = sizeof(R) == 4 ? h->n_chunks_tc : h->n_chunks;
   ITP_LAUNCH(h, ITP_KERNEL_GRAM_REDUCE,
              launch_gram_reduce(h->partial, chunks, h->m, h->dV, 1, h->Hs, h->st));
   if (flags & ITP_RITZ) {

@@ -74,9 +74,7 @@ extern "C" int itp_orthonormalize_noalloc(const double* phi_device, double* psi_
   using namespace itp;
   // fewer states leave room for more partial sums, up to two CTAs per SM
   const int room = (int)(kPartialDoubles / ((size_t)m * m));
-  int chunks = room < 304 ? room : 304;
-  const int nb = (m + 63) / 64, blocks = nb * (nb + 1) / 2;   // CTAs per chunk: whole waves
-  if (chunks * blocks > 152) chunks = chunks * blocks / 152 * 152 / blocks;
+  const int chunks = gram_chunks(m, true, n_points, room < 304 ? room : 304);
   if (launch_gram_partial(phi_device, phi_device, m, n_points, chunks, partial, st) != cudaSuccess ||
       launch_gram_reduce(partial, chunks, m, dV, 1, S, st) != cudaSuccess ||
       launch_cholesky_inverse(S, m, Minv, status, st) != cudaSuccess ||
