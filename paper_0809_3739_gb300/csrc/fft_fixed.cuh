@@ -2,7 +2,8 @@
 //
 // A GB300 SM issues one FP64 instruction per sub-partition and about 78
 // cycles, but a 64-bit integer add takes 2 cycles and a 32 x 32 + 64-bit
-// multiply-add (IMAD.WIDE) 2 as well (measured with chains of independent
+// multiply-add (IMAD.WIDE) 2 in a chain and 3.2 with general operands, a
+// shift or a bit operation 2 (measured with chains of independent
 // instructions at 8 warps per sub-partition).  The passes are bound by that
 // FP64 rate alone, so their transforms run in integers instead: the values
 // that one thread transforms together (a vector of up to 16 complex numbers)

@@ -1,15 +1,20 @@
-// FP64 contractions over the grid in integer arithmetic: the overlap and the
-// subspace matrix (Gram), and the update by an m x m matrix.
+// FP64 contractions over the grid: the overlap and the subspace matrix (Gram),
+// and the update by an m x m matrix.
 //
 // The FP64 form of these kernels was bound by the FP64 pipe, one instruction
 // per 78 cycles and sub-partition (128 states at 128^3: 65 ms per Gram matrix,
 // 58 ms per update, and the Gram computed 128 x 128 products however few the
-// states).  A 32 x 32 + 64-bit integer multiply-add (IMAD.WIDE) issues every
-// 2 cycles.  So the operands are scaled to integers of 55 or 56 bits, split
-// into two signed halves v = h 2^28 + l, and a product takes
+// states).  So the operands are scaled to integers of 55 or 56 bits.
+//
+// Up to 32 states they are split into two signed halves v = h 2^28 + l, and a
+// product takes
 //   Gram:   h h', and h l' + l h' (l l' is below the precision, see there);
 //   update: h h', h l' + l h', and l l',
-// accumulated exactly in 64-bit integers over up to 512 terms.
+// accumulated exactly in 64-bit integers over up to 512 terms: a 32 x 32 + 64-
+// bit multiply-add (IMAD.WIDE) issues every 3.2 cycles with general operands
+// (every 2 in a chain).  More states have enough products per element to pay
+// for splitting it into base-256 digits: the tensor cores multiply those
+// exactly (128 states at 64^3, an eighth of those points: 0.98 and 0.81 ms).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -22,7 +27,6 @@ namespace itp {
 namespace {
 
 constexpr int kMaxM = 256;   // states of the n x n work at most
-constexpr int kBlk = 128;    // rows of one state block of the update
 constexpr int kHalf = 28;    // bits of the lower half
 constexpr int kSms = 152;    // SMs of a GB300
 
@@ -92,12 +96,11 @@ __device__ __forceinline__ void load_pairs(const int2* p, int2 (&v)[N]) {
 
 // ---------------------------------------------------------------------------
 // Gram partial sums P[c][i][j] = sum over the points p of chunk c of
-// A[i][p] B[j][p].  The result is cut into blocks of 16 TT rows and columns;
-// a CTA of 16 x 16 threads sums one block over one chunk, TT x TT entries per
-// thread (TT up to 4: 64 x 64 blocks, so that few states do not pay for
-// 128).  A chunk is walked in runs of kRun points: the run's largest
-// exponent of every row first (the reads bring the run into L2), then tiles
-// of kTile points converted into shared memory as halves, [point][row].
+// A[i][p] B[j][p], up to 16 TT states (one: A and B are the same).  A CTA of
+// 16 x 16 threads sums one chunk, TT x TT entries per thread.  A chunk is
+// walked in runs of kRun points: the run's largest exponent of every row first
+// (the reads bring the run into L2), then tiles of kTile points converted into
+// shared memory as halves, [point][row].
 //
 // Precision: with the row's largest value in the run scaled to 2^54, an
 // element is off by at most 2^-55 of it and the missing l l' by about 2^-56
@@ -111,27 +114,16 @@ constexpr int kGramBits = 54;
 // 0.019 here, 0.037 there.
 constexpr int kGramMmaMin = 32;
 
-// (bi, bj) of the blocks, packed as bi * 256 + bj.
-struct GramBlocks {
-  int n;
-  short ij[64];
-};
-
 template <int TT>
-__global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
+__global__ void __launch_bounds__(256, 3)
     fx_gram_kernel(const double* __restrict__ A, const double* __restrict__ B, int m, long long N,
-                   long long chunk, double* __restrict__ partial, const GramBlocks blocks,
-                   int same) {
-  constexpr int ROWS = 16 * TT;            // rows of a block
+                   long long chunk, double* __restrict__ partial, int one) {
+  constexpr int ROWS = 16 * TT;            // rows of a tile
   constexpr int PITCH = ROWS + 2;          // 16-byte rows of pairs, few bank conflicts
-  constexpr int PER = ROWS * kTile / 256;  // elements per thread and operand tile (TT)
   __shared__ __align__(16) int2 sA[2][kTile][PITCH];   // two tiles: one barrier per tile
   __shared__ __align__(16) int2 sB[2][kTile][PITCH];
   __shared__ int eA[ROWS], eB[ROWS];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
-  const int bi = blocks.ij[blockIdx.y] >> 8, bj = blocks.ij[blockIdx.y] & 255;
-  const bool one = same && bi == bj;       // a diagonal block: one operand
-  const int ia = ROWS * bi, jb = ROWS * bj;
   const long long p_begin = (long long)blockIdx.x * chunk;
   const long long p_end = p_begin + chunk < N ? p_begin + chunk : N;
   double* out = partial + (long long)blockIdx.x * m * m;
@@ -140,22 +132,21 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
     if (i >= m || j >= m) return;
     if (!first) v += out[i * m + j];
     out[i * m + j] = v;
-    if (same && bi != bj) out[j * m + i] = v;
   };
   if (p_begin >= p_end) {
 #pragma unroll
     for (int q = 0; q < TT; ++q)
 #pragma unroll
-      for (int r = 0; r < TT; ++r) add_sum(ia + ty * TT + q, jb + tx * TT + r, 0.0, true);
+      for (int r = 0; r < TT; ++r) add_sum(ty * TT + q, tx * TT + r, 0.0, true);
   }
 
   // element q of this thread's share of a tile: point tx, row ty + 16 q
-  auto load = [&](const double* X, int r0, long long p0, long long pe, double (&v)[PER]) {
+  auto load = [&](const double* X, long long p0, long long pe, double (&v)[TT]) {
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
+    for (int q = 0; q < TT; ++q) {
       const int i = ty + 16 * q;
       const long long p = p0 + tx;
-      v[q] = (r0 + i < m && p < pe) ? X[(long long)(r0 + i) * N + p] : 0.0;
+      v[q] = (i < m && p < pe) ? X[(long long)i * N + p] : 0.0;
     }
   };
   for (long long run = p_begin; run < p_end; run += kRun) {
@@ -163,11 +154,10 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
     // largest exponents, one warp per row
     for (int op = 0; op < (one ? 1 : 2); ++op) {
       const double* X = op == 0 ? A : B;
-      const int r0 = op == 0 ? ia : jb;
       for (int i = warp; i < ROWS; i += 8) {
         int e = 0;
-        if (r0 + i < m) {
-          const double* row = X + (long long)(r0 + i) * N + run;
+        if (i < m) {
+          const double* row = X + (long long)i * N + run;
 #pragma unroll 8
           for (int k = lane; k < (int)(re - run); k += 32) e = fx_max(e, exponent(row[k]));
         }
@@ -181,12 +171,12 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
     for (int q = 0; q < TT; ++q)
 #pragma unroll
       for (int r = 0; r < TT; ++r) hh[q][r] = hl[q][r] = 0;
-    double va[PER], vb[PER];
-    load(A, ia, run, re, va);
-    if (!one) load(B, jb, run, re, vb);
+    double va[TT], vb[TT];
+    load(A, run, re, va);
+    if (!one) load(B, run, re, vb);
     auto store = [&](int buf) {
 #pragma unroll
-      for (int q = 0; q < PER; ++q) {
+      for (int q = 0; q < TT; ++q) {
         const int i = ty + 16 * q;
         sA[buf][tx][i] = to_halves<kGramBits>(va[q], eA[i]);
         if (!one) sB[buf][tx][i] = to_halves<kGramBits>(vb[q], eB[i]);
@@ -198,8 +188,8 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
       const bool more = t + 1 < ntile;
       if (more) {   // the next tile's loads are in flight meanwhile
         const long long p0 = run + (long long)(t + 1) * kTile;
-        load(A, ia, p0, re, va);
-        if (!one) load(B, jb, p0, re, vb);
+        load(A, p0, re, va);
+        if (!one) load(B, p0, re, vb);
       }
       __syncthreads();
       const int2(*tA)[PITCH] = sA[t & 1];
@@ -245,7 +235,7 @@ __global__ void __launch_bounds__(256, TT >= 3 ? 2 : 3)
         const double s = fma((double)hh[q][r], (double)(1LL << kHalf), (double)hl[q][r]);
         double v = scale2(s, ea + eb - 2 * (1022 + kGramBits) + kHalf);
         if (ea == 2047 || eb == 2047) v = __longlong_as_double(0x7ff8000000000000LL);
-        add_sum(ia + ty * TT + q, jb + tx * TT + r, v, run == p_begin);
+        add_sum(ty * TT + q, tx * TT + r, v, run == p_begin);
       }
     }
     __syncthreads();   // the exponents are rewritten by the next run
@@ -314,6 +304,12 @@ __device__ __forceinline__ void digit_pairs(long long v0, long long v1, uint32_t
   d[5] = digits_f16(__byte_perm(l0, l1, 0x0501), 0x00ff00ffu);
   d[6] = digits_f16(__byte_perm(l0, l1, 0x0400), 0x00ff00ffu);
 }
+
+// (bi, bj) of the blocks, packed as bi * 256 + bj.
+struct GramBlocks {
+  int n;
+  short ij[64];
+};
 
 __global__ void __launch_bounds__(kMmaThreads, 1)
     fx_gram_mma_kernel(const double* __restrict__ A, const double* __restrict__ B, int m,
@@ -464,18 +460,15 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// Y[r0 + i] (=|+=) sum_k M[r0 + i][k0 + k] X[k0 + k] for i < nr, k < nk (both
-// <= 4 RG): one block of Y = M X.  Persistent CTAs of 512 threads over tiles
-// of PT = 1024 / RG points.  State k is scaled by the power of two nearest
-// to its norm, from the diagonal of its overlap matrix S (null: all states of
-// norm one), and column k of M by the inverse; the rows of that M, scaled by
-// their largest entry to 55 bits, stay in shared memory as halves [k][i]; a
-// tile of X, each point scaled by its largest value over the states, comes
-// as halves [k][point] into one of two buffers while the other one is
+// Y[i] = sum_k M[i][k] X[k], up to 4 RG states.  Persistent CTAs of 512
+// threads over tiles of PT = 1024 / RG points.  State k is scaled by the power
+// of two nearest to its norm, from the diagonal of its overlap matrix S (null:
+// all states of norm one), and column k of M by the inverse; the rows of that
+// M, scaled by their largest entry to 55 bits, stay in shared memory as halves
+// [k][i]; a tile of X, each point scaled by its largest value over the states,
+// comes as halves [k][point] into one of two buffers while the other one is
 // multiplied (one barrier per tile).  A thread holds 4 rows x 2 points.
-// lower: M[i][k] = 0 for k > i (global indices), so a row group stops there;
-// the four warps that share a sub-partition take row groups that add up to
-// the same work.
+// lower: M[i][k] = 0 for k > i, so a row group stops there.
 //
 // Precision: products are exact in 110 bits, so a sum is off by the rounding
 // of its operands, 2^-56 of the largest |M_ik| times the point's largest
@@ -512,14 +505,13 @@ __device__ __forceinline__ double sum_to_double(long long hh, long long hl, long
 template <int RG>
 __global__ void __launch_bounds__(kApplyThreads)
     fx_apply_kernel(const double* __restrict__ M, int m, int lower, const double* __restrict__ S,
-                    const double* __restrict__ X, double* __restrict__ Y, long long N, int r0,
-                    int nr, int k0, int nk, int add) {
+                    const double* __restrict__ X, double* __restrict__ Y, long long N) {
   constexpr int NP = 2;                           // points per thread
   constexpr int ROWS = 4 * RG, TX = kApplyThreads / RG, PT = NP * TX;
   constexpr int MP = ROWS + 2;                    // pitch of sM (16-byte rows)
   constexpr int STEP = kApplyThreads / PT;        // threads per point of a tile load
   constexpr int PER = ROWS / STEP;
-  static_assert(PT <= 256 && STEP >= 2, "four to thirty-two row groups");
+  static_assert(PT <= 256 && STEP >= 2, "four row groups at least");
   extern __shared__ __align__(16) unsigned char smraw[];
   int2* sM = reinterpret_cast<int2*>(smraw);      // [ROWS k][MP]
   int2* sX = sM + ROWS * MP;                      // [2][ROWS k][PT]
@@ -528,29 +520,21 @@ __global__ void __launch_bounds__(kApplyThreads)
   int* eX = xs + ROWS;                            // [3][STEP][PT]: tile t in slot t % 3, as
                                                   // slower warps still read tile t - 1's
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // thread -> (row group, point).  Warps w, w + 4, w + 8, w + 12 share a
-  // sub-partition: every other group of four warps is taken in reverse.
-  constexpr int WPG = TX >= 32 ? TX / 32 : 1;     // warps per row group
-  const int wr = (warp & 4) ? (warp ^ 3) : warp;
-  const int vt = TX > 32 ? tid : wr * 32 + lane;  // (row groups wider than a warp: as they come)
-  const int ty = vt / TX, tx = vt - ty * TX;
-  (void)WPG;
+  const int ty = tid / TX, tx = tid - ty * TX;    // row group, point
   for (int k = tid; k < ROWS; k += kApplyThreads) {
-    const int e = S && k < nk ? exponent(S[(long long)(k0 + k) * (m + 1)]) : 0;
+    const int e = S && k < m ? exponent(S[(long long)k * (m + 1)]) : 0;
     xs[k] = e > 0 && e < 2047 ? (e - 1023) >> 1 : 0;
   }
   __syncthreads();
   for (int i = warp; i < ROWS; i += kApplyThreads / 32) {
     int e = kNone;
-    if (i < nr)
-      for (int k = lane; k < nk; k += 32)
-        e = fx_max(e, scaled_exponent(M[(long long)(r0 + i) * m + k0 + k], xs[k]));
+    if (i < m)
+      for (int k = lane; k < m; k += 32) e = fx_max(e, scaled_exponent(M[i * m + k], xs[k]));
     e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0) eM[i] = e;
     for (int k = lane; k < ROWS; k += 32)
-      sM[k * MP + i] = i < nr && k < nk
-                           ? to_halves<kApplyBits>(M[(long long)(r0 + i) * m + k0 + k], e - xs[k])
-                           : make_int2(0, 0);
+      sM[k * MP + i] = i < m && k < m ? to_halves<kApplyBits>(M[i * m + k], e - xs[k])
+                                      : make_int2(0, 0);
   }
   const long long ntiles = (N + PT - 1) / PT;
   const int lp = tid & (PT - 1), lk = tid / PT;   // tile load: point, first state
@@ -560,7 +544,7 @@ __global__ void __launch_bounds__(kApplyThreads)
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       const int k = lk + STEP * q;
-      v[q] = (tile < ntiles && k < nk && p < N) ? X[(long long)(k0 + k) * N + p] : 0.0;
+      v[q] = (tile < ntiles && k < m && p < N) ? X[(long long)k * N + p] : 0.0;
     }
   };
   auto put_exponent = [&](int slot) {
@@ -587,7 +571,7 @@ __global__ void __launch_bounds__(kApplyThreads)
   __syncthreads();
   convert(0, 0);
   load((long long)blockIdx.x + gridDim.x);
-  const int kmax = lower ? fx_max(0, fx_min(nk, r0 + 4 * ty + 4 - k0)) : nk;
+  const int kmax = lower ? fx_min(m, 4 * ty + 4) : m;
   int buf = 0, slot = 0;
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int next = slot == 2 ? 0 : slot + 1;
@@ -610,7 +594,7 @@ __global__ void __launch_bounds__(kApplyThreads)
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int r = 0; r < NP; ++r) {   // 128 terms: <= 2^61, 2^62, 2^61
+        for (int r = 0; r < NP; ++r) {   // (128 terms would be <= 2^61, 2^62, 2^61)
           hh[q][r] = fx_wide(a[q].x, b[r].x, hh[q][r]);
           hl[q][r] = fx_wide(a[q].x, b[r].y, hl[q][r]);
           ll[q][r] = fx_wide(a[q].y, b[r].y, ll[q][r]);
@@ -628,13 +612,12 @@ __global__ void __launch_bounds__(kApplyThreads)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int i = 4 * ty + q;
-        if (i >= nr) continue;
+        if (i >= m) continue;
         const int em = eM[i];
         const double d = sum_to_double(hh[q][r], hl[q][r], ll[q][r],
                                        em + ex - 2 * (1022 + kApplyBits),
                                        em == kNotFinite || ex == kNotFinite);
-        double* y = Y + (long long)(r0 + i) * N + p;
-        *y = add ? *y + d : d;
+        Y[(long long)i * N + p] = d;
       }
     }
     buf ^= 1;
@@ -798,15 +781,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
   }
 }
 
-template <int TT>
-cudaError_t gram_launch(const double* A, const double* B, int m, long long N, long long chunk,
-                        int n_chunks, double* partial, const GramBlocks& blocks, int same,
-                        cudaStream_t st) {
-  fx_gram_kernel<TT><<<dim3(n_chunks, blocks.n), 256, 0, st>>>(A, B, m, N, chunk, partial, blocks,
-                                                              same);
-  return cudaGetLastError();
-}
-
 template <int RG>
 cudaError_t apply_launch(const double* M, int m, int lower, const double* S, const double* X,
                          double* Y, long long N, int sms, cudaStream_t st) {
@@ -816,20 +790,10 @@ cudaError_t apply_launch(const double* M, int m, int lower, const double* S, con
   cudaError_t e = cudaFuncSetAttribute(fx_apply_kernel<RG>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const long long ntiles = (N + PT - 1) / PT, cap = (long long)sms * (RG == 32 ? 1 : 2);
+  const long long ntiles = (N + PT - 1) / PT, cap = 2LL * sms;
   const int grid = (int)(ntiles < cap ? ntiles : cap);
-  // Y block bi = sum over bk of M[bi][bk] X[bk] (bk <= bi when lower), in
-  // stream order: the first block product sets Y[bi], the others add to it
-  for (int r0 = 0; r0 < m; r0 += kBlk) {
-    const int nr = m - r0 < kBlk ? m - r0 : kBlk;
-    for (int k0 = 0; k0 < m && (!lower || k0 <= r0 + nr - 1); k0 += kBlk) {
-      const int nk = m - k0 < kBlk ? m - k0 : kBlk;
-      fx_apply_kernel<RG><<<grid, kApplyThreads, smem, st>>>(M, m, lower, S, X, Y, N, r0, nr, k0, nk, k0 > 0);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return cudaSuccess;
+  fx_apply_kernel<RG><<<grid, kApplyThreads, smem, st>>>(M, m, lower, S, X, Y, N);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -853,12 +817,10 @@ cudaError_t launch_gram_partial(const double* A, const double* B, int m, long lo
   if (m < 1 || m > kMaxM) return cudaErrorInvalidValue;
   long long chunk = (n_points + n_chunks - 1) / n_chunks;
   chunk = (chunk + kTile - 1) / kTile * kTile;
-  // blocks of at most 64 rows, as few as that takes and then as small; A A^T:
-  // the lower blocks, mirrored.  Smaller blocks where that leaves SMs idle
-  // (few chunks: a caller's scratch limits them).
-  const bool same = A == B;
-  GramBlocks blocks{};
   if (m > kGramMmaMin) {
+    // A A^T: the lower blocks, mirrored
+    const bool same = A == B;
+    GramBlocks blocks{};
     const int nb = (m + kMmaRows - 1) / kMmaRows;
     chunk = (chunk + kMmaTile - 1) / kMmaTile * kMmaTile;
     for (int bi = 0; bi < nb; ++bi)
@@ -872,24 +834,11 @@ cudaError_t launch_gram_partial(const double* A, const double* B, int m, long lo
         A, B, m, n_points, chunk, partial, blocks, same);
     return cudaGetLastError();
   }
-  int tt = 4;
-  for (int cap = 64; cap >= 32; cap -= 16) {
-    const int nb = (m + cap - 1) / cap;
-    tt = (m + 16 * nb - 1) / (16 * nb);
-    blocks.n = same ? nb * (nb + 1) / 2 : nb * nb;
-    if (blocks.n * (long long)n_chunks >= 304) break;
-  }
-  const int nb = (m + 16 * tt - 1) / (16 * tt);
-  blocks.n = 0;
-  for (int bi = 0; bi < nb; ++bi)
-    for (int bj = 0; bj < nb; ++bj)
-      if (!same || bj <= bi) blocks.ij[blocks.n++] = (short)(bi * 256 + bj);
-  switch (tt) {
-    case 1: return gram_launch<1>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
-    case 2: return gram_launch<2>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
-    case 3: return gram_launch<3>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
-    default: return gram_launch<4>(A, B, m, n_points, chunk, n_chunks, partial, blocks, same, st);
-  }
+  if (m <= 16)
+    fx_gram_kernel<1><<<n_chunks, 256, 0, st>>>(A, B, m, n_points, chunk, partial, A == B);
+  else
+    fx_gram_kernel<2><<<n_chunks, 256, 0, st>>>(A, B, m, n_points, chunk, partial, A == B);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_apply_matrix(const double* M, int m, int lower, const double* S,
@@ -920,9 +869,7 @@ cudaError_t launch_apply_matrix(const double* M, int m, int lower, const double*
     return cudaSuccess;
   }
   if (m <= 16) return apply_launch<4>(M, m, lower, S, X, Y, n_points, sms, st);
-  if (m <= 32) return apply_launch<8>(M, m, lower, S, X, Y, n_points, sms, st);
-  if (m <= 64) return apply_launch<16>(M, m, lower, S, X, Y, n_points, sms, st);
-  return apply_launch<32>(M, m, lower, S, X, Y, n_points, sms, st);
+  return apply_launch<8>(M, m, lower, S, X, Y, n_points, sms, st);
 }
 
 }  // namespace itp
