@@ -5,6 +5,7 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include "fx_scalar.cuh"
 #include "itp_kernels.cuh"
 
 namespace cg = cooperative_groups;
@@ -56,19 +57,6 @@ constexpr int kClus = 8;            // CTAs per cluster (portable size)
 constexpr int kClusThreads = 256;   // Cholesky: a panel row per thread
 constexpr int kClusMinM = 28;       // from this m on the cluster is faster (24: even, 32: 10 %)
 constexpr int kPanel = 8;           // columns per Cholesky panel
-
-// 1/d for a finite d > 0: a single-precision seed and one third-order step,
-// three dependent FP64 instructions.
-__device__ __forceinline__ double recip(double d) {
-  const long long b = __double_as_longlong(d);
-  const int e = (int)(b >> 52) - 1023;   // d = f 2^e, 1 <= f < 2
-  if (e < -1000 || e > 1000) return 1.0 / d;
-  const double f = __longlong_as_double((b & 0xfffffffffffffLL) | 0x3ff0000000000000LL);
-  const double y = (double)(1.0f / (float)f);
-  const double r = fma(-f, y, 1.0);
-  const double z = fma(y, fma(r, r, r), y);   // in (1/2, 1]
-  return __longlong_as_double(__double_as_longlong(z) - ((long long)e << 52));
-}
 
 // Cholesky S = L L^T and M = L^{-1}, in the form S = U D U^T (U unit lower
 // triangular, D = diag d): M = D^{-1/2} U^{-1}, so that no square root lies on
@@ -147,7 +135,7 @@ __global__ void __launch_bounds__(kClusThreads)
       const double d = s_col[tid][tid];
       const bool ok = d > 0.0 && isfinite(d);
       if (!ok) s_bad = 1;
-      s_rs[tid] = ok ? 1.0 / sqrt(d) : 1.0;
+      s_rs[tid] = ok ? rsqrt64(d) : 1.0;
     }
     for (int j = tid; j < k0 + w; j += NT) {
       double x[kPanel];
@@ -191,18 +179,6 @@ __global__ void __launch_bounds__(kClusThreads)
   }
   if (tid == 0 && s_bad) atomicOr(status, 1);
   if (nr > 1) cl.sync();   // no CTA leaves while another may still read its shared memory
-}
-
-// 1/sqrt(a) for 2^-1000 < a < 2^1000: a single-precision seed and one
-// third-order step.
-__device__ __forceinline__ double rsqrt64(double a) {
-  const long long b = __double_as_longlong(a);
-  const int e = ((int)(b >> 52) - 1023) & ~1;   // a = f 2^e, e even, 1 <= f < 4
-  const double f = __longlong_as_double(b - ((long long)e << 52));
-  const double y = (double)rsqrtf((float)f);
-  const double r = fma(-f * y, y, 1.0);
-  const double z = fma(y * r, fma(0.375, r, 0.5), y);   // y (1 + r/2 + 3 r^2/8)
-  return __longlong_as_double(__double_as_longlong(z) - ((long long)(e / 2) << 52));
 }
 
 // Householder tridiagonalisation (eigenvalues only).  An FP64 operation costs
@@ -259,24 +235,22 @@ __global__ void __launch_bounds__(kTriThreads)
     double* Yb = Y + b * m;
     double* Cb = C + b * m;
     if (warp == NW - 1) {   // the reflector
+      const double x0 = x[n0];
       double s = 0.0;
       for (int j = n0 + 1 + lane; j < m; j += 32) s = fma(x[j], x[j], s);
-      s = warp_sum(s, 32);
+      const bool any = __any_sync(0xffffffffu, s != 0.0);
+      if (lane == 31) s = fma(x0, x0, s);
+      long long t;
+      int ex;
+      const bool fast = fx_warp_sum(s, &t, &ex) && ex > 100;
+      if (!fast) s = warp_sum(s, 32);
       if (lane == 0) {
-        const double x0 = x[n0], s2 = fma(x0, x0, s);
         double alpha = x0, beta = 0.0, v0 = 0.0;
-        if (s != 0.0) {
-          double nrm;
-          const int ex = (__double2hiint(s2) >> 20) & 0x7ff;
-          if (ex > 100 && ex < 1900) {
-            const double z = rsqrt64(s2);
-            nrm = s2 * z;
-            nrm = fma(0.5 * z, fma(-nrm, nrm, s2), nrm);
-            beta = recip(fma(fabs(x0), nrm, s2));   // 2 / v^T v = 1 / (|x|^2 + |x_0| |x|)
-          } else {
-            nrm = sqrt(s2);
-            beta = 1.0 / fma(fabs(x0), nrm, s2);
-          }
+        if (any && fast) {
+          fx_reflector(fx_normal((unsigned long long)t, ex - 1079), x0, &alpha, &beta, &v0);
+        } else if (any) {
+          const double nrm = sqrt(s);
+          beta = 1.0 / fma(fabs(x0), nrm, s);
           alpha = x0 > 0 ? -nrm : nrm;
           v0 = x0 - alpha;
         }
@@ -332,7 +306,7 @@ __global__ void __launch_bounds__(kTriThreads)
     const double y1 = Yb[n0], c1 = Cb[n0];
     const double hb = 0.5 * beta * beta, rest = alpha * fma(alpha, c1, -2.0 * y1);
     const double p1 = beta * fma(-alpha, c1, y1);
-    xy = warp_sum(xy, 32);
+    xy = warp_sum64(xy);
     const double K = hb * (xy + rest);
     const double w1 = fma(-K, v0, p1);
     double* xn = xf + (b ^ 1) * m;
