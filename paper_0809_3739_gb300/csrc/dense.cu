@@ -17,34 +17,41 @@ namespace {
 constexpr int kMaxM = 256;   // states of the n x n work at most
 
 // ---------------------------------------------------------------------------
-// G = scale * the sum of the chunks' partial sums: 32 entries per CTA, eight
-// warps over the chunks (one thread per entry walked all of them, a chain of
-// up to 608 dependent FP64 additions, 78 cycles each).
+// G = scale * the sum of the chunks' partial sums: E entries per CTA, 256 / E
+// slots over the chunks, the slots' sums added in integers.  It is bound by
+// FP64 additions, 78 cycles of a sub-partition each, so few states (few
+// entries) are spread over many CTAs: 10 and 24 states with 304 chunks 20 us
+// with 32 entries per CTA, 6 with four; 57 13 and 7; 89 and 128 (152 chunks) 7
+// and 9 either way, with the fewer CTAs.
+constexpr int kReduceFewM = 64;
+template <int E>
 __global__ void __launch_bounds__(256) gram_reduce_kernel(const double* __restrict__ partial,
                                                           int n_chunks, int m, double scale,
                                                           int sym, double* __restrict__ G) {
-  __shared__ double ss[8][32], st[8][32];
+  constexpr int kSlots = 256 / E;
+  __shared__ double ss[E][kSlots + 1];
+  const int el = threadIdx.x % E, slot = threadIdx.x / E;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int e = blockIdx.x * 32 + lane;
+  const int e = blockIdx.x * E + el;
   double s = 0.0, t = 0.0;
   if (e < m * m) {
     const int i = e / m, j = e - i * m;
     const double* p = partial + e;
     const double* q = partial + j * m + i;
-    for (int c = warp; c < n_chunks; c += 8) {
+#pragma unroll 4
+    for (int c = slot; c < n_chunks; c += kSlots) {
       s += p[(long long)c * m * m];
       if (sym) t += q[(long long)c * m * m];
     }
   }
-  ss[warp][lane] = s;
-  st[warp][lane] = t;
+  ss[el][slot] = sym ? s + t : s;
   __syncthreads();
-  if (warp == 0 && e < m * m) {
-    for (int w = 1; w < 8; ++w) {
-      s += ss[w][lane];
-      t += st[w][lane];
-    }
-    G[e] = sym ? 0.5 * scale * (s + t) : scale * s;
+  for (int k = warp; k < E; k += 8) {
+    double v = 0.0;
+    for (int c = lane; c < kSlots; c += 32) v += ss[k][c];
+    v = warp_sum64(v);
+    const int o = blockIdx.x * E + k;
+    if (lane == 0 && o < m * m) G[o] = (sym ? 0.5 * scale : scale) * v;
   }
 }
 
@@ -688,7 +695,10 @@ __global__ void convert_kernel(const TS* __restrict__ src, TD* __restrict__ dst,
 
 cudaError_t launch_gram_reduce(const double* partial, int n_chunks, int m, double scale, int sym,
                                double* G, cudaStream_t st) {
-  gram_reduce_kernel<<<(m * m + 31) / 32, 256, 0, st>>>(partial, n_chunks, m, scale, sym, G);
+  if (m <= kReduceFewM)
+    gram_reduce_kernel<4><<<(m * m + 3) / 4, 256, 0, st>>>(partial, n_chunks, m, scale, sym, G);
+  else
+    gram_reduce_kernel<32><<<(m * m + 31) / 32, 256, 0, st>>>(partial, n_chunks, m, scale, sym, G);
   return cudaGetLastError();
 }
 
