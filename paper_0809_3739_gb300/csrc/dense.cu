@@ -65,6 +65,12 @@ constexpr int kClusThreads = 256;   // Cholesky: a panel row per thread
 constexpr int kClusMinM = 28;       // from this m on the cluster is faster (24: even, 32: 10 %)
 constexpr int kPanel = 8;           // columns per Cholesky panel
 
+// d > 0 and finite, on the bits (a comparison of doubles takes the FP64 unit)
+__device__ __forceinline__ bool is_pivot(double d) {
+  const long long b = __double_as_longlong(d);
+  return b > 0 && b < 0x7ff0000000000000LL;
+}
+
 // Cholesky S = L L^T and M = L^{-1}, in the form S = U D U^T (U unit lower
 // triangular, D = diag d): M = D^{-1/2} U^{-1}, so that no square root lies on
 // the chain from pivot to pivot.  Right-looking in panels of kPanel columns:
@@ -126,7 +132,7 @@ __global__ void __launch_bounds__(kClusThreads)
         __syncthreads();
         if (i > k0 + c && i < m) {
           double d = s_col[c][c];
-          if (!(d > 0.0) || !isfinite(d)) d = 1.0;
+          if (!is_pivot(d)) d = 1.0;
           const double u = a[c] * recip(d);
           U[i * UP + c] = u;
           Ac[i * UP + c] = a[c];
@@ -140,7 +146,7 @@ __global__ void __launch_bounds__(kClusThreads)
     // the panel's own rows of R, a column per thread; 1/sqrt(d) meanwhile
     if (tid < w) {
       const double d = s_col[tid][tid];
-      const bool ok = d > 0.0 && isfinite(d);
+      const bool ok = is_pivot(d);
       if (!ok) s_bad = 1;
       s_rs[tid] = ok ? rsqrt64(d) : 1.0;
     }
@@ -196,22 +202,25 @@ __global__ void __launch_bounds__(kClusThreads)
 //   the groups form y = A x for their rows and publish y and their entries C
 //   of column k + 1 to all CTAs, while the last warp forms the reflector
 //   v = x - alpha e_1, beta = 2 / v^T v from x; (cluster) barrier;
-//   A v = y - alpha C, so p = beta (y - alpha C), K = beta/2 v^T p =
-//   beta^2/2 (x^T y - 2 alpha y_1 + alpha^2 C_1) and w = p - K v follow from
-//   one dot product, and so does the next column, C - v w_1 - w v_1, in every
-//   CTA alike; block barrier;
+//   A v = y - alpha C, so p = beta (y - alpha C), K = beta/2 v^T p and w = p -
+//   K v follow from one dot product, and so does the next column, C - v w_1 -
+//   w v_1, in every CTA alike; block barrier;
 //   the groups apply A -= v w^T + w v^T to their rows and in the same pass form
 //   the next y.
-// (The form with two cluster barriers, five block barriers and 256 threads took
-// 5.4 us per step; tridiagonalisation and bisection of 57 states 0.34 -> 0.23
-// ms, of 24 0.13 -> 0.10, of 128 0.92 -> 0.67.)
+// Every warp forms p and its sum itself and a thread keeps its own entry: the
+// count of FP64 instructions per warp (78 cycles each) and the length of the
+// chain decide alike.  (The form with two cluster barriers, five block barriers
+// and 256 threads took 5.4 us per step; now 24 states take 47 us, 57 122, 89
+// 222 and 128 459; with FP64 scalars and warp sums and the dot product x^T y
+// 24 states took 55 and 57 states 144 us.  From 128 states on the product y
+// takes most of a step.)
 template <int kTriThreads>
 __global__ void __launch_bounds__(kTriThreads)
     tridiag_kernel(const double* __restrict__ H, int m, double* __restrict__ d,
                    double* __restrict__ e) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ double csh[];
-  __shared__ double s_alpha[2], s_beta[2], s_v0[2];
+  __shared__ double s_alpha[2], s_beta[2], s_hbeta[2], s_v0[2];
   const int nr = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int rp = (m + nr - 1) / nr, pitch = m + 1;
   double* A_ = csh;                       // [rp][pitch] own rows
@@ -245,7 +254,7 @@ __global__ void __launch_bounds__(kTriThreads)
       const double x0 = x[n0];
       double s = 0.0;
       for (int j = n0 + 1 + lane; j < m; j += 32) s = fma(x[j], x[j], s);
-      const bool any = __any_sync(0xffffffffu, s != 0.0);
+      const bool any = __any_sync(0xffffffffu, fx_bits(s) != 0);   // (no FP64 comparison)
       if (lane == 31) s = fma(x0, x0, s);
       long long t;
       int ex;
@@ -263,6 +272,7 @@ __global__ void __launch_bounds__(kTriThreads)
         }
         s_alpha[b] = alpha;
         s_beta[b] = beta;
+        s_hbeta[b] = 0.5 * beta;
         s_v0[b] = v0;
         if (rank == 0) e[k] = alpha;
       }
@@ -308,23 +318,38 @@ __global__ void __launch_bounds__(kTriThreads)
     else __syncthreads();
     // scalars, in every warp alike
     const double alpha = s_alpha[b], beta = s_beta[b], v0 = s_v0[b];
-    double xy = 0.0;
-    for (int j = n0 + lane; j < m; j += 32) xy = fma(x[j], Yb[j], xy);
-    const double y1 = Yb[n0], c1 = Cb[n0];
-    const double hb = 0.5 * beta * beta, rest = alpha * fma(alpha, c1, -2.0 * y1);
-    const double p1 = beta * fma(-alpha, c1, y1);
-    xy = warp_sum64(xy);
-    const double K = hb * (xy + rest);
-    const double w1 = fma(-K, v0, p1);
-    double* xn = xf + (b ^ 1) * m;
+    // p = beta (y - alpha C) and v^T p in every warp; lane l has the entries n0 + l
+    // + 32 q and keeps that of q = warp, entry j = n0 + tid (m <= kTriThreads)
+    double vp = 0.0, p1 = 0.0, vj = 0.0, pj = 0.0, cj = 0.0;
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+      if (n0 + 32 * q >= m) break;
+      const int i = n0 + 32 * q + lane;
+      double v = 0.0, p = 0.0, c = 0.0;
+      if (i < m) {
+        c = Cb[i];
+        v = i == n0 ? v0 : x[i];
+        p = beta * fma(-alpha, c, Yb[i]);
+        vp = fma(v, p, vp);
+      }
+      if (q == 0) p1 = __shfl_sync(0xffffffffu, p, 0);
+      if (q == warp) {
+        vj = v;
+        pj = p;
+        cj = c;
+      }
+    }
+    // the next column is C - v w_1 - w v_1 with w = p - K v, K = beta/2 v^T p: two
+    // operations after the sum
+    const int j = n0 + tid;
+    const double cp = fma(-pj, v0, fma(-vj, p1, cj)), vv = vj * v0;
+    const double sum = warp_sum64(vp), K2 = beta * sum, K = s_hbeta[b] * sum;
     if (tid == 0 && (n0 - 1) == 0 && rank == 0) d[0] = A_[0];
-    for (int j = n0 + tid; j < m; j += kTriThreads) {
-      const double vj = j == n0 ? v0 : x[j], cj = Cb[j];
-      const double wj = fma(-K, vj, beta * fma(-alpha, cj, Yb[j]));
-      const double cn = fma(-wj, v0, fma(-vj, w1, cj));   // column n0 of the updated matrix
+    if (j < m) {
+      const double cn = fma(K2, vv, cp);
       vf[j] = vj;
-      wf[j] = wj;
-      xn[j] = cn;
+      wf[j] = fma(-K, vj, pj);
+      xf[(b ^ 1) * m + j] = cn;
       if (j == n0 && rank == 0) d[n0] = cn;
     }
     __syncthreads();
@@ -565,6 +590,7 @@ __global__ void __launch_bounds__(kBisPts) bisect_kernel(const double* __restric
   __shared__ double sd[kMaxM], se2[kMaxM];
   __shared__ double s_lo, s_hi, s_scale;
   __shared__ unsigned s_ball[2][kBisWarps];
+  __shared__ double s_x[2][kBisPts];   // the points of a round
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (warp == 0) {
     double lo = dg[0], hi = dg[0];
@@ -599,11 +625,16 @@ __global__ void __launch_bounds__(kBisPts) bisect_kernel(const double* __restric
   __syncthreads();
   const int j = blockIdx.x;
   double lo = s_lo, hi = s_hi;
+  const double part = (double)(tid + 1) / (double)kBisPts;
   for (int it = 0; it < 16; ++it) {
+    // (positive doubles order as their bits; a comparison takes the FP64 unit)
     const double width = hi - lo;
-    if (width <= 4.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi)) + 0x1p-70) break;
+    const long long al = fx_bits(lo) & 0x7fffffffffffffffLL, ah = fx_bits(hi) & 0x7fffffffffffffffLL;
+    const double tol = fma(4.0 * 2.220446049250313e-16, fx_from_bits(al > ah ? al : ah), 0x1p-70);
+    if (fx_bits(width) <= fx_bits(tol)) break;
     // points lo + width (t+1)/128, t < 127; point 127 is hi (count m + 1)
-    const double x = lo + width * (double)(tid + 1) / (double)kBisPts;
+    const double x = fma(width, part, lo);
+    s_x[it & 1][tid] = x;
     const int c = tid < kBisPts - 1 ? sturm_count(sd, se2, m, x) : m + 1;
     const unsigned ball = __ballot_sync(0xffffffffu, c > j);
     if (lane == 0) s_ball[it & 1][warp] = ball;
@@ -614,11 +645,8 @@ __global__ void __launch_bounds__(kBisPts) bisect_kernel(const double* __restric
       const unsigned b = s_ball[it & 1][w];
       if (b) first = 32 * w + __ffs(b) - 1;
     }
-    const double nlo = first == 0 ? lo : lo + width * (double)first / (double)kBisPts;
-    const double nhi =
-        first == kBisPts - 1 ? hi : lo + width * (double)(first + 1) / (double)kBisPts;
-    lo = nlo;
-    hi = nhi;
+    if (first > 0) lo = s_x[it & 1][first - 1];
+    if (first < kBisPts - 1) hi = s_x[it & 1][first];
   }
   if (tid == 0) E[j] = 0.5 * (lo + hi) / g;
 }

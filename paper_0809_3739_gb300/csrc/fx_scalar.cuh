@@ -146,7 +146,7 @@ ITP_HD void fx_reflector(FxNum s2, double x0, double* alpha, double* beta, doubl
   const int down = fx_exponent(x0) == 0 ? 64 : en - x.e;
   const unsigned long long X = down > 63 ? 0 : (down < 0 ? ~0ULL : x.m >> down);
   const unsigned long long D = (F >> 1) + (fx_mulhi(X, N) >> 1);   // scaled 2^61, 2^E
-  const long long sx = x0 > 0 ? 0 : -1;                            // the sign of v_0
+  const long long sx = fx_bits(x0) > 0 ? 0 : -1;                   // the sign of v_0
   FxNum nn;
   nn.m = N;
   nn.e = en;
