@@ -99,6 +99,15 @@ __host__ __device__ constexpr int plane64_threads(int nx) {
   return nx == 128 ? 512 : nx == 64 ? 264 : kThreads;
 }
 
+// CTAs per SM of the FP64 passes whose shared memory admits them (planes up to
+// 64 x 64, pencils up to 64): with two, 17 warps waited at barriers and on the
+// integer pipe; three have 72 registers, which spills little.  57 states at
+// 64^3: pencil 0.142 -> 0.124 ms, forward 0.149 -> 0.133, merged 0.219 -> 0.211,
+// last pass 0.166 -> 0.154 (four CTAs of the pencil 0.120, but slower at 32).
+// The radix-16 stages of 128-point pencils do not fit: 0.97 ms with two, 1.18
+// with three, 48 states at 128^3.
+constexpr int kFixedCtas = 3;
+
 // Threads per CTA of a plane kernel, and of its launch bounds.
 template <typename R>
 __host__ __device__ constexpr int plane_threads(int nx) {
@@ -1049,7 +1058,7 @@ __global__ void __launch_bounds__(plane_threads<R>(NX),
 // row y is a state of one of the terms p.)
 template <int NX, int NY, int MODE>
 __global__ void __launch_bounds__(plane_threads<double>(NX),
-                                  min_blocks(plane_smem_ct(NX, NY, 8), 2))
+                                  min_blocks(plane_smem_ct(NX, NY, 8), kFixedCtas))
     plane64_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<double>> p,
                    const PlaneArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
   const int t = rows ? 0 : blockIdx.y / p.a[0].m;
@@ -1630,7 +1639,8 @@ __global__ void __launch_bounds__(launch_threads(task_threads(W)),
 // FP64 pencil pass, single or grouped (rows set) launches, either mode.
 template <int NZ, int W>
 __global__ void __launch_bounds__(launch_threads(task_threads(W)),
-                                  NZ ? min_blocks(pencil_smem_ct(NZ, W, 8), pencil_min_ctas(NZ, 8)) : kGenericCtas64)
+                                  NZ ? min_blocks(pencil_smem_ct(NZ, W, 8), NZ <= 64 ? kFixedCtas : pencil_min_ctas(NZ, 8))
+                                     : kGenericCtas64)
     pencil64_kernel(const GridDesc g, const __grid_constant__ TermPack<PencilArgs<double>> p,
                     const PencilArgs<double>* __restrict__ args, const int2* __restrict__ rows) {
   const int t = rows ? 0 : blockIdx.y / p.a[0].m;
