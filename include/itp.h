@@ -56,7 +56,8 @@ extern "C" {
 #define ITP_ERR_NOCONV 7   /* subspace eigen-decomposition did not converge */
 
 typedef enum {
-  ITP_FP64 = 0,  /* every step in FP64                                      */
+  ITP_FP64 = 0,  /* every step to FP64 accuracy (transforms and contractions
+                    in 64-bit fixed point, states and matrices FP64)        */
   ITP_MIXED = 1  /* FP32 FFT passes, FP64 combination / Cholesky / energies */
 } itp_precision;
 
@@ -244,7 +245,9 @@ int itp_synchronize(itp_handle h);
  * the handle's next `launches` tensor-core kernel launches made outside a
  * CUDA-graph capture first waits, before issuing any copy or MMA, on an
  * mbarrier phase that nothing completes, with a 2 ms limit instead of 2 s.
- * 0 switches it off.  ITP_FP64 handles launch no tensor-core kernels.
+ * 0 switches it off.  (Up to 64 states these contractions run on the FP32
+ * cores unless the hook is on.)  ITP_FP64 handles launch no kernel with such
+ * waits.
  * Returns ITP_OK or ITP_ERR_ARG (launches < 0). */
 int itp_test_expire_waits(itp_handle h, int launches);
 
@@ -302,7 +305,8 @@ int itp_profile_read(itp_handle h, int kind, long long* launches, double* total_
  *                        8, 16, or 32 (32: FP32 with nx = 256 only); it
  *                        divides ny/2
  *   [ITP_TUNE_GRAM]      CTAs (partial sums) of the overlap kernel,
- *                        1..2 x the SM count
+ *                        1..2 x the SM count (FP64 with more than 32
+ *                        states: at most that many)
  * Results depend on the shapes only through rounding. */
 #define ITP_TUNE_PENCIL_W 0
 #define ITP_TUNE_SPLIT 1

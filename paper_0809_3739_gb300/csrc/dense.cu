@@ -80,7 +80,7 @@ __device__ __forceinline__ bool is_pivot(double d) {
 //   A[i][j] -= sum_c U[i][c] A[j][c]  (j <= i),   R[i][j] -= sum_c U[i][c] R[c][j].
 // One cluster barrier per panel (the column-by-column form took one cluster
 // and two block barriers, a square root and a division per column: 2.5 us;
-// 57 states 0.118 -> 0.063 ms, 128 states 0.35 -> 0.165).
+// 57 states 0.118 -> 0.055 ms, 128 states 0.35 -> 0.148).
 __global__ void __launch_bounds__(kClusThreads)
     cholesky_inverse_kernel(const double* __restrict__ S, int m, double* __restrict__ Minv,
                             int* status) {
