@@ -84,13 +84,13 @@ NCU_TRAFFIC = {
     # DRAM bytes (read + write) per full launch from one ncu capture of the
     # 16-state case, scaled by the number of states; valid only while the
     # kernel's source file is the one that was profiled
-    ("c60_128", "plane_merged"): {"bytes": 1.784e9,
+    ("c60_128", "plane_merged"): {"bytes": 1.755e9,
                                   "source": "paper_0809_3739_gb300/csrc/fft_passes.cuh",
-                                  "sha1": "6982298585d4fd2f311b2719a76cc47cd560377c",
+                                  "sha1": "fd1d17321919571493a0c52b5a3dfdd31b5d9297",
                                   "profile": "profiles/plane_merged_c60_128.md"},
-    ("c60_128", "pencil"): {"bytes": 1.697e9,
+    ("c60_128", "pencil"): {"bytes": 1.668e9,
                             "source": "paper_0809_3739_gb300/csrc/fft_tmem.cuh",
-                            "sha1": "5657d3abdd160f6831798c09342aa04ad0083a70",
+                            "sha1": "6dbcf2502cb70f6918dd4464464046f1601e74c4",
                             "profile": "profiles/pencil_tmem_c60_128.md"},
 }
 

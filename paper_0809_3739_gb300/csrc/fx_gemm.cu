@@ -14,7 +14,7 @@
 // bit multiply-add (IMAD.WIDE) issues every 3.2 cycles with general operands
 // (every 2 in a chain).  More states have enough products per element to pay
 // for splitting it into base-256 digits: the tensor cores multiply those
-// exactly (128 states at 64^3, an eighth of those points: 0.98 and 0.81 ms).
+// exactly (128 states at 64^3, an eighth of those points: 0.76 and 0.81 ms).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
