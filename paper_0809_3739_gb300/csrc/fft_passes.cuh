@@ -1449,8 +1449,11 @@ struct RowGeo : PlaneGeo<R, NX, 2 * TB, kThreads> {
   }
 };
 
+// (256-point FP32 rows: three CTAs per SM, as shared memory admits; the merged
+// pass took 108 registers without the bound, which left two: 16 states at 256^3
+// 1.99 -> 1.84 ms, 89 on 256^2 0.0574 -> 0.0532.)
 template <typename R, int NX, int TB, int MODE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, NX == 256 && sizeof(R) == 4 ? 3 : 1)
     rowpass_kernel(const GridDesc g, const __grid_constant__ TermPack<PlaneArgs<R>> p) {
   const int term = blockIdx.y / p.a[0].m;
   const PlaneArgs<R>& a = p.a[term];
