@@ -86,7 +86,7 @@ NCU_TRAFFIC = {
     # kernel's source file is the one that was profiled
     ("c60_128", "plane_merged"): {"bytes": 1.755e9,
                                   "source": "paper_0809_3739_gb300/csrc/fft_passes.cuh",
-                                  "sha1": "fd1d17321919571493a0c52b5a3dfdd31b5d9297",
+                                  "sha1": "262836b9fac4012292ded19bd13ea175d65a0055",
                                   "profile": "profiles/plane_merged_c60_128.md"},
     ("c60_128", "pencil"): {"bytes": 1.668e9,
                             "source": "paper_0809_3739_gb300/csrc/fft_tmem.cuh",
