@@ -7,12 +7,9 @@
 // states).  So the operands are scaled to integers of 55 or 56 bits.
 //
 // Up to 32 states they are split into two signed halves v = h 2^28 + l, and a
-// product takes
-//   Gram:   h h', and h l' + l h' (l l' is below the precision, see there);
-//   update: h h', h l' + l h', and l l',
-// accumulated exactly in 64-bit integers over up to 512 terms: a 32 x 32 + 64-
-// bit multiply-add (IMAD.WIDE) issues every 3.2 cycles with general operands
-// (every 2 in a chain).  More states have enough products per element to pay
+// product is h h', h l' + l h' and l l', accumulated exactly in 64-bit integers
+// over up to 512 terms: a 32 x 32 + 64-bit multiply-add (IMAD.WIDE) issues
+// every 3.2 cycles with general operands (every 2 in a chain).  More states have enough products per element to pay
 // for splitting it into base-256 digits: the tensor cores multiply those
 // exactly (128 states at 64^3, an eighth of those points: 0.76 and 0.81 ms).
 #include <cuda_fp16.h>
@@ -103,9 +100,13 @@ __device__ __forceinline__ void load_pairs(const int2* p, int2 (&v)[N]) {
 // shared memory as halves, [point][row].
 //
 // Precision: with the row's largest value in the run scaled to 2^54, an
-// element is off by at most 2^-55 of it and the missing l l' by about 2^-56
-// of the two largest values, with random signs, so a sum is off by less than
-// one FP64 rounding of |A_i| |B_j| whatever the states' shape.
+// element is off by at most 2^-55 of it, with random signs, and the products
+// are exact, so a sum is off by less than one FP64 rounding of |A_i| |B_j|
+// whatever the states' shape.  l l' is part of that: on the diagonal it is a
+// square, and without it every squared norm came out too small, by about 2^-55
+// of the run's largest square per point (relative error of S_ii 8e-16 for
+// oscillator states on 32^3, 4e-15 for one large value per run with 1e-5 beside
+// it; with it 7e-17 and 1e-16, below the FP64 sums' 1.2e-16 and equal to them).
 constexpr int kRun = 512;
 constexpr int kTile = 16;   // (32 points needed more registers for the tile in flight)
 constexpr int kGramBits = 54;
@@ -166,11 +167,11 @@ __global__ void __launch_bounds__(256, 3)
       }
     }
     __syncthreads();
-    long long hh[TT][TT], hl[TT][TT];
+    long long hh[TT][TT], hl[TT][TT], ll[TT][TT];
 #pragma unroll
     for (int q = 0; q < TT; ++q)
 #pragma unroll
-      for (int r = 0; r < TT; ++r) hh[q][r] = hl[q][r] = 0;
+      for (int r = 0; r < TT; ++r) hh[q][r] = hl[q][r] = ll[q][r] = 0;
     double va[TT], vb[TT];
     load(A, run, re, va);
     if (!one) load(B, run, re, vb);
@@ -212,27 +213,33 @@ __global__ void __launch_bounds__(256, 3)
 #pragma unroll
         for (int q = 0; q < TT; ++q)
 #pragma unroll
-          for (int r = 0; r < TT; ++r) hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
+          for (int r = 0; r < TT; ++r) {
+            hl[q][r] = fx_wide(a[q].y, b[r].x, hl[q][r]);
+            ll[q][r] = fx_wide(a[q].y, b[r].y, ll[q][r]);   // <= 256 * 2^54
+          }
       }
       if (more) store((t + 1) & 1);
-      if ((t + 1) * kTile == kRun / 2) {   // keep the middle sums within 64 bits
+      if ((t + 1) * kTile == kRun / 2) {   // keep the lower sums within 64 bits
 #pragma unroll
         for (int q = 0; q < TT; ++q)
 #pragma unroll
           for (int r = 0; r < TT; ++r) {
+            hl[q][r] += ll[q][r] >> kHalf;
+            ll[q][r] &= (1LL << kHalf) - 1;
             hh[q][r] += hl[q][r] >> kHalf;
             hl[q][r] &= (1LL << kHalf) - 1;
           }
       }
     }
-    // the run's sums to FP64: (hh 2^56 + hl 2^28) 2^(ea + eb - 2 * (1022 + 54))
+    // the run's sums to FP64: (hh 2^56 + hl 2^28 + ll) 2^(ea + eb - 2 * (1022 + 54))
 #pragma unroll
     for (int q = 0; q < TT; ++q) {
       const int ea = eA[ty * TT + q];
 #pragma unroll
       for (int r = 0; r < TT; ++r) {
         const int eb = (one ? eA : eB)[tx * TT + r];
-        const double s = fma((double)hh[q][r], (double)(1LL << kHalf), (double)hl[q][r]);
+        const long long mid = hl[q][r] + (ll[q][r] >> kHalf);
+        const double s = fma((double)hh[q][r], (double)(1LL << kHalf), (double)mid);
         double v = scale2(s, ea + eb - 2 * (1022 + kGramBits) + kHalf);
         if (ea == 2047 || eb == 2047) v = __longlong_as_double(0x7ff8000000000000LL);
         add_sum(ty * TT + q, tx * TT + r, v, run == p_begin);
