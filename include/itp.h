@@ -385,7 +385,9 @@ long long itp_batch_kernel_launches(itp_batch_handle b);
 /* How a batch step's graph is built.  grouped != 0 (the default): problems
  * with the same grid, precision lane, launch shapes and pass sequence form a
  * group, and each FFT pass of a step (plane, pencil, exact term sum) is one
- * launch over all the states of the group's problems -- a CTA row looks up
+ * launch over all the states of the group's problems (at most 65535 states
+ * in a group, else ITP_ERR_ARG; several launches where the states times the
+ * terms of a pass are more than that) -- a CTA row looks up
  * its (problem, state) and that problem's arguments in tables the batch
  * keeps in device memory -- while the remaining kernels of each problem
  * (overlap, Cholesky, update, eigenvalues, copies) run as parallel branches

@@ -1279,6 +1279,19 @@ std::string group_key(itp_handle h, const std::vector<RecOp>& ops) {
   return key;
 }
 
+// A grouped pass over the rows of its table: launch(rows, count) in pieces of
+// at most kGroupRows rows, the y extent of a grid (a row is a state of a term:
+// six per state at order 12).
+constexpr int kGroupRows = 65535;
+template <typename F>
+cudaError_t launch_rows(const int2* rows, int nrows, F&& launch) {
+  for (int r = 0; r < nrows; r += kGroupRows) {
+    const cudaError_t e = launch(rows + r, std::min(kGroupRows, nrows - r));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // Build the graph of one step of every problem with grouped launches: each
 // FFT pass (plane, pencil, exact term sum) of the problems in a group (same
 // grid, lane, launch shapes and pass sequence) is one launch over all their
@@ -1334,6 +1347,7 @@ int build_grouped_graph(itp_batch* b, int k, double tau, int eflags, cudaGraph_t
       if (G.size() < 2) continue;
       std::vector<int2> rows;
       std::vector<unsigned char> args;
+      int states = 0;
       for (int q = 0; q < (int)G.size(); ++q) {
         const RecOp& op = ops[G[q]][t];
         // a table entry and its states per term
@@ -1354,13 +1368,14 @@ int build_grouped_graph(itp_batch* b, int k, double tau, int eflags, cudaGraph_t
           a = &op.ts;
           asz = sizeof(op.ts);
         }
+        states += nrow;
         for (size_t e = 0; e < nt; ++e)
           for (int r = 0; r < nrow; ++r) rows.push_back(make_int2((int)(q * nt + e), r));
         const size_t o = args.size();
         args.resize(o + nt * asz);
         memcpy(args.data() + o, a, nt * asz);
       }
-      if (rows.size() > 65535)
+      if (states > kGroupRows)
         return batch_fail(b, ITP_ERR_ARG, "a group has more than 65535 states; "
                                           "use itp_batch_set_grouping(b, 0)");
       Planned pl;
@@ -1406,25 +1421,30 @@ int build_grouped_graph(itp_batch* b, int k, double tau, int eflags, cudaGraph_t
           e = o0[t].fn();
         } else {
           const Planned& pl = plan[gi][t];
-          const int2* rows = reinterpret_cast<const int2*>(dev + pl.rows);
           const RecOp& op = o0[t];
-          if (op.kind == RecOp::kPlane)
-            e = op.lane ? launch_plane_group<double>(
-                              h0->g, op.mode, reinterpret_cast<const PlaneArgs<double>*>(dev + pl.args),
-                              rows, pl.nrows, gst)
-                        : launch_plane_group<float>(
-                              h0->g, op.mode, reinterpret_cast<const PlaneArgs<float>*>(dev + pl.args),
-                              rows, pl.nrows, gst);
-          else if (op.kind == RecOp::kPencil)
-            e = op.lane ? launch_pencil_group<double>(
-                              h0->g, op.mode, reinterpret_cast<const PencilArgs<double>*>(dev + pl.args),
-                              rows, pl.nrows, gst)
-                        : launch_pencil_group<float>(
-                              h0->g, op.mode, reinterpret_cast<const PencilArgs<float>*>(dev + pl.args),
-                              rows, pl.nrows, gst);
-          else
-            e = launch_term_sum_group(reinterpret_cast<const TermSumArgs*>(dev + pl.args), rows,
-                                      pl.nrows, op.ts.nz, op.ts.plane_pts, gst);
+          const unsigned char* args = dev + pl.args;
+          e = launch_rows(
+              reinterpret_cast<const int2*>(dev + pl.rows), pl.nrows,
+              [&](const int2* rows, int n) {
+                if (op.kind == RecOp::kPlane)
+                  return op.lane
+                             ? launch_plane_group<double>(
+                                   h0->g, op.mode, reinterpret_cast<const PlaneArgs<double>*>(args),
+                                   rows, n, gst)
+                             : launch_plane_group<float>(
+                                   h0->g, op.mode, reinterpret_cast<const PlaneArgs<float>*>(args),
+                                   rows, n, gst);
+                if (op.kind == RecOp::kPencil)
+                  return op.lane
+                             ? launch_pencil_group<double>(
+                                   h0->g, op.mode, reinterpret_cast<const PencilArgs<double>*>(args),
+                                   rows, n, gst)
+                             : launch_pencil_group<float>(
+                                   h0->g, op.mode, reinterpret_cast<const PencilArgs<float>*>(args),
+                                   rows, n, gst);
+                return launch_term_sum_group(reinterpret_cast<const TermSumArgs*>(args), rows, n,
+                                             op.ts.nz, op.ts.plane_pts, gst);
+              });
         }
         ++t;
         continue;
