@@ -77,9 +77,20 @@ typedef struct itp_grid* itp_handle;
  *                overlap and three times the update per block of states)
  *   precision    ITP_FP64 or ITP_MIXED
  *   cuda_stream  cudaStream_t to issue work on (NULL: default stream)
- * Allocates all device memory for the states, the half-spectrum workspace
- * and the FP64 accumulator.  Returns ITP_ERR_ARG / ITP_ERR_OOM /
- * ITP_ERR_CUDA on failure. */
+ * Allocates the device memory for the states, the half-spectrum workspace,
+ * the factor tables and the FP64 accumulator.  Later calls add
+ *  - the FP64 lane of an ITP_MIXED handle (states, workspace and tables in
+ *    FP64) at its first FP64 work;
+ *  - k - 1 more half-spectrum workspaces at the first propagation or step of
+ *    order 2k: with ITP_MIXED except on row + column planes; else by steps
+ *    of small problems (itp_step, itp_step_host, itp_polish,
+ *    itp_solve_adaptive, itp_propagate_romberg6, itp_autotune,
+ *    itp_batch_step), which run the terms together, at most 1 GiB for the
+ *    handle or for all problems of a batch and only if an eighth of the
+ *    device's memory stays free.  They are taken whole or not at all (the
+ *    terms then run one after another) and kept until itp_destroy;
+ *  - what the calls below name.
+ * Returns ITP_ERR_ARG / ITP_ERR_OOM / ITP_ERR_CUDA on failure. */
 int itp_create_grid(itp_handle* out, int nx, int ny, int nz, double lx, double ly, double lz,
                     int n_states, int n_guard, int precision, void* cuda_stream);
 

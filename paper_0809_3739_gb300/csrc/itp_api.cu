@@ -33,7 +33,7 @@ struct Lane {
   void* work = nullptr;      // [m][n_half] complex
   void* work_terms[kMaxTerms] = {};  // per-term spectra / contributions (mixed)
   bool fused_ok = true;              // per-term workspaces could be allocated
-  bool together_ok = true;
+  bool together_ok = true;           // and those that only running the terms together needs
   R* f_half[kMaxTerms] = {}; // exp(-tau_i V / 2)
   R* f_full[kMaxTerms] = {}; // exp(-tau_i V)      (terms i >= 2)
   R* ktab = nullptr;         // per term: nxh + ny + nz propagation factors
@@ -488,20 +488,52 @@ bool terms_fused(itp_handle h) {
   return sizeof(R) == 4 && lane_of<R>(h).fused_ok && h->g.split_planes[0] != 1;
 }
 
-// A workspace per term, where the terms run together or keep their
-// contributions; without the memory for it both are off for the handle.
+// Bytes of the term workspaces that the handle has not got yet.
+template <typename R>
+size_t missing_workspaces(itp_handle h, int k) {
+  size_t n = 0;
+  for (int i = 1; i < k; ++i) n += !lane_of<R>(h).work_terms[i];
+  return n * h->m * h->g.n_half * 2 * sizeof(R);
+}
+// The same where only running the terms together asks for them.
+template <typename R>
+size_t optional_workspaces(itp_handle h, int k) {
+  const bool wanted = !terms_fused<R>(h) && lane_of<R>(h).together_ok && terms_together<R>(h, k);
+  return wanted ? missing_workspaces<R>(h, k) : 0;
+}
+
+// A workspace per term, where the terms run together (step) or keep their
+// contributions.  All or none: what a failing allocation leaves is given back,
+// and both are off for the handle.  Workspaces for running together alone are
+// taken only while an eighth of the device's memory stays free, and not by a
+// step that is being captured or recorded (its resources are there already).
 template <typename R>
 void term_workspaces(itp_handle h, int k, bool step = true) {
   Lane<R>& L = lane_of<R>(h);
   L.work_terms[0] = L.work;
-  if (!terms_fused<R>(h) && !(step && L.together_ok && terms_together<R>(h, k))) return;
-  for (int i = 1; i < k; ++i) {
-    if (!L.work_terms[i] &&
-        cudaMalloc(&L.work_terms[i], (size_t)h->m * h->g.n_half * 2 * sizeof(R)) != cudaSuccess) {
-      cudaGetLastError();   // clear the allocation error; use the per-term path
-      L.fused_ok = L.together_ok = false;
+  if (!terms_fused<R>(h)) {
+    if (!step || h->capturing || h->rec) return;
+    const size_t need = optional_workspaces<R>(h, k);
+    size_t unused = 0, total = 0;
+    if (need == 0) return;
+    if (cudaMemGetInfo(&unused, &total) != cudaSuccess || unused < need + total / 8) {
+      cudaGetLastError();
+      L.together_ok = false;
       return;
     }
+  }
+  void* got[kMaxTerms] = {};
+  bool ok = true;
+  for (int i = 1; i < k && ok; ++i)
+    if (!L.work_terms[i])
+      ok = cudaMalloc(&got[i], (size_t)h->m * h->g.n_half * 2 * sizeof(R)) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();   // clear the allocation error; use the per-term path
+    L.fused_ok = L.together_ok = false;
+  }
+  for (int i = 1; i < k; ++i) {
+    if (got[i] && ok) L.work_terms[i] = got[i];
+    else if (got[i]) cudaFree(got[i]);
   }
 }
 
@@ -523,7 +555,8 @@ int propagate_lane(itp_handle h, int k, double tau, int s0 = 0, const R* in = nu
   const size_t tl = (size_t)g.nxh + g.ny + g.nz;
   term_workspaces<R>(h, k, step);
   const bool fused = terms_fused<R>(h);
-  const bool together = step && L.together_ok && terms_together<R>(h, k);
+  const bool together = step && L.together_ok && terms_together<R>(h, k) &&
+                        missing_workspaces<R>(h, k) == 0;
   // states s0..s1-1 only (s1 < 0: to the last state; the others are kept)
   const int ms = (s1 < 0 ? h->m : s1) - s0;
   const long long so = s0;
@@ -821,11 +854,12 @@ int step_work(itp_handle h, int k, double tau, int flags) {
 }
 
 // Everything a step allocates or builds once, done outside any capture.
+// optional: also the workspaces that only running the terms together needs.
 template <typename R>
-int step_resources(itp_handle h, int k, double tau) {
+int step_resources(itp_handle h, int k, double tau, bool optional = true) {
   Lane<R>& L = lane_of<R>(h);
   ITP_TRY(prepare_tables<R>(h, L, k, tau));
-  term_workspaces<R>(h, k);
+  term_workspaces<R>(h, k, optional);
   return ITP_OK;
 }
 
@@ -2165,16 +2199,19 @@ int itp_batch_step(itp_batch_handle b, int order, double tau, int flags, double*
     return batch_fail(b, rc, "problem " + std::to_string(p) + ": " + b->probs[p]->err);
   };
   // per problem, outside any capture: lane, tables and workspaces
+  size_t optional = 0;
   for (int p = 0; p < np; ++p) {
     itp_handle h = b->probs[p];
     int rc = check_ready(h, true);
     if (rc == ITP_OK) {
       if (h->precision == ITP_MIXED && !(flags & ITP_STEP_FP64)) {
         rc = switch_lane<float>(h);
-        if (rc == ITP_OK) rc = step_resources<float>(h, k, tau);
+        if (rc == ITP_OK) rc = step_resources<float>(h, k, tau, false);
+        if (rc == ITP_OK) optional += optional_workspaces<float>(h, k);
       } else {
         if (h->precision == ITP_MIXED) rc = switch_lane<double>(h);
-        if (rc == ITP_OK) rc = step_resources<double>(h, k, tau);
+        if (rc == ITP_OK) rc = step_resources<double>(h, k, tau, false);
+        if (rc == ITP_OK) optional += optional_workspaces<double>(h, k);
       }
     }
     if (rc != ITP_OK) return prob_fail(p, rc);
@@ -2182,6 +2219,13 @@ int itp_batch_step(itp_batch_handle b, int order, double tau, int flags, double*
     if (cudaEventRecord(b->join[p], h->st) != cudaSuccess ||
         cudaStreamWaitEvent(b->st, b->join[p], 0) != cudaSuccess)
       return batch_fail(b, ITP_ERR_CUDA, "stream ordering");
+  }
+  // the optional workspaces after all others, for every problem or for none
+  if (optional > 0 && optional <= kTogetherBytes) {
+    for (itp_handle h : b->probs) {
+      if (h->cur64) term_workspaces<double>(h, k);
+      else term_workspaces<float>(h, k);
+    }
   }
   bool stale = (int)b->versions.size() != np;
   for (int p = 0; p < np && !stale; ++p) stale = b->versions[p] != b->probs[p]->tune_version;
