@@ -25,7 +25,6 @@ namespace {
 
 constexpr int kMaxM = 256;   // states of the n x n work at most
 constexpr int kHalf = 28;    // bits of the lower half
-constexpr int kSms = 152;    // SMs of a GB300
 
 // The double d as an integer of scale 2^(BITS - 1) at the biased exponent e
 // (|d| < 2^(e - 1022)): |result| <= 2^BITS, rounded to nearest, 0 for
@@ -810,12 +809,12 @@ cudaError_t apply_launch(const double* M, int m, int lower, const double* S, con
 // for a ragged last run and for its m x m sums).  Against 304 chunks always: 37
 // states at 72 x 48 x 36 2.10 -> 2.06 ms per step, orthonormalisation of a
 // 100 x 250047 block 1.65 -> 1.63 ms.
-int gram_chunks(int m, bool same, long long n_points, int most) {
+int gram_chunks(int m, bool same, long long n_points, int most, int sms) {
   if (m <= kGramMmaMin) return most;
   const int nb = (m + kMmaRows - 1) / kMmaRows, blocks = same ? nb * (nb + 1) / 2 : nb * nb;
-  int c = kSms / blocks > 1 ? kSms / blocks : 1;
-  for (int w = 2; w * kSms / blocks <= most && n_points / (w * kSms / blocks) >= 4 * kRun; ++w)
-    c = w * kSms / blocks;
+  int c = sms / blocks > 1 ? sms / blocks : 1;
+  for (int w = 2; w * sms / blocks <= most && n_points / (w * sms / blocks) >= 4 * kRun; ++w)
+    c = w * sms / blocks;
   return c < most ? c : most;
 }
 

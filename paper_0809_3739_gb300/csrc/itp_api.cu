@@ -84,6 +84,7 @@ struct itp_grid {
   Lane<double> f64;
   bool cur64 = true;          // which lane holds the states
   bool have_V = false, have_states = false, have_phi = false;
+  int sms = 152;              // SMs of the device
   int n_chunks = 0;           // Gram partial sums (CUDA-core kernels)
   int n_chunks_tc = 0;        // Gram partial sums (tensor-core kernel: one CTA per SM, FP32
                               // cores: two)
@@ -660,7 +661,7 @@ int orthonormalize_lane(itp_handle h);
 template <>
 int orthonormalize_lane<double>(itp_handle h) {
   Lane<double>& L = h->f64;
-  const int chunks = gram_chunks(h->m, true, h->g.n_points, h->n_chunks);
+  const int chunks = gram_chunks(h->m, true, h->g.n_points, h->n_chunks, h->sms);
   ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_gram_partial(h->acc, h->acc, h->m, h->g.n_points, chunks,
                                                       h->partial, h->st)));
   ITP_LAUNCH(h, ITP_KERNEL_GRAM_REDUCE,
@@ -736,7 +737,7 @@ int energies_lane(itp_handle h, int flags) {
   }
   ITP_LAUNCH_PASS(h, ITP_KERNEL_PLANE_HPSI, plane_counted<R>(h, &ph));
   const int chunks = sizeof(R) == 4 ? h->n_chunks_tc
-                                    : gram_chunks(h->m, false, g.n_points, h->n_chunks);
+                                    : gram_chunks(h->m, false, g.n_points, h->n_chunks, h->sms);
   if (sizeof(R) == 4) {
     ITP_LAUNCH(h, ITP_KERNEL_GRAM, (launch_tc_gram(
                                        reinterpret_cast<const float*>(L.psi),
@@ -1005,13 +1006,16 @@ int autotune_lane(itp_handle h, int k, double tau, std::string& rep) {
     }
     ITP_TRY(set_tuning(h, best));
   }
-  // 3. CTAs of the overlap kernel, timed on the propagated block
+  // 3. CTAs of the overlap kernel, timed on the propagated block as a step
+  // launches it (FP64: gram_chunks of the candidate, where two may be the same)
   {
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     float best_ms = 1e30f;
+    int last = -1;
     rep += "; gram:";
-    for (int chunks : {sms, 2 * sms}) {
+    for (int most : {h->sms, 2 * h->sms}) {
+      const int chunks = pi == 0 ? most : gram_chunks(h->m, true, g.n_points, most, h->sms);
+      if (chunks == last) continue;
+      last = chunks;
       float ms = 0.f;
       auto gram = [&]() -> int {
         cudaError_t e;
@@ -1019,8 +1023,7 @@ int autotune_lane(itp_handle h, int k, double tau, std::string& rep) {
           e = launch_tc_gram(h->f32.psi_tmp, h->f32.psi_tmp, h->m, g.n_points, chunks,
                              h->partial, h->status, h->st);
         else
-          e = launch_gram_partial(h->acc, h->acc, h->m, g.n_points,
-                                                          chunks, h->partial, h->st);
+          e = launch_gram_partial(h->acc, h->acc, h->m, g.n_points, chunks, h->partial, h->st);
         return e == cudaSuccess ? ITP_OK : fail(h, ITP_ERR_CUDA, "gram: %s",
                                                 cudaGetErrorString(e));
       };
@@ -1029,7 +1032,7 @@ int autotune_lane(itp_handle h, int k, double tau, std::string& rep) {
       rep += buf;
       if (ms < best_ms) {
         best_ms = ms;
-        best[ITP_TUNE_GRAM] = chunks;
+        best[ITP_TUNE_GRAM] = most;   // (the subspace matrix's count follows from it too)
       }
     }
     ITP_TRY(set_tuning(h, best));
@@ -1625,10 +1628,9 @@ int itp_create_grid(itp_handle* out, int nx, int ny, int nz, double lx, double l
   }
   if (cudaGetDevice(&h->device) != cudaSuccess)
     return bail(fail(h, ITP_ERR_CUDA, "no CUDA device"));
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  h->n_chunks = 2 * sms;
-  h->n_chunks_tc = h->m <= kF32MaxM ? 2 * sms : sms;
+  cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
+  h->n_chunks = 2 * h->sms;
+  h->n_chunks_tc = h->m <= kF32MaxM ? 2 * h->sms : h->sms;
   const size_t N = (size_t)g.n_points, m = (size_t)h->m;
   int rc;
 #define ITP_CREATE(expr)           \

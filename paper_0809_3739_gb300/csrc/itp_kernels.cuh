@@ -162,8 +162,9 @@ cudaError_t launch_transpose_planes(const TS* src, TD* dst, long long nplanes, i
 // accuracy, in integer arithmetic (fx_gemm.cu).
 cudaError_t launch_gram_partial(const double* A, const double* B, int m, long long n_points,
                                 int n_chunks, double* partial, cudaStream_t st);
-// The chunk count, at most `most`, that suits launch_gram_partial (same: A == B).
-int gram_chunks(int m, bool same, long long n_points, int most);
+// The chunk count, at most `most`, that suits launch_gram_partial (same: A == B)
+// on a device of `sms` SMs.
+int gram_chunks(int m, bool same, long long n_points, int most, int sms);
 // G = scale * sum_c P[c] (fixed order), symmetrised if sym.
 cudaError_t launch_gram_reduce(const double* partial, int n_chunks, int m, double scale,
                                int sym, double* G, cudaStream_t st);

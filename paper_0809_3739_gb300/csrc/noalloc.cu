@@ -74,7 +74,10 @@ extern "C" int itp_orthonormalize_noalloc(const double* phi_device, double* psi_
   using namespace itp;
   // fewer states leave room for more partial sums, up to two CTAs per SM
   const int room = (int)(kPartialDoubles / ((size_t)m * m));
-  const int chunks = gram_chunks(m, true, n_points, room < 304 ? room : 304);
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int chunks = gram_chunks(m, true, n_points, room < 2 * sms ? room : 2 * sms, sms);
   if (launch_gram_partial(phi_device, phi_device, m, n_points, chunks, partial, st) != cudaSuccess ||
       launch_gram_reduce(partial, chunks, m, dV, 1, S, st) != cudaSuccess ||
       launch_cholesky_inverse(S, m, Minv, status, st) != cudaSuccess ||
