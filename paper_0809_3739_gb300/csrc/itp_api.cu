@@ -203,10 +203,13 @@ void prof_end(itp_handle h, long idx) {
   } while (0)
 
 // Kernels behind one launch_* call of the n x n work, which walks 128-state
-// blocks when m > 128: the update Y = M X (lower: M lower triangular) and
+// blocks when m > 128: the update Y = M X (mixed: a launch per 128 x 128
+// block, lower: of the lower triangle; FP64: one per 128 columns of M) and
 // the tensor-core Gram (A A^T: diagonal and off-diagonal blocks apart).
+template <typename R>
 int apply_launches(int m, bool lower) {
   const int nb = (m + 127) / 128;
+  if (sizeof(R) == 8) return nb;
   return lower ? nb * (nb + 1) / 2 : nb * nb;
 }
 int tc_gram_launches(int m, bool same) { return same && m > 128 ? 2 : 1; }
@@ -669,7 +672,7 @@ int orthonormalize_lane<double>(itp_handle h) {
   ITP_LAUNCH(h, ITP_KERNEL_CHOLESKY, launch_cholesky_inverse(h->S, h->m, h->Mx, h->status, h->st));
   ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix(
                                       h->Mx, h->m, 1, h->S, h->acc, L.psi, h->g.n_points, h->st)));
-  h->launches += apply_launches(h->m, true) - 1;
+  h->launches += apply_launches<double>(h->m, true) - 1;
   return ITP_OK;
 }
 // Mixed path: phi is FP32 (rounded from the FP64 sum) in psi_tmp; S and the
@@ -688,7 +691,7 @@ int orthonormalize_lane<float>(itp_handle h) {
   ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_tc_apply<float, float>(h->Mx, h->m, L.psi_tmp, L.psi,
                                                                  h->g.n_points, h->status,
                                                                  h->st, tc_expire(h), 1)));
-  h->launches += apply_launches(h->m, true) - 1;
+  h->launches += apply_launches<float>(h->m, true) - 1;
   return ITP_OK;
 }
 
@@ -758,13 +761,13 @@ int energies_lane(itp_handle h, int flags) {
                                           h->Mx, h->m, reinterpret_cast<const float*>(L.psi),
                                           reinterpret_cast<float*>(L.psi_tmp), g.n_points,
                                           h->status, h->st, tc_expire(h))));
-      h->launches += apply_launches(h->m, false) - 1;
+      h->launches += apply_launches<R>(h->m, false) - 1;
     } else {
       ITP_LAUNCH(h, ITP_KERNEL_APPLY, (launch_apply_matrix(
                                           h->Mx, h->m, 0, nullptr, reinterpret_cast<const double*>(L.psi),
                                           reinterpret_cast<double*>(L.psi_tmp), g.n_points,
                                           h->st)));
-      h->launches += apply_launches(h->m, false) - 1;
+      h->launches += apply_launches<R>(h->m, false) - 1;
     }
     R* t = L.psi;
     L.psi = L.psi_tmp;
