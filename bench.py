@@ -147,26 +147,6 @@ def measure_peaks(P):
     return out
 
 
-def fft_pass_flops(kind, g, m):
-    """Algorithmic flops of one FFT pass over m states: a complete complex
-    FFT of length L counts 5 L log2 L, a real one half that; the plane pass
-    does the 2D real transform(s) of its plane (two for the merged pass),
-    the pencil pass a forward and an inverse complex transform along z of
-    each of the nx/2+1 columns, plus one multiply per point for the factors."""
-    import math
-    P2 = g.nx * g.ny
-    Nh = g.nz * g.ny * (g.nx // 2 + 1)
-    real2d = 2.5 * P2 * math.log2(P2) if P2 > 1 else 0.0
-    zfft = 5.0 * g.nz * math.log2(g.nz) if g.nz > 1 else 0.0
-    per = {"plane_merged": 2 * real2d + P2, "plane_fwd": real2d + P2,
-           "plane_combine": real2d + 3 * P2, "plane_hpsi": real2d + 2 * P2}
-    if kind in per:
-        return m * g.nz * per[kind]
-    if kind in ("pencil", "pencil_kinetic"):
-        return m * (Nh // g.nz) * (2 * zfft + 2 * g.nz)
-    return None
-
-
 def _hbm_peak():
     try:
         return json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"]
@@ -192,6 +172,18 @@ def algorithmic_bytes(kind, g, m, s, mixed=False):
         "plane_hpsi": (spec + 2 * m * N * s + N * s) if mixed
                       else (spec + m * N * s + N * 8 + m * N * 8),
     }.get(kind)
+
+
+def pass_roofline(kind, g, m, s, ms, hbm_peak, mixed=False):
+    """One FFT pass of `ms` per launch against the measured HBM bandwidth, in
+    the bytes it must move.  (The FP64 passes are limited by their 64-bit
+    integer arithmetic, for which the probes have no rate; a rate of a unit
+    that they do not use, the FP64 one, is no roof.)"""
+    b = algorithmic_bytes(kind, g, m, s, mixed=mixed)
+    achieved = b / (ms / 1e3) / 1e9
+    return {"kernel": kind, "bound": "hbm", "achieved": achieved, "peak": hbm_peak,
+            "unit": "GB/s", "frac": achieved / hbm_peak, "algorithmic_bytes_per_launch": b,
+            "avg_launch_ms": ms}
 
 
 def step_bytes(g, m, k, s=4):
@@ -1122,14 +1114,9 @@ def main():
     # this GPU's own arithmetic rates (FP32, FP64, TF32 tensor), measured here
     probes = measure_peaks(P)
     roof = None
-    ab = algorithmic_bytes(top, g, m, 4, mixed=True)
-    if ab is not None:
-        per_launch_s = kinds[top][1] / 1e3 / kinds[top][0]
-        achieved = ab / per_launch_s / 1e9
-        roof = {"kernel": top, "bound": "hbm", "achieved": achieved, "peak": hbm_peak,
-                "peak_source": peak_src, "unit": "GB/s", "frac": achieved / hbm_peak,
-                "traffic": ncu_traffic(args.workload, top), "algorithmic_bytes_per_launch": ab,
-                "avg_launch_ms": per_launch_s * 1e3}
+    if algorithmic_bytes(top, g, m, 4, mixed=True) is not None:
+        roof = pass_roofline(top, g, m, 4, kinds[top][1] / kinds[top][0], hbm_peak, mixed=True)
+        roof.update(peak_source=peak_src, traffic=ncu_traffic(args.workload, top))
     # the same figure for every FFT pass (achieved GB/s of algorithmic bytes)
     roof_all = {}
     for k in kinds:
@@ -1139,10 +1126,11 @@ def main():
             roof_all[k] = {"avg_launch_ms": round(t * 1e3, 4),
                            "achieved_gbs": round(b / t / 1e9, 1),
                            "frac": round(b / t / 1e9 / hbm_peak, 4)}
-    # the tensor-core Gram (overlap and subspace matrix, 128 x 128 blocks):
-    # three TF32 products per FP32 product, against the measured TF32 MMA rate
+    # the tensor-core Gram (overlap and subspace matrix, 128 x 128 blocks; up to
+    # 64 states the FP32 cores take it): three TF32 products per FP32 product,
+    # against the measured TF32 MMA rate
     gram_tc = None
-    if "gram" in kinds and probes.get("tf32_mma_tflops"):
+    if m > 64 and "gram" in kinds and probes.get("tf32_mma_tflops"):
         nb = (m + 127) // 128
         t = kinds["gram"][1] / 1e3 / kinds["gram"][0]
         # per launch on average: the overlap (nb(nb+1)/2 blocks) and the
@@ -1220,19 +1208,13 @@ def main():
                 "ms_per_step": 1e3 * dt64 / K, "launch_shapes": tuned64,
                 "breakdown": {k: {"launches": v[0], "ms": round(v[1], 3),
                                   "share": round(v[1] / tot64, 4)} for k, v in prof64.items()}}
-        # the FP64 path's dominant FFT pass, in the transform's FP64 operations,
-        # against the measured DFMA rate; the passes run in 64-bit integers,
-        # bound by the integer ALU, so the fraction exceeds one
-        top64 = max((k for k in prof64 if fft_pass_flops(k, g, m) is not None),
+        # the FP64 path's dominant FFT pass
+        top64 = max((k for k in prof64 if algorithmic_bytes(k, g, m, 8) is not None),
                     key=lambda k: prof64[k][1], default=None)
-        if top64 is not None and probes.get("dfma_tflops"):
-            t = prof64[top64][1] / 1e3 / prof64[top64][0]
-            ach = fft_pass_flops(top64, g, m) / t / 1e12
-            fp64["roofline"] = {"kernel": top64, "bound": "alu (64-bit integer)", "achieved": ach,
-                                "peak": probes["dfma_tflops"], "unit": "TFLOP/s",
-                                "frac": ach / probes["dfma_tflops"],
-                                "avg_launch_ms": round(t * 1e3, 3),
-                                "peak_source": "measured (itp_peak_probe DFMA)"}
+        if top64 is not None:
+            fp64["roofline"] = pass_roofline(top64, g, m, 8, prof64[top64][1] / prof64[top64][0],
+                                             hbm_peak)
+            fp64["roofline"]["peak_source"] = peak_src
         h.close()
 
     # ---- time to n states at tol: mixed vs FP64 --------------------------------
