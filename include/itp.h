@@ -57,7 +57,9 @@ extern "C" {
 
 typedef enum {
   ITP_FP64 = 0,  /* every step to FP64 accuracy (transforms and contractions
-                    in 64-bit fixed point, states and matrices FP64)        */
+                    in 64-bit fixed point, states and matrices FP64): errors
+                    of a state relative to its norm.  Subnormal numbers
+                    count as zero                                           */
   ITP_MIXED = 1  /* FP32 FFT passes, FP64 combination / Cholesky / energies */
 } itp_precision;
 
@@ -430,7 +432,11 @@ void itp_batch_destroy(itp_batch_handle b);
  * path that must not allocate between set-up and a deadline.  The paper has
  * no counterpart; this computes the same FP64 orthonormalisation as
  * itp_orthonormalize (S = Phi Phi^T dV = L L^T, psi = L^{-1} phi) on
- * caller-owned buffers.
+ * caller-owned buffers.  Its accuracy is that of FP64 relative to the norms of
+ * the states, whatever these are, not value by value: at each point a result
+ * carries an error of 2^-56 times the largest state there (each state taken
+ * relative to its norm), so the tail of a localised state is known to that
+ * where another state is large.  Subnormal numbers count as zero.
  *   phi_device  [m][n_points] doubles on the current device (input, not
  *               modified); any point order, the same for every state
  *   psi_device  [m][n_points] doubles (output); its byte range must not
