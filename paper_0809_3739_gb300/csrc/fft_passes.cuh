@@ -380,34 +380,27 @@ __device__ __forceinline__ void xA_fwd_global(const PlaneGeo<R, NX, NY, NTT>& G,
   ITP_WITH_RADIX(G.ax.r2, (outlined<C, NX>), xA_fwd_global_r, G, sm, src, f, tw)
 }
 
-// Stage B (DIR = -1 forward, +1 inverse with the conjugate twiddle after).
-template <int R1, int DIR, typename R, int NX, int NY, int NTT, typename C>
-__device__ __forceinline__ void xB_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
+// Inverse stage B' (the conjugate twiddle after; the forward one is
+// xB_fwd_split).
+template <int R1, typename R, int NX, int NY, int NTT, typename C>
+__device__ __forceinline__ void xB_inv_r(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
   constexpr int NT = PlaneGeo<R, NX, NY, NTT>::NT;
   for_tasks<NT>(G.npair, G.ax.r2, [&](int t, int b) {
     SVec<C, R1> a;
 #pragma unroll
     for (int i = 0; i < R1; ++i) a.v[i] = sm[G.rowB(t, b, i)];
     a.open();
-    a.template dft<DIR>();
-    if (DIR > 0) twiddle_direct<true>(a, tw, b);
+    a.template dft<1>();
+    twiddle_direct<true>(a, tw, b);
     a.close();
 #pragma unroll
     for (int i = 0; i < R1; ++i) sm[G.rowB(t, b, i)] = a.v[i];
   });
 }
-template <int R1, typename G_, typename C>
-__device__ __forceinline__ void xB_fwd_r(const G_& G, C* sm, const C* tw) { xB_r<R1, -1>(G, sm, tw); }
-template <int R1, typename G_, typename C>
-__device__ __forceinline__ void xB_inv_r(const G_& G, C* sm, const C* tw) { xB_r<R1, 1>(G, sm, tw); }
-template <int DIR, typename R, int NX, int NY, int NTT, typename C>
-__device__ __forceinline__ void xB(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
+template <typename R, int NX, int NY, int NTT, typename C>
+__device__ __forceinline__ void xB_inv(const PlaneGeo<R, NX, NY, NTT>& G, C* sm, const C* tw) {
   if (G.ax.r1 == 1) return;
-  if (DIR < 0) {
-    ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_fwd_r, G, sm, tw)
-  } else {
-    ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_inv_r, G, sm, tw)
-  }
+  ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_inv_r, G, sm, tw)
 }
 
 // Inverse stage A' followed by an epilogue on the natural-order row data:
@@ -718,7 +711,7 @@ __device__ __forceinline__ void xB_inv_merge(const PlaneGeo<R, NX, NY, NTT>& G, 
   if (G.ax.r1 == 1 || G.ax.r2 > 32) {
     x_merge(G, sm);
     __syncthreads();
-    xB<1>(G, sm, tw);
+    xB_inv(G, sm, tw);
     return;
   }
   ITP_WITH_RADIX(G.ax.r1, (outlined<C, NX>), xB_inv_merge_r, G, sm, tw)
