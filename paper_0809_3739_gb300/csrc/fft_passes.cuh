@@ -52,7 +52,7 @@ constexpr int kThreads = 256;
 // compiled for, FP64 (128 registers) and FP32 (80), in CTAs of any size up to
 // that; one CTA of 256 threads with up to 255 registers left most of the SM
 // idle: FP64 merged pass at 72 x 48 90 -> 58 ps per value, FP32 at 96 x 72 19.2
-// -> 10.4 ps.
+// -> 9.5 ps.
 constexpr int kGenericThreads64 = 512, kGenericThreads32 = 768;
 constexpr int kGenericCtas64 = 2;   // FP64 pencils of run-time sizes
 
@@ -91,10 +91,11 @@ __host__ __device__ constexpr int launch_threads(int nt) { return (nt + 31) / 32
 
 // Threads doing the tasks of an FP64 plane pass.  128 x 128 (one CTA fills the
 // SM's shared memory): 512 threads at 128 registers, four warps per
-// scheduler, merged pass of 48 states 2.16 ms, against 2.74 ms with 256
-// threads, 2.41 with 384 and 2.47 with 544 (96 registers, spills).  64 x 64:
-// the column stages have 264 tasks, one round of 264 threads instead of two
-// of 256 (0.268 ms against 0.289).
+// scheduler, merged pass of 48 states 1.74 ms, against 1.95 ms with 256
+// threads, 1.76 with 384 and 2.05 with 544 (96 registers, spills), last pass
+// 1.29 ms against 1.55, 1.48 and 1.29.  64 x 64: the column stages have 264
+// tasks, one round of 264 threads instead of two of 256 (merged pass of 57
+// states 0.211 ms against 0.216, the others within 1 %).
 __host__ __device__ constexpr int plane64_threads(int nx) {
   return nx == 128 ? 512 : nx == 64 ? 264 : kThreads;
 }

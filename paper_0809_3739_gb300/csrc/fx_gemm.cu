@@ -109,9 +109,10 @@ __device__ __forceinline__ void load_pairs(const int2* p, int2 (&v)[N]) {
 constexpr int kRun = 512;
 constexpr int kTile = 16;   // (32 points needed more registers for the tile in flight)
 constexpr int kGramBits = 54;
-// More states than this: the tensor-core form below.  57 states at 64^3: 0.50 ms
-// here, 0.27 there; 128: 1.74, 1.00; 48 at 128^3: 2.30, 1.92; but 32 at 24^3
-// 0.019 here, 0.037 there.
+// More states than this: the tensor-core form below.  32 states at 64^3 0.184 ms
+// here, 0.218 there; at 24^3 0.019 and 0.023; 16 at 64^3 0.066 and 0.206.  With
+// this form extended to 64 states (before l l') 57 at 64^3 took 0.50 ms, 0.24
+// there; 48 at 128^3 2.30 and 1.68.
 constexpr int kGramMmaMin = 32;
 
 template <int TT>
@@ -256,8 +257,11 @@ __global__ void __launch_bounds__(256, 3)
 // FP32: up to 7 * 128 products of at most 2^14 stay below 2^24, so the sums
 // over 128 points are exact whatever the rounding.  They are then moved to
 // 64-bit integers in shared memory (levels 0-3 and 4-6), and the run's sums to
-// FP64.  The levels above 6 are below the precision: about 2^-56 of the two
-// largest values per product, with random signs.
+// FP64.  The levels above 6 left out are about 2^-56 of the two largest values
+// per product, with random signs (squares start at level 8), which is below
+// the rounding of an FP64 sum: squared norms of 33 and 64 rows off by 4e-16 at
+// most for smooth, random and decaying rows (FP64 sums 3e-15 to 1.2e-14), and by
+// 3.5e-15 for one large value and 1e-4 beside it (FP64 sums 1.6e-14).
 //
 // mma.sync reaches 1000 FMAs per clock and SM here, a quarter of tcgen05, but
 // its sums are in registers: the seven accumulators of a 128 x 128 tile would
@@ -478,8 +482,12 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
 //
 // Precision: products are exact in 110 bits, so a sum is off by the rounding
 // of its operands, 2^-56 of the largest |M_ik| times the point's largest
-// |X_k| (both scaled) per term with random signs, and the rounding to a double;
-// an FP64 sum rounds by up to 2^-53 of the same size.
+// |X_k| (both scaled) per term with random signs, and the rounding to a double.
+// In the norm of a state that is below an FP64 sum's 2^-53 of the largest
+// |M_ik X_k|.  It is not value by value: where a state is in its tail, another
+// one is large and their M_ik is small, the FP64 sum's error was as small as
+// the tail, this one's is 2^-56 of the other state's size there (and smaller
+// values come out as zero).
 constexpr int kApplyBits = 55;
 constexpr int kApplyThreads = 512;
 
@@ -641,8 +649,8 @@ __global__ void __launch_bounds__(kApplyThreads)
 // (One level more than the Gram, 34 digit products: a sum over few states has
 // no averaging over the grid, and without level 7 its error, about 2^-53 of
 // the largest product, was that of the FP64 form instead of below it.)
-// 57 states at 64^3 0.40 ms in integers, 128 1.44, 48 at 128^3 2.92; up to 32
-// states both forms take the same time.
+// 57 states at 64^3 0.40 ms in integers, 0.25 here; 128 1.44 and 0.81; 48 at
+// 128^3 2.92 and 1.76; but 32 at 64^3 0.142 and 0.203, at 24^3 0.018 either way.
 constexpr int kApplyMmaMin = 32;
 constexpr int kApplyMmaPts = 32;
 constexpr int kApplyLevels = 8;
